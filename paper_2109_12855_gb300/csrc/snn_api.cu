@@ -373,13 +373,18 @@ size_t stdp_bytes_per_target(const snn_net* net, int window) {
   return net->stdp_on ? (size_t)net->stdp.history * 4 + 4 + 4 * (size_t)window : 0;
 }
 
+// Whether a tile with a window of `window` steps fits shared memory.
+bool tile_fits(const snn_net* net, int window) {
+  return (size_t)net->tile_w * ((size_t)window * 4 * net->acc_words +
+                                stdp_bytes_per_target(net, window)) <=
+         kTileSmemBudget;
+}
+
+// (a split store is built for the widest window its net can have, which
+// bounds the finalized one)
 bool use_tiled(const snn_net* net) {
   return net->p.deliver_mode == SNN_DELIVER_TILED && net->n_syn > 0 &&
-         net->tile_off &&
-         (size_t)net->tile_w *
-                 ((size_t)net->window * 4 * net->acc_words +
-                  stdp_bytes_per_target(net, net->window)) <=
-             kTileSmemBudget;
+         net->lay != kLayRecords && tile_fits(net, net->window);
 }
 
 // ---- one-word accumulator cells -----------------------------------------
@@ -450,6 +455,7 @@ void decide_acc_words(snn_net* net, const WeightBounds& b, uint32_t k_in_max,
                       int max_interval) {
   net->acc_words = 2;
   net->acc_qs_min = 0;
+  net->int_w = false;
   if (net->p.acc_words == 2 || net->stdp_on || !b.ok ||
       net->fmt != SNN_W_BF16_8B)
     return;
@@ -464,6 +470,8 @@ void decide_acc_words(snn_net* net, const WeightBounds& b, uint32_t k_in_max,
   if (qs >= 0 && qs >= -b.g_min) {
     net->acc_words = 1;
     net->acc_qs_min = -b.g_min;
+    // (scales of a normal float, as the layout's conversions take them)
+    net->int_w = abs(b.g_min) <= 60 && ldexp(b.w_max, -b.g_min) <= 32767.0;
   }
 }
 
@@ -508,7 +516,6 @@ int build_store(snn_net* net, uint32_t* d_deg, Scatter scatter,
   const uint64_t n_syn = rp[n];
   const uint32_t ch = (uint32_t)chunk_records(net->fmt);
   const uint64_t padded = (n_syn + ch - 1) / ch * ch + ch;
-  const int rec_bytes = net->fmt == SNN_W_FP32_12B ? 12 : 8;
   CK(dalloc(&net->row_ptr, (n + 1) * sizeof(uint64_t), net->stream));
   CK(cudaMemcpyAsync(net->row_ptr, rp.data(), (n + 1) * sizeof(uint64_t),
                      cudaMemcpyHostToDevice, s));
@@ -523,12 +530,25 @@ int build_store(snn_net* net, uint32_t* d_deg, Scatter scatter,
     balance_plastic_tiles(net->n, net->p.n_exc, &net->tile_w, &net->lo_bits,
                           &net->n_tiles, &net->pl_tiles, &net->tile_grp);
   CK(dalloc(&net->tile_off, (uint64_t)n * (net->n_tiles + 1) * sizeof(uint32_t), net->stream));
+  // layout of the store: split by field for the tiled delivery (its cells fit
+  // 16 bits whenever the tile fits, but for windows of one step and the like)
+  net->d_base = d_lo;
+  net->n_pad = padded;
+  net->lay = kLayRecords;
+  if (net->p.deliver_mode == SNN_DELIVER_TILED && n_syn > 0 &&
+      tile_fits(net, iv + (d_hi - d_lo)) &&
+      (uint64_t)(d_hi - d_lo + 1) * net->tile_w <= 0xFFFFull)
+    net->lay = net->hom && !net->stdp_on ? kLayHom
+               : net->fmt == SNN_W_FP32_12B ? kLayF32
+               : net->int_w ? kLayI16 : kLayJ16;
   // keys; for 8-byte records the key array becomes the record array
   uint64_t* keys = nullptr;
   CK(dalloc(&keys, padded * sizeof(uint64_t), net->stream));
   uint32_t* cursor = d_deg;  // reuse as the scatter cursor
   CK(cudaMemsetAsync(cursor, 0, n * sizeof(uint32_t), s));
   CK(scatter(net->row_ptr, cursor, keys, net->tile_w, net->lo_bits));
+  const int rec_bytes =
+      net->fmt != SNN_W_FP32_12B ? 8 : net->lay == kLayRecords ? 12 : 10;
   void* recs = nullptr;
   if (rec_bytes == 8) {
     recs = keys;
@@ -541,8 +561,16 @@ int build_store(snn_net* net, uint32_t* d_deg, Scatter scatter,
     }
   }
   // zero the padding records once (target 0, weight 0; never delivered)
-  CK(cudaMemsetAsync(static_cast<char*>(recs) + n_syn * rec_bytes, 0,
-                     (padded - n_syn) * rec_bytes, s));
+  if (rec_bytes == 10) {
+    char* const p = static_cast<char*>(recs);
+    const uint64_t pad = padded - n_syn;
+    CK(cudaMemsetAsync(p + 4 * n_syn, 0, 4 * pad, s));
+    CK(cudaMemsetAsync(p + 4 * padded + 4 * n_syn, 0, 4 * pad, s));
+    CK(cudaMemsetAsync(p + 8 * padded + 2 * n_syn, 0, 2 * pad, s));
+  } else {
+    CK(cudaMemsetAsync(static_cast<char*>(recs) + n_syn * rec_bytes, 0,
+                       (padded - n_syn) * rec_bytes, s));
+  }
   uint32_t* d_long = nullptr;
   uint64_t *d_loff = nullptr, *d_scr = nullptr;
   if (!long_rows.empty()) {
@@ -557,18 +585,27 @@ int build_store(snn_net* net, uint32_t* d_deg, Scatter scatter,
                        cudaMemcpyHostToDevice, s));
   }
   uint32_t* d_stats = nullptr;
-  CK(dalloc(&d_stats, 2 * sizeof(uint32_t), net->stream));
-  CK(cudaMemsetAsync(d_stats, 0, 2 * sizeof(uint32_t), s));
-  CK(build_sort_pack(net->fmt, n, net->row_ptr, keys, recs, bf, d_edge_w,
+  uint32_t h_stats[4] = {0, 0, 0xFFFFFFFFu, 0};
+  CK(dalloc(&d_stats, sizeof h_stats, net->stream));
+  CK(cudaMemcpyAsync(d_stats, h_stats, sizeof h_stats, cudaMemcpyHostToDevice, s));
+  StoreOut so{net->lay, d_lo, net->acc_qs_min, recs, nullptr, nullptr, nullptr};
+  if (rec_bytes == 10) {
+    char* const p = static_cast<char*>(recs);
+    so.wts = reinterpret_cast<float*>(p);
+    so.tgts = reinterpret_cast<uint32_t*>(p + 4 * padded);
+    so.cells = reinterpret_cast<uint16_t*>(p + 8 * padded);
+  }
+  CK(build_sort_pack(net->fmt, n, net->row_ptr, keys, so, bf, d_edge_w,
                      max_row, d_long, (uint32_t)long_rows.size(), d_scr,
                      d_loff, net->tile_w, net->lo_bits, net->n_tiles,
                      net->tile_off, d_stats, s));
-  uint32_t h_stats[2] = {0, 0};
   CK(cudaMemcpyAsync(h_stats, d_stats, sizeof h_stats, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   dfree(d_stats, net->stream);
   net->mult_max = h_stats[0];
   memcpy(&net->max_abs_w, &h_stats[1], sizeof(float));
+  net->dmin = n_syn ? (int)h_stats[2] : 0;
+  net->dmax = n_syn ? (int)h_stats[3] : 0;
   if (recs != keys) dfree(keys, net->stream);
   dfree(d_long, net->stream);
   dfree(d_loff, net->stream);
@@ -898,6 +935,13 @@ int snn_connect_fixed_indegree(snn_net* net, const snn_conn_params* c) {
     if (c->k_inh) add_population(&wb, c->w_inh, c->sd_inh, false, c->clip_inh != 0, net->fmt);
     decide_acc_words(net, wb, c->k_exc + c->k_inh,
                      net->p.interval ? net->p.interval : c->d_hi);
+    // without a spread every synapse of a population has one weight
+    net->hom = (c->k_exc == 0 || c->sd_exc == 0.0) && (c->k_inh == 0 || c->sd_inh == 0.0);
+    net->hom_split = p.n_exc;
+    const double we = c->clip_exc ? std::max(c->w_exc, 0.0) : c->w_exc;
+    const double wi = c->clip_inh ? std::min(c->w_inh, 0.0) : c->w_inh;
+    net->hom_w[0] = c->k_exc ? (float)stored_weight(we, net->fmt) : 0.f;
+    net->hom_w[1] = c->k_inh ? (float)stored_weight(wi, net->fmt) : 0.f;
   }
   rc = build_store(
       net, deg,
@@ -981,7 +1025,17 @@ int snn_connect_edges(snn_net* net, const uint32_t* src, const uint32_t* tgt,
   CK(build_count_edges(d_src, n, deg, s));
   {
     WeightBounds wb;
-    for (uint64_t e = 0; e < n; ++e) wb.add_value(stored_weight(pw[e], net->fmt));
+    net->hom = n > 0;  // one weight for the E sources' edges, one for the I's
+    net->hom_split = net->p.n_exc;
+    bool seen[2] = {false, false};
+    for (uint64_t e = 0; e < n; ++e) {
+      const double w_e = stored_weight(pw[e], net->fmt);
+      wb.add_value(w_e);
+      const int c = ps[e] >= net->hom_split;
+      if (!seen[c]) net->hom_w[c] = (float)w_e;
+      seen[c] = true;
+      net->hom = net->hom && net->hom_w[c] == (float)w_e;
+    }
     decide_acc_words(net, wb, k_in_max, net->p.interval ? net->p.interval : e_hi);
   }
   rc = build_store(
@@ -1015,10 +1069,10 @@ int setup_stdp(snn_net* net) {
   const snn_stdp_params& q = net->stdp;
   StdpView& sp = net->sp;
   const uint64_t n = net->n, H = (uint64_t)q.history;
-  const uint64_t n_rec = net->recs_bytes / (net->fmt == SNN_W_FP32_12B ? 12 : 8);
+  const uint64_t n_rec = net->n_pad;
   CK(dalloc(&sp.wp, std::max<uint64_t>(n_rec, 1) * sizeof(float), s));
   CK(cudaMemsetAsync(sp.wp, 0, std::max<uint64_t>(n_rec, 1) * sizeof(float), s));
-  CK(unpack_store(net->fmt, net->recs, net->n_syn, nullptr, nullptr, sp.wp, s));
+  CK(unpack_store(net->view(), net->n_syn, nullptr, nullptr, sp.wp, s));
   CK(dalloc(&sp.pre_t, n * sizeof(int32_t), s));
   CK(dalloc(&sp.prev_t, n * sizeof(int32_t), s));
   CK(dalloc(&sp.pre_k, n * sizeof(float), s));
@@ -1063,16 +1117,6 @@ int snn_finalize(snn_net* net) {
     net->n_syn = 0;
     net->connected = true;
   }
-  unsigned* dd = nullptr;
-  unsigned h[2] = {0xFFFFFFFFu, 0u};
-  CK(dalloc(&dd, 2 * sizeof(unsigned), net->stream));
-  CK(cudaMemcpyAsync(dd, h, sizeof h, cudaMemcpyHostToDevice, s));
-  CK(delay_range(net->fmt, net->recs, net->n_syn, dd, s));
-  CK(cudaMemcpyAsync(h, dd, sizeof h, cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  dfree(dd, net->stream);
-  net->dmin = net->n_syn ? (int)h[0] : 0;
-  net->dmax = net->n_syn ? (int)h[1] : 0;
   int iv = net->p.interval;
   if (iv == 0) iv = net->n_syn ? net->dmin : net->n_slots;
   REQ(iv >= 1 && (net->n_syn == 0 || iv <= net->dmin), SNN_E_ARG,
@@ -1615,7 +1659,7 @@ int snn_read_store(snn_net* net, uint64_t* row_ptr, uint32_t* tgt,
   const uint64_t m = net->n_syn;
   if (m && (tgt || delay || w)) {
     if (mem == SNN_MEM_DEVICE) {
-      CK(unpack_store(net->fmt, net->recs, m, tgt, delay, w, s));
+      CK(unpack_store(net->view(), m, tgt, delay, w, s));
     } else {
       uint32_t* dt = nullptr;
       uint8_t* dd = nullptr;
@@ -1623,7 +1667,7 @@ int snn_read_store(snn_net* net, uint64_t* row_ptr, uint32_t* tgt,
       CK(dalloc(&dt, m * 4, net->stream));
       CK(dalloc(&dd, m, net->stream));
       CK(dalloc(&dw, m * 4, net->stream));
-      CK(unpack_store(net->fmt, net->recs, m, dt, dd, dw, s));
+      CK(unpack_store(net->view(), m, dt, dd, dw, s));
       if (tgt) CK(cudaMemcpyAsync(tgt, dt, m * 4, cudaMemcpyDeviceToHost, s));
       if (delay) CK(cudaMemcpyAsync(delay, dd, m, cudaMemcpyDeviceToHost, s));
       if (w) CK(cudaMemcpyAsync(w, dw, m * 4, cudaMemcpyDeviceToHost, s));
@@ -1912,11 +1956,11 @@ int snn_read_weights(snn_net* net, float* w, int32_t mem) {
   if (net->sp.wp) {
     CK(cudaMemcpyAsync(w, net->sp.wp, m * sizeof(float), kind_to(mem), s));
   } else if (mem == SNN_MEM_DEVICE) {
-    CK(unpack_store(net->fmt, net->recs, m, nullptr, nullptr, w, s));
+    CK(unpack_store(net->view(), m, nullptr, nullptr, w, s));
   } else {
     float* dw = nullptr;
     CK(dalloc(&dw, m * sizeof(float), s));
-    CK(unpack_store(net->fmt, net->recs, m, nullptr, nullptr, dw, s));
+    CK(unpack_store(net->view(), m, nullptr, nullptr, dw, s));
     CK(cudaMemcpyAsync(w, dw, m * sizeof(float), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     dfree(dw, s);
@@ -2000,11 +2044,37 @@ int snn_debug_poke_record(snn_net* net, uint64_t index, int field,
       "field %d / value %u", field, value);
   int rc;
   if ((rc = set_device(net)) != SNN_OK) return rc;
-  // target: word 0 of both formats; delay: low byte of word 2 (FP32
-  // records) or of word 1 (BF16 records)
-  const size_t rb = net->fmt == SNN_W_FP32_12B ? 12 : 8;
-  const size_t off = field == 0 ? 0 : (net->fmt == SNN_W_FP32_12B ? 8 : 4);
-  char* p = static_cast<char*>(net->recs) + index * rb + off;
+  char* p = static_cast<char*>(net->recs);
+  if (net->lay == kLayRecords) {
+    // target: word 0 of both formats; delay: low byte of word 2 (FP32
+    // records) or of word 1 (BF16 records)
+    const size_t rb = net->fmt == SNN_W_FP32_12B ? 12 : 8;
+    p += index * rb + (field == 0 ? 0 : (net->fmt == SNN_W_FP32_12B ? 8 : 4));
+  } else {
+    // split stores: the target, or the cell of the delay (a cell past 16
+    // bits is kept as the largest, which no window holds)
+    std::vector<uint64_t> rp(net->n_src + 1);
+    CK(cudaMemcpyAsync(rp.data(), net->row_ptr, rp.size() * 8, cudaMemcpyDeviceToHost,
+                       net->stream));
+    CK(cudaStreamSynchronize(net->stream));
+    const uint64_t row = std::upper_bound(rp.begin(), rp.end(), index) - rp.begin() - 1;
+    const uint64_t len = rp[row + 1] - rp[row], at = index - rp[row];
+    const bool f32 = net->fmt == SNN_W_FP32_12B;
+    if (field == 0) {
+      p += f32 ? 4 * net->n_pad + 4 * index : 8 * rp[row] + 4 * len + 4 * at;
+    } else {
+      p += f32 ? 8 * net->n_pad + 2 * index
+               : 8 * rp[row] + (net->lay == kLayHom ? 2 : 4) * at;
+      uint16_t cell = 0;
+      CK(cudaMemcpyAsync(&cell, p, 2, cudaMemcpyDeviceToHost, net->stream));
+      CK(cudaStreamSynchronize(net->stream));
+      const int64_t c = ((int64_t)value - net->d_base) * net->tile_w + cell % net->tile_w;
+      cell = c < 0 || c > 0xFFFF ? 0xFFFFu : (uint16_t)c;
+      CK(cudaMemcpyAsync(p, &cell, 2, cudaMemcpyHostToDevice, net->stream));
+      CK(cudaStreamSynchronize(net->stream));
+      return SNN_OK;
+    }
+  }
   uint32_t word = 0;
   CK(cudaMemcpyAsync(&word, p, 4, cudaMemcpyDeviceToHost, net->stream));
   CK(cudaStreamSynchronize(net->stream));

@@ -165,58 +165,64 @@ __device__ uint16_t bf16_weight_bits(const BuildFixed& b, bool exc,
   return bf16_bits_rne(weight_of<0>(b, nullptr, exc, tgt, tie));
 }
 
-// Writes a record; returns |stored weight| (as stored, widened to float).
-// FP32 records also carry, above the delay byte, the record's cell in its
-// tile's ring-buffer window (d TW + position in the tile; below 2^24 for
-// tiles narrower than 2^16 targets, else 0), so that interval-list
-// deliveries need neither the target word nor the index arithmetic.
-template <int FMT>
-__device__ __forceinline__ float store_rec(void* recs, uint64_t idx,
-                                           uint32_t tgt, uint32_t d, double w,
-                                           uint32_t cell = 0u) {
-  if (FMT == SNN_W_FP32_12B) {
-    uint32_t* p = reinterpret_cast<uint32_t*>(recs) + idx * 3u;
-    const float wf = __double2float_rn(w);
-    p[0] = tgt;
-    p[1] = __float_as_uint(wf);
-    p[2] = (d & 0xFFu) | (cell < (1u << 24) ? cell << 8 : 0u);
-    return fabsf(wf);
-  } else {
-    uint2 r;
-    const uint16_t bits = bf16_bits_rne(w);
-    r.x = tgt;
-    r.y = (d & 0xFFu) | ((uint32_t)bits << 16);
-    reinterpret_cast<uint2*>(recs)[idx] = r;
-    return fabsf(bf16_to_f32(bits));
-  }
+// Stored form of a fixed-rule or edge weight: the float, or the bfloat16 bits.
+template <int FMT, int WMODE>
+__device__ __forceinline__ uint32_t stored_bits(const BuildFixed& b,
+                                                const double* edge_w, bool exc,
+                                                uint32_t tgt, uint32_t tie) {
+  if (FMT == SNN_W_BF16_8B)
+    return WMODE == 0 ? bf16_weight_bits(b, exc, tgt, tie)
+                      : bf16_bits_rne(edge_w[tie]);
+  return __float_as_uint(
+      __double2float_rn(weight_of<WMODE>(b, edge_w, exc, tgt, tie)));
 }
 
+// Writes the row's synapses in the store's layout, its tile index and its
+// part of the statistics.
 template <int FMT, int WMODE>
 __device__ void pack_row(const uint64_t* sorted, uint32_t len, uint32_t row,
-                         uint64_t beg, void* recs, const BuildFixed& b,
+                         uint64_t beg, const StoreOut& o, const BuildFixed& b,
                          const double* edge_w, TileGeom g, uint32_t n_tiles,
                          uint32_t* tile_off, uint32_t* stats) {
   const bool exc = row < b.n_e;
   float wmax = 0.f;
-  uint32_t run_max = 0;
+  uint32_t run_max = 0, d_min = 0xFFFFFFFFu, d_max = 0;
   for (uint32_t p = threadIdx.x; p < len; p += blockDim.x) {
     uint64_t key = sorted[p];
     uint32_t d = key_delay(key, g);
     uint32_t tgt = key_target(key, g);
     uint32_t tie = (uint32_t)key;
-    if (FMT == SNN_W_BF16_8B && WMODE == 0) {
-      const uint16_t bits = bf16_weight_bits(b, exc, tgt, tie);
-      uint2 rec;
-      rec.x = tgt;
-      rec.y = (d & 0xFFu) | ((uint32_t)bits << 16);
-      reinterpret_cast<uint2*>(recs)[beg + p] = rec;
-      wmax = fmaxf(wmax, fabsf(bf16_to_f32(bits)));
+    const uint32_t bits = stored_bits<FMT, WMODE>(b, edge_w, exc, tgt, tie);
+    wmax = fmaxf(wmax, fabsf(FMT == SNN_W_BF16_8B ? bf16_to_f32(bits)
+                                                  : __uint_as_float(bits)));
+    d_min = min(d_min, d);
+    d_max = max(d_max, d);
+    const uint32_t in_tile = (uint32_t)(key >> 32) & ((1u << g.lb) - 1u);
+    const uint32_t cell = (d - (uint32_t)o.d_base) * g.tw + in_tile;
+    if (o.lay == kLayRecords) {
+      if (FMT == SNN_W_FP32_12B) {
+        uint32_t* r = reinterpret_cast<uint32_t*>(o.recs) + (beg + p) * 3u;
+        r[0] = tgt;
+        r[1] = bits;
+        r[2] = d & 0xFFu;
+      } else {
+        reinterpret_cast<uint2*>(o.recs)[beg + p] =
+            make_uint2(tgt, (d & 0xFFu) | (bits << 16));
+      }
+    } else if (FMT == SNN_W_FP32_12B) {
+      o.wts[beg + p] = __uint_as_float(bits);
+      o.tgts[beg + p] = tgt;
+      o.cells[beg + p] = (uint16_t)cell;
     } else {
-      const uint32_t in_tile = (uint32_t)(key >> 32) & ((1u << g.lb) - 1u);
-      const uint32_t cell = g.tw < (1u << 16) ? d * g.tw + in_tile : (1u << 24);
-      wmax = fmaxf(wmax, store_rec<FMT>(recs, beg + p, tgt, d,
-                                        weight_of<WMODE>(b, edge_w, exc, tgt, tie),
-                                        cell));
+      uint32_t* r = reinterpret_cast<uint32_t*>(o.recs) + 2u * beg;
+      r[len + p] = tgt;
+      if (o.lay == kLayHom) {
+        reinterpret_cast<uint16_t*>(r)[p] = (uint16_t)cell;
+        reinterpret_cast<uint16_t*>(r)[len + p] = (uint16_t)bits;
+      } else {
+        r[p] = (cell & 0xFFFFu) |
+               (o.lay == kLayI16 ? i16_bits(bf16_to_f32(bits), o.qs) : bits) << 16;
+      }
     }
     // multiplicity of (target, delay): length of the run of equal keys
     // (ignoring the tie field) that starts here
@@ -229,9 +235,17 @@ __device__ void pack_row(const uint64_t* sorted, uint32_t len, uint32_t row,
   // |w| >= 0 orders like its bit pattern as an unsigned integer
   const uint32_t wbits = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(wmax));
   run_max = __reduce_max_sync(0xFFFFFFFFu, run_max);
+  d_min = __reduce_min_sync(0xFFFFFFFFu, d_min);
+  d_max = __reduce_max_sync(0xFFFFFFFFu, d_max);
   if ((threadIdx.x & 31u) == 0) {
-    if (run_max) atomicMax(&stats[0], run_max);
-    if (wbits) atomicMax(&stats[1], wbits);
+    // the four words settle after a few rows: only a value beyond the
+    // current one goes to the atomic (millions of warps would otherwise
+    // queue on one line)
+    const volatile uint32_t* st = stats;
+    if (run_max > st[0]) atomicMax(&stats[0], run_max);
+    if (wbits > st[1]) atomicMax(&stats[1], wbits);
+    if (d_min < st[2]) atomicMin(&stats[2], d_min);
+    if (d_max > st[3]) atomicMax(&stats[3], d_max);
   }
   // tile index: first position whose tile is >= tau (lower bound)
   uint32_t* out = tile_off + (uint64_t)row * (n_tiles + 1);
@@ -369,7 +383,7 @@ __device__ void sort_row(uint64_t* a, uint32_t len, uint32_t* cnt,
 
 template <int FMT, int WMODE>
 __global__ void __launch_bounds__(1024) k_sort_pack(uint32_t n, const uint64_t* row_ptr,
-                            uint64_t* keys, void* recs, BuildFixed b,
+                            uint64_t* keys, StoreOut recs, BuildFixed b,
                             const double* edge_w, uint32_t cap, TileGeom g,
                             uint32_t n_tiles, uint32_t* tile_off,
                             uint32_t* stats) {
@@ -391,7 +405,7 @@ __global__ void __launch_bounds__(1024) k_sort_pack(uint32_t n, const uint64_t* 
 template <int FMT, int WMODE>
 __global__ void __launch_bounds__(1024) k_sort_long(const uint32_t* rows, uint32_t n_long,
                             const uint64_t* row_ptr,
-                            uint64_t* keys, void* recs, BuildFixed b,
+                            uint64_t* keys, StoreOut recs, BuildFixed b,
                             const double* edge_w, uint64_t* scratch,
                             const uint64_t* scratch_off, TileGeom g,
                             uint32_t n_tiles, uint32_t* tile_off,
@@ -436,37 +450,32 @@ __global__ void k_unpack(const void* recs, uint64_t n, uint32_t* tgt,
   }
 }
 
-template <int FMT>
-__global__ void __launch_bounds__(1024) k_delay_range(const void* recs, uint64_t n, unsigned* out) {
-  __shared__ unsigned s_lo, s_hi;
-  if (threadIdx.x == 0) {
-    s_lo = 0xFFFFFFFFu;
-    s_hi = 0u;
-  }
-  __syncthreads();
-  unsigned lo = 0xFFFFFFFFu, hi = 0u;
-  for (uint64_t s = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; s < n;
-       s += (uint64_t)gridDim.x * blockDim.x) {
-    unsigned d = FMT == SNN_W_FP32_12B
-                     ? reinterpret_cast<const uint32_t*>(recs)[s * 3u + 2u] & 0xFFu
-                     : reinterpret_cast<const uint2*>(recs)[s].y & 0xFFu;
-    lo = min(lo, d);
-    hi = max(hi, d);
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = min(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
-    hi = max(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-  }
-  // one pair of global atomics per block (not per warp: every warp would
-  // hit the same two words)
-  if ((threadIdx.x & 31u) == 0) {
-    atomicMin(&s_lo, lo);
-    atomicMax(&s_hi, hi);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    atomicMin(&out[0], s_lo);
-    atomicMax(&out[1], s_hi);
+// The same for a split store, row by row: targets, and delays from the cells.
+__global__ void __launch_bounds__(256) k_unpack_split(NetView v, uint32_t* tgt,
+                                                      uint8_t* delay, float* w) {
+  const bool f32 = v.fmt == SNN_W_FP32_12B;
+  for (uint32_t row = blockIdx.x; row < v.n_src; row += gridDim.x) {
+    const uint64_t beg = v.row_ptr[row];
+    const uint32_t len = (uint32_t)(v.row_ptr[row + 1] - beg);
+    const uint32_t* r = reinterpret_cast<const uint32_t*>(v.recs) + 2u * beg;
+    const uint16_t* r16 = reinterpret_cast<const uint16_t*>(r);
+    for (uint32_t p = threadIdx.x; p < len; p += blockDim.x) {
+      uint32_t cell, t, wb;
+      if (f32) {
+        cell = v.cells[beg + p];
+        t = v.tgts[beg + p];
+        wb = reinterpret_cast<const uint32_t*>(v.recs)[beg + p];
+      } else {
+        t = r[len + p];
+        cell = v.lay == kLayHom ? r16[p] : r[p] & 0xFFFFu;
+        wb = v.lay == kLayHom ? (uint32_t)r16[len + p] << 16
+             : v.lay == kLayI16 ? __float_as_uint(i16_weight(r[p], v.acc_qs_min))
+                                : r[p] & 0xFFFF0000u;
+      }
+      if (tgt) tgt[beg + p] = t;
+      if (delay) delay[beg + p] = (uint8_t)(cell / v.tile_w + (uint32_t)v.d_base);
+      if (w) w[beg + p] = __uint_as_float(wb);
+    }
   }
 }
 
@@ -524,7 +533,7 @@ cudaError_t build_shape(Kernel kernel, unsigned blocks, unsigned threads,
 
 template <int FMT, int WMODE>
 cudaError_t sort_pack_t(uint32_t n, const uint64_t* row_ptr, uint64_t* keys,
-                        void* recs, const BuildFixed* b, const double* edge_w,
+                        StoreOut recs, const BuildFixed* b, const double* edge_w,
                         uint32_t max_row, const uint32_t* long_rows,
                         uint32_t n_long, uint64_t* long_scratch,
                         const uint64_t* long_off, TileGeom g, uint32_t n_tiles,
@@ -604,7 +613,7 @@ cudaError_t build_scatter_edges(const uint32_t* src, const uint32_t* tgt,
 }
 
 cudaError_t build_sort_pack(int fmt, uint32_t n, const uint64_t* row_ptr,
-                            uint64_t* keys, void* recs, const BuildFixed* b,
+                            uint64_t* keys, StoreOut recs, const BuildFixed* b,
                             const double* edge_w, uint32_t max_row,
                             const uint32_t* long_rows, uint32_t n_long,
                             uint64_t* long_scratch,
@@ -623,37 +632,17 @@ cudaError_t build_sort_pack(int fmt, uint32_t n, const uint64_t* row_ptr,
 #undef SNN_SORT_ARGS
 }
 
-cudaError_t unpack_store(int fmt, const void* recs, uint64_t n_syn,
-                         uint32_t* tgt, uint8_t* delay, float* w,
-                         cudaStream_t s) {
+cudaError_t unpack_store(const NetView& v, uint64_t n_syn, uint32_t* tgt,
+                         uint8_t* delay, float* w, cudaStream_t s) {
   if (n_syn == 0) return cudaSuccess;
-  if (fmt == SNN_W_FP32_12B)
-    k_unpack<SNN_W_FP32_12B><<<grid_for(n_syn, 256), 256, 0, s>>>(recs, n_syn,
-                                                                  tgt, delay, w);
+  if (v.lay != kLayRecords)
+    k_unpack_split<<<std::min(v.n_src, 1u << 16), 256, 0, s>>>(v, tgt, delay, w);
+  else if (v.fmt == SNN_W_FP32_12B)
+    k_unpack<SNN_W_FP32_12B><<<grid_for(n_syn, 256), 256, 0, s>>>(
+        v.recs, n_syn, tgt, delay, w);
   else
-    k_unpack<SNN_W_BF16_8B><<<grid_for(n_syn, 256), 256, 0, s>>>(recs, n_syn,
-                                                                 tgt, delay, w);
-  return cudaGetLastError();
-}
-
-cudaError_t delay_range(int fmt, const void* recs, uint64_t n_syn,
-                        unsigned int* dmin_dmax, cudaStream_t s) {
-  if (n_syn == 0) return cudaSuccess;
-  BuildShape sh;
-  cudaError_t e;
-  if (fmt == SNN_W_FP32_12B) {
-    if ((e = build_shape(k_delay_range<SNN_W_FP32_12B>, std::min(grid_for(n_syn, 256), 4096u), 256,
-                         0, &sh)) != cudaSuccess)
-      return e;
-    k_delay_range<SNN_W_FP32_12B><<<sh.blocks, sh.threads, sh.smem, s>>>(
-        recs, n_syn, dmin_dmax);
-  } else {
-    if ((e = build_shape(k_delay_range<SNN_W_BF16_8B>, std::min(grid_for(n_syn, 256), 4096u), 256,
-                         0, &sh)) != cudaSuccess)
-      return e;
-    k_delay_range<SNN_W_BF16_8B><<<sh.blocks, sh.threads, sh.smem, s>>>(
-        recs, n_syn, dmin_dmax);
-  }
+    k_unpack<SNN_W_BF16_8B><<<grid_for(n_syn, 256), 256, 0, s>>>(
+        v.recs, n_syn, tgt, delay, w);
   return cudaGetLastError();
 }
 

@@ -30,6 +30,50 @@ struct RecBF16 {      // 8 bytes
   uint32_t meta;      // bits 0-7 delay, 8-15 pad, 16-31 bfloat16 weight
 };
 
+// ---------------------------------------------------------------------------
+// Store layouts.  Records (above) serve the atomic delivery.  A net whose
+// delivery is tiled keeps its synapses split by field instead, so that a
+// delivery reads only what it adds: a record's place in its tile's window,
+// cell = (delay - d_base) TW + (target - first target of the tile), fits 16
+// bits whenever the tile's accumulator fits shared memory (d_base: the
+// delay range's lower end at build; TW: targets per tile), and the row's
+// tile index says which tile a run of records belongs to, so neither the
+// target nor the delay is read.  Per event that is 6 bytes (FP32 weights), 4
+// (BF16) or 2 (uniform weights) instead of 12 or 8.
+//  kLayF32   three arrays over all records: float weight, uint32 target,
+//            uint16 cell.
+//  kLayJ16   BF16, per row of len records at byte 8 row_ptr: len words
+//            {cell | weight << 16}, then len uint32 targets (the row's 8 len
+//            bytes, so that the build's sort keys turn into the row in
+//            place).
+//  kLayI16   the same with the weight as an integer multiple of
+//            2^-acc_qs_min (one-word cells whose weights fit 16 bits so):
+//            the delivery adds it as it stands.
+//  kLayHom   uniform weights: every synapse of a source below hom_split has
+//            weight hom_w[0], every other hom_w[1].  FP32: the arrays of
+//            kLayF32, only the cells being read; BF16, per row: len uint16
+//            cells, len bfloat16 weights, len uint32 targets.
+// Targets (and uniform weights) stay for snn_read_store and the checks.
+// ---------------------------------------------------------------------------
+enum StoreLayout {
+  kLayRecords = 0, kLayF32 = 1, kLayJ16 = 2, kLayHom = 3, kLayI16 = 4
+};
+// The bfloat16 weight of a kLayI16 word's upper half (exact: 8 significant
+// bits), and back.
+__host__ __device__ inline float i16_weight(uint32_t word, int qs) {
+  const int e = 127 - qs;  // (within a normal float's range)
+  const uint32_t u = (uint32_t)e << 23;
+  float s;
+  memcpy(&s, &u, 4);
+  return (float)((int32_t)word >> 16) * s;
+}
+__host__ __device__ inline uint32_t i16_bits(float w, int qs) {
+  const uint32_t u = (uint32_t)(127 + qs) << 23;
+  float s;
+  memcpy(&s, &u, 4);
+  return (uint32_t)(int32_t)(w * s) & 0xFFFFu;
+}
+
 template <int FMT> struct Fmt;
 template <> struct Fmt<SNN_W_FP32_12B> {
   static constexpr int kRecBytes = 12;
@@ -229,6 +273,18 @@ struct NetView {
   uint32_t* counts;         // [n_slots][pitch] or null
   const uint64_t* row_ptr;  // [n+1]
   const void* recs;
+  // store layout (StoreLayout); dat: the array a tiled delivery streams
+  // (weights, joined words or cells), cells: the FP32 cells, row_mul: elements
+  // of dat per record index, d_base: the delay of cell 0
+  int lay;
+  const void* dat;
+  const uint16_t* cells;
+  const uint32_t* tgts;     // kLayF32 and FP32 kLayHom: the targets
+  uint32_t row_mul;
+  int d_base;
+  int lg;                   // log2 of the lanes that share a run
+  uint32_t hom_split;
+  float hom_w[2];
   const uint32_t* tile_off; // [n][n_tiles + 1] row-relative tile starts
   uint32_t tile_w;          // targets per tile (tile tau: [tau tile_w, ...))
   uint32_t n_tiles;
@@ -248,7 +304,6 @@ struct NetView {
   // scale has q - s >= acc_qs_min has lo = 0 for every event
   int acc_words;
   int acc_qs_min;
-  float mean_run;           // synapses per (source, tile): the mean run length
   SpikeEntry* list;         // interval list, capacity list_cap
   uint64_t list_cap;
   // partition exchange: the update also writes its spikes as {src, t} pairs
@@ -385,11 +440,23 @@ cudaError_t build_scatter_edges(const uint32_t* src, const uint32_t* tgt,
 // (n rows of n_tiles + 1 entries).  weights: either the
 // fixed-rule parameters (edge_w == null) or per-edge FP64 weights.
 constexpr uint32_t kSortCap = 16384;  // keys sorted in shared memory (128 KiB)
-// stats (device, 2 words, zeroed by the caller): [0] = largest number of
-// synapses sharing (source, target, delay); [1] = bits of the largest
-// |stored weight| (a non-negative float, ordered as an unsigned integer).
+// stats (device, 4 words, {0, 0, 0xFFFFFFFF, 0} from the caller): [0] =
+// largest number of synapses sharing (source, target, delay); [1] = bits of
+// the largest |stored weight| (a non-negative float, ordered as an unsigned
+// integer); [2], [3] = smallest and largest delay.
+// The arrays of a store: lay, and for FP32 split stores the weight, target
+// and cell arrays inside the allocation (null otherwise).
+struct StoreOut {
+  int lay;
+  int d_base;
+  int qs;       // kLayI16: acc_qs_min
+  void* recs;
+  float* wts;
+  uint32_t* tgts;
+  uint16_t* cells;
+};
 cudaError_t build_sort_pack(int fmt, uint32_t n, const uint64_t* row_ptr,
-                            uint64_t* keys, void* recs, const BuildFixed* b,
+                            uint64_t* keys, StoreOut out, const BuildFixed* b,
                             const double* edge_w, uint32_t max_row,
                             const uint32_t* long_rows, uint32_t n_long,
                             uint64_t* long_scratch,
@@ -400,9 +467,7 @@ cudaError_t launch_fill_i32(int32_t* p, int32_t value, uint64_t n,
                             cudaStream_t s);
 cudaError_t launch_list_to_arrays(const SpikeEntry* list, uint64_t n,
                                   uint32_t* src, int32_t* t, cudaStream_t s);
-cudaError_t unpack_store(int fmt, const void* recs, uint64_t n_syn,
-                         uint32_t* tgt, uint8_t* delay, float* w,
-                         cudaStream_t s);
-cudaError_t delay_range(int fmt, const void* recs, uint64_t n_syn,
-                        unsigned int* dmin_dmax, cudaStream_t s);
+// The store's synapses in row order (any output may be null).
+cudaError_t unpack_store(const NetView& v, uint64_t n_syn, uint32_t* tgt,
+                         uint8_t* delay, float* w, cudaStream_t s);
 }  // namespace snn

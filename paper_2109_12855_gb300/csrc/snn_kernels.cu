@@ -591,15 +591,19 @@ k_deliver(NetView v, unsigned long long* pair_p, unsigned int* done_p,
 // CTA tau owns the targets [tau TW, (tau+1) TW) and accumulates, in shared
 // memory, every event of the list aimed at them for the ring steps
 // base .. base + window - 1 that one interval can reach (base = interval
-// start + min delay).  Rows are sorted by target tile, so the records of
+// start + min delay).  Rows are sorted by target tile, so the synapses of
 // spike j for tile tau are one contiguous run, located by the row's tile
 // index.  (A) the CTA describes a batch of runs in shared memory; (B) its 32
-// warps take U runs at a time from a shared counter and load up to PER
-// records per lane of each before adding any (independent loads in flight).
-// (Staging the runs through shared memory, with bulk copies or per-lane
-// asynchronous copies, was measured slower: each record then passes through
-// shared memory twice beside its two atomics, and every run of ~74 records
-// pays a copy and a wait.)
+// warps take 32 / 2^lg runs at a time, 2^lg lanes a run; a lane reads aligned 16-byte vectors of its run (the store's split
+// layouts, snn_internal.cuh: 8 cells, 4 {cell, weight} words, or 4 weights
+// with their 4 cells), the next runs' vectors being loaded before the current
+// ones are added, and masks the elements outside the run.
+//
+// What bounds it: with 12- or 8-byte records one event cost 1.35 (FP32) or
+// about 1.2 (BF16) warp instructions and the launch was half issue, half
+// load latency (39.6 us FP32 and 31.6 us BF16 at 1.27e9 synapses, 1,350
+// spikes; 118 us at 6.3e9).  The split layouts move 2, 4 or 6 bytes an event,
+// and a 16-byte vector costs one load for 8 or 4 events.
 //
 // Accumulation is exact fixed point: a weight w becomes x = w 2^(q-s),
 // split into hi = rint(x) and lo = rint((x - hi) 2^s) in [-2^(s-1), 2^(s-1)]
@@ -612,76 +616,110 @@ k_deliver(NetView v, unsigned long long* pair_p, unsigned int* done_p,
 // E max|w| 2^(q-s) + E < 2^31, so neither sum can overflow, and the
 // rounding error (<= 2^-(q+1) per event) is below that of FP32
 // accumulation.  If no such scales exist the CTA falls back to FP32
-// shared-memory atomics.  The CTA then adds its cells into the ring buffer
-// with plain coalesced read-modify-writes: no other CTA touches them.
-// An external list whose emission steps span more than the window is
-// delivered by the same CTAs with global atomics instead.
+// shared-memory atomics.
+//
+// Uniform weights (kLayHom): a cell's sum is n0 w0 + n1 w1, so only the two
+// counts are accumulated, in the halves of one 32-bit word (E <= 65,535; one
+// addition of a constant per event, no weight to split), and the flush forms
+// the same hi and lo sums from them.
+//
+// The CTA then adds its cells into the ring buffer with fire-and-forget
+// reductions: no other CTA touches them.  An external list whose emission
+// steps span more than the window is delivered by the same CTAs with global
+// atomics instead.
 // ---------------------------------------------------------------------------
 constexpr int kTileThreads = 1024;
 constexpr int kTileWarps = kTileThreads / 32;
 
-template <int FMT> struct Rec1;
-template <> struct Rec1<SNN_W_FP32_12B> { uint32_t a, b, c; };
-template <> struct Rec1<SNN_W_BF16_8B> { uint32_t a, b; };
+// One lane's vector of a run's stream.
+template <int LAY> struct Vec { uint4 a; };
+template <> struct Vec<kLayF32> {
+  uint4 a;  // weights
+  uint2 c;  // cells
+};
+template <int LAY> struct Lay {
+  static constexpr uint32_t kElems = LAY == kLayHom ? 8u : 4u;
+};
+constexpr int kAhead = 3;  // vectors of a lane loaded ahead, for each of two runs
+template <int LAY>
+__device__ __forceinline__ Vec<LAY> load_vec(const NetView& v, uint64_t i) {
+  Vec<LAY> x;
+  x.a = __ldcs(reinterpret_cast<const uint4*>(v.dat) + i);
+  if constexpr (LAY == kLayF32)
+    x.c = __ldcs(reinterpret_cast<const uint2*>(v.cells) + i);
+  return x;
+}
+// Element k of a vector: its cell and weight (uniform stores: w is unused).
+template <int LAY>
+__device__ __forceinline__ uint32_t vec_cell(const Vec<LAY>& x, int k) {
+  if constexpr (LAY == kLayHom) {
+    const uint32_t w = k < 2 ? x.a.x : k < 4 ? x.a.y : k < 6 ? x.a.z : x.a.w;
+    return k & 1 ? w >> 16 : w & 0xFFFFu;
+  } else if constexpr (LAY == kLayF32) {
+    const uint32_t w = k < 2 ? x.c.x : x.c.y;
+    return k & 1 ? w >> 16 : w & 0xFFFFu;
+  } else {
+    const uint32_t w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
+    return w & 0xFFFFu;
+  }
+}
+template <int LAY>
+__device__ __forceinline__ float vec_weight(const Vec<LAY>& x, int k) {
+  const uint32_t w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
+  return __uint_as_float(LAY == kLayJ16 ? w & 0xFFFF0000u : w);
+}
+template <int LAY>
+__device__ __forceinline__ int vec_int(const Vec<LAY>& x, int k) {
+  const uint32_t w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
+  return (int)w >> 16;
+}
+// Elements of vector jv of a run that lie in it (bit k: element k); the run
+// takes the elements [head, total) of its vectors.
+template <int LAY>
+__device__ __forceinline__ uint32_t vec_mask(uint32_t jv, uint32_t head,
+                                             uint32_t total) {
+  constexpr uint32_t E = Lay<LAY>::kElems;
+  const int hi = (int)total - (int)(jv * E);
+  uint32_t m = hi >= (int)E ? (1u << E) - 1u : hi <= 0 ? 0u : (1u << hi) - 1u;
+  if (jv == 0) m &= ~0u << head;
+  return m;
+}
 
-template <int FMT>
-__device__ __forceinline__ Rec1<FMT> load_rec(const void* recs, uint64_t r);
-template <>
-__device__ __forceinline__ Rec1<SNN_W_FP32_12B> load_rec<SNN_W_FP32_12B>(
-    const void* recs, uint64_t r) {
-  const uint32_t* p = reinterpret_cast<const uint32_t*>(recs) + r * 3u;
-  Rec1<SNN_W_FP32_12B> x;
-  x.a = __ldcs(p);
-  x.b = __ldcs(p + 1);
-  x.c = __ldcs(p + 2);
-  return x;
+__device__ __forceinline__ void red_shared_u32(uint32_t addr, uint32_t x) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
 }
-template <>
-__device__ __forceinline__ Rec1<SNN_W_BF16_8B> load_rec<SNN_W_BF16_8B>(
-    const void* recs, uint64_t r) {
-  const uint2 u = __ldcs(reinterpret_cast<const uint2*>(recs) + r);
-  Rec1<SNN_W_BF16_8B> x;
-  x.a = u.x;
-  x.b = u.y;
-  return x;
-}
-// FP32 records, interval-list launches: only the weight and the delay word,
-// whose upper 24 bits hold the record's cell in its tile's window,
-// d TW + (target - first target of the tile), written by the store build.
-__device__ __forceinline__ Rec1<SNN_W_FP32_12B> load_rec_wc(const void* recs,
-                                                           uint64_t r) {
-  const uint32_t* p = reinterpret_cast<const uint32_t*>(recs) + r * 3u;
-  Rec1<SNN_W_FP32_12B> x;
-  x.a = 0u;
-  x.b = __ldcs(p + 1);
-  x.c = __ldcs(p + 2);
-  return x;
-}
-__device__ __forceinline__ void rec_fields(const Rec1<SNN_W_FP32_12B>& x,
-                                           uint32_t& tgt, uint32_t& d,
-                                           float& w) {
-  tgt = x.a;
-  w = __uint_as_float(x.b);
-  d = x.c & 0xFFu;
-}
-__device__ __forceinline__ void rec_fields(const Rec1<SNN_W_BF16_8B>& x,
-                                           uint32_t& tgt, uint32_t& d,
-                                           float& w) {
-  tgt = x.a;
-  d = x.b & 0xFFu;
-  w = __uint_as_float(x.b & 0xFFFF0000u);
+// The same where K < n (and, CLIP, K >= lo), else into the lane's own spare
+// word `none`: a select, as a conditional reduction compiles to a branch (three
+// branch instructions per reduction, 1.25 against 0.8 instructions per event).
+template <int K, bool CLIP>
+__device__ __forceinline__ void red_shared_u32_at(uint32_t addr, uint32_t x,
+                                                  int n, int lo, uint32_t none) {
+  const bool on = CLIP ? (K < n && K >= lo) : K < n;
+  red_shared_u32(on ? addr : none, x);
 }
 
-// Per-spike run of records for this CTA's tile.
+// base + 4 x the low (0) or high (1) half of w: one integer dot product.
+template <int HALF>
+__device__ __forceinline__ uint32_t cell_addr(uint32_t w, uint32_t base) {
+  return __dp2a_lo(w, HALF ? 0x0400u : 0x0004u, base);
+}
+
+// Per-spike run for this CTA's tile: its first element in the store's stream,
+// its length (top bit: uniform weight class), and the offset of its cells in
+// the accumulator, (t - base + d_base) TW (a list outside the window: t).
 struct SegDesc {
   uint64_t beg;
   uint32_t len;
-  int32_t t;
+  int32_t off;
+#if SNN_CHECK
+  uint64_t tgt;  // index of the run's first target, in words of its array
+#endif
 };
 
 // Fixed-point scales of one launch (see above); fixed = 0: use FP32.
 struct FixScale {
   int fixed;
+  int packed;      // uniform weights: the counts fit 16 bits
   int sh;          // s
   float scale_hs;  // 2^(q - s)
   float scale_s;   // 2^s
@@ -708,12 +746,13 @@ constexpr int kFixMaxShift = 23;
 
 __device__ FixScale fix_scale(const NetView& v, uint64_t n_sp,
                               bool per_interval) {
-  FixScale f{0, 0, 1.f, 1.f, 1.f, 1.f};
+  FixScale f{0, 0, 0, 1.f, 1.f, 1.f, 1.f};
   uint64_t e = n_sp * (uint64_t)(v.mult_max ? v.mult_max : 1u);
   if (per_interval) {
     const uint64_t e2 = (uint64_t)v.k_in_max * (v.spikes_per_iv ? v.spikes_per_iv : 1u);
     if (e2 < e) e = e2;
   }
+  f.packed = e <= 0xFFFFull;
   if (e == 0 || e >= (1ull << 30) || !(v.max_abs_w > 0.f) ||
       !(v.max_abs_w <= 3.0e38f))
     return f;
@@ -732,6 +771,8 @@ __device__ FixScale fix_scale(const NetView& v, uint64_t n_sp,
   qs = min(qs, 100);
   // one-word cells hold hi only: lo must be zero for every weight
   if (v.acc_words == 1 && qs < v.acc_qs_min) return f;
+  // (integer weights: the store's own scale, at most the launch's)
+  if (v.lay == kLayI16) qs = v.acc_qs_min;
   const int q = sh + qs;
   f.fixed = 1;
   f.sh = sh;
@@ -742,20 +783,50 @@ __device__ FixScale fix_scale(const NetView& v, uint64_t n_sp,
   return f;
 }
 
+// The two scales a split needs.
+struct SplitScale {
+  float scale_hs, scale_s;
+};
+
 // Exact split of x = w 2^(q-s) (|x| < 2^22, s <= 23): hi = rint(x),
 // lo = rint((x - hi) 2^s), so hi 2^s + lo = rint(w 2^q).  Adding
 // M = 1.5 2^23 puts a value of magnitude <= 2^22 into [2^23, 2^24], where
 // the float spacing is 1: the sum is rounded to an integer (to nearest,
 // ties to even) whose value is the bit pattern minus M's.  Only FMA-pipe
-// arithmetic and integer subtractions; x - hi is exact.
-__device__ __forceinline__ void fixed_split(float w, const FixScale& fx,
+// arithmetic and integer subtractions; x (a product with a power of two) and
+// x - hi are exact, so the fused forms round once, at the additions of M.
+constexpr float kFixM = 12582912.0f;  // 1.5 * 2^23
+template <class Scale>
+__device__ __forceinline__ void fixed_split(float w, const Scale& fx,
                                             int& hi, int& lo) {
-  constexpr float kM = 12582912.0f;  // 1.5 * 2^23
-  const float x = __fmul_rn(w, fx.scale_hs);
-  const float y = __fadd_rn(x, kM);
-  hi = __float_as_int(y) - __float_as_int(kM);
-  const float fr = __fsub_rn(x, __fsub_rn(y, kM));
-  lo = __float_as_int(__fmaf_rn(fr, fx.scale_s, kM)) - __float_as_int(kM);
+  const float y = __fmaf_rn(w, fx.scale_hs, kFixM);
+  hi = __float_as_int(y) - __float_as_int(kFixM);
+  const float fr = __fmaf_rn(w, fx.scale_hs, -__fsub_rn(y, kFixM));
+  lo = __float_as_int(__fmaf_rn(fr, fx.scale_s, kFixM)) - __float_as_int(kFixM);
+}
+
+// Delay steps above d_base of a cell (cell / TW) by a multiplication: with
+// m = floor(2^32 / TW) + 1, cell m / 2^32 exceeds cell / TW by less than
+// cell / 2^32 < 1 / TW (cells are below 2^16), so the floor is the same.
+__device__ __forceinline__ uint32_t cell_magic(uint32_t tw) {
+  return tw > 1u ? (uint32_t)(0x100000000ull / tw) + 1u : 0u;
+}
+__device__ __forceinline__ uint32_t cell_step(uint32_t cell, uint32_t magic) {
+  return magic ? __umulhi(cell, magic) : cell;  // (one target a tile)
+}
+
+// Bounds-checked builds: a cell outside the store's window or one that
+// disagrees with the synapse's target is skipped and flagged; so are targets
+// outside the tile.  Production builds compile this to `true`.
+__device__ __forceinline__ bool cell_in_bounds(const NetView& v, uint32_t cell,
+                                               uint32_t tgt, uint32_t tgt_lo) {
+  if (!kChecked) return true;
+  const uint32_t d = cell / v.tile_w, j = cell - d * v.tile_w;
+  const bool ok = tgt < v.n && tgt == tgt_lo + j &&
+                  d + (uint32_t)v.d_base >= (uint32_t)v.d_min &&
+                  d + (uint32_t)v.d_base <= (uint32_t)v.d_max;
+  if (!ok) atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_CHECK);
+  return ok;
 }
 
 // Plastic weight of an E->E synapse at its presynaptic spike t with delay
@@ -816,58 +887,351 @@ __device__ __noinline__ StdpOut stdp_weight(float w, int32_t t, uint32_t d,
   return o;
 }
 
-// FAST: an interval's own list (inside the window) whose fixed-point scales
-// the host has shown to exist for every spike count: no per-event test of
-// either.
-// ONE: one-word cells known at compile time (BF16 stores).  SHORT: runs of
-// a few dozen records (BF16, static): eight runs per warp pass, each on half
-// a warp (48 record slots per run instead of 96).
-template <int FMT, bool COUNT, bool PL, bool FAST = false, bool ONE = false,
-          bool SHORT = false, bool GX = false>
+// The launch's list as a delivery sees it: its length, the window's base
+// step, whether its steps lie inside the window, and the clock.
+struct ListView {
+  uint32_t n_sp;
+  bool inwin;
+  long long base, t_now;
+};
+
+// Descriptors of the runs of spikes [j0, j0 + nb) for this CTA's tile: DU
+// list entries per thread in flight, then their tile-index words and row
+// starts.  pre (pre_g): entries threadIdx.x + u blockDim.x of the list, read
+// ahead of its length (have_pre).  Returns the events described (gathered
+// lists).  PL: also the presynaptic history the plastic rule needs.
+template <int DU, bool PL, bool GX>
+__device__ __forceinline__ unsigned long long describe_runs(
+    const NetView& v, const ListView& lv, const SpikeEntry* list, uint32_t tile,
+    uint32_t j0, uint32_t nb, bool have_pre, const SpikeEntry* pre,
+    const uint2* pre_g, const uint32_t* s_gstart, SegDesc* s_desc,
+    int32_t* s_tprev, float* s_kprev, uint32_t* s_at) {
+  const uint32_t row_stride = v.n_tiles + 1;
+  const uint32_t iv_span = (uint32_t)(v.window - (v.d_max - v.d_min));
+  unsigned long long my_events = 0;
+  for (uint32_t k0 = threadIdx.x; k0 < nb; k0 += DU * blockDim.x) {
+    uint32_t src[DU];
+    int32_t t[DU];
+    const bool have = have_pre && j0 == 0 && k0 == threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < DU; ++u) {
+      const uint32_t k = k0 + u * blockDim.x;
+      src[u] = 0xFFFFFFFFu;
+      t[u] = 0;
+      if (k < nb) {
+        if constexpr (GX) {
+          const uint32_t g = j0 + k;
+          uint32_t p = 0;
+          while (s_gstart[p + 1] <= g) ++p;
+          const uint2 x = (have && p == 0)
+              ? pre_g[u]
+              : reinterpret_cast<const uint2*>(
+                    v.gx + (uint64_t)p * v.gx_stride + 4)[g - s_gstart[p]];
+          // entries come from the caller's buffers: a source outside the
+          // store or a step outside this interval is skipped and flagged
+          // (its cells would lie outside the tile's window)
+          const bool ok = x.x < v.n_src &&
+                          (uint32_t)((int32_t)x.y - (int32_t)lv.t_now) < iv_span;
+          if (!ok) atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_BAD_SOURCE);
+          src[u] = ok ? x.x : 0xFFFFFFFFu;
+          t[u] = (int32_t)x.y;
+        } else {
+          const SpikeEntry e = have ? pre[u] : list[j0 + k];
+          src[u] = e.src;
+          t[u] = e.t;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < DU; ++u) {
+      const uint32_t k = k0 + u * blockDim.x;
+      if (k >= nb) continue;
+      SegDesc sd{};
+      sd.off = lv.inwin ? (int32_t)((long long)t[u] - lv.base + v.d_base) *
+                              (int32_t)v.tile_w
+                        : t[u];
+      if (src[u] < v.n_src) {
+        const uint32_t* to = v.tile_off + (uint64_t)src[u] * row_stride + tile;
+        const uint32_t a = to[0], b = to[1];
+        const uint64_t row = v.row_ptr[src[u]];
+        sd.beg = row * v.row_mul + a;
+        sd.len = b - a;
+#if SNN_CHECK
+        const uint64_t row_end = v.row_ptr[src[u] + 1];
+        sd.tgt = v.fmt == SNN_W_FP32_12B ? row + a
+                                         : 2 * row + (row_end - row) + a;
+        if (b < a || row + b > row_end) {
+          atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_CHECK);
+          sd.len = 0;
+        }
+#endif
+        if (GX) my_events += sd.len;
+        if (v.lay == kLayHom && src[u] >= v.hom_split) sd.len |= 0x80000000u;
+        if constexpr (PL) s_at[k] = a;
+      }
+      s_desc[k] = sd;
+      if constexpr (PL) {
+        const bool exc = src[u] < v.sp.n_exc;
+        s_tprev[k] = exc ? v.sp.prev_t[src[u]] : kNoSpike;
+        s_kprev[k] = exc ? v.sp.prev_k[src[u]] : -1.f;
+      }
+    }
+  }
+  // gathered lists: the warp's events (all threads of the CTA reach this)
+  if (GX) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) my_events += __shfl_xor_sync(kFull, my_events, o);
+  }
+  return my_events;
+}
+
+// Value of one accumulator cell, the FP32 sum of its events: exact sums
+// (H 2^s + L) 2^-q as H 2^(s-q) + L 2^-q (both products are exact while |H|
+// and |L| are below 2^24 -- then only the addition rounds, so the result is
+// the correctly rounded sum; larger words round once more; no 64-bit
+// conversion or FP64 arithmetic, whose rate is low on this part).  Uniform
+// weights: H and L from the two counts of the cell.
+enum CellKind { kCellFloat, kCellOne, kCellTwo, kCellCounts, kCellCountsOne,
+                kCellCountsFloat };
+struct CellValue {
+  float scale_sq, inv_q;
+  int h0, l0, h1, l1;
+  float w0, w1;
+  __device__ __forceinline__ CellValue(const NetView& v, const FixScale& f)
+      : scale_sq(f.scale_sq), inv_q(f.inv_q), h0(0), l0(0), h1(0), l1(0),
+        w0(v.hom_w[0]), w1(v.hom_w[1]) {
+    if (v.lay == kLayHom && f.fixed) {
+      fixed_split(w0, f, h0, l0);
+      fixed_split(w1, f, h1, l1);
+    }
+  }
+  // c: the cell's index; cells: the accumulator's
+  template <int KIND>
+  __device__ __forceinline__ float get(const int* acc, uint32_t c,
+                                       uint32_t cells) const {
+    int H = acc[c], L = 0;
+    if (KIND == kCellFloat) return __int_as_float(H);
+    if (KIND >= kCellCounts) {
+      const int n0 = H & 0xFFFF, n1 = (int)((uint32_t)H >> 16);
+      if (KIND == kCellCountsFloat) return (float)n0 * w0 + (float)n1 * w1;
+      H = n0 * h0 + n1 * h1;
+      L = n0 * l0 + n1 * l1;
+    } else if (KIND == kCellTwo) {
+      L = acc[cells + c];
+    }
+    float a = __fmul_rn(__int2float_rn(H), scale_sq);
+    if (KIND == kCellTwo || KIND == kCellCounts)
+      a = __fadd_rn(a, __fmul_rn(__int2float_rn(L), inv_q));
+    return a;
+  }
+};
+
+// Adds the tile's window into the ring buffer: every cell belongs to this CTA
+// alone, so its sum goes out as a fire-and-forget global reduction: the one
+// addition rb + sum that a read-modify-write would make, without a memory
+// round trip (the slots of a column are independent: unrolled, so that their
+// shared-memory reads and conversions overlap).
+template <int KIND>
+__device__ __forceinline__ void flush_kind(const NetView& v, const CellValue& val,
+                                           const int* acc, uint32_t tgt_lo,
+                                           long long base) {
+  const uint32_t TW = v.tile_w, W = (uint32_t)v.window, cells = W * TW;
+  const uint32_t x_end = tgt_lo < v.n ? min(TW, v.n - tgt_lo) : 0u;
+  for (uint32_t x = threadIdx.x; x < x_end; x += blockDim.x) {
+    float* const col = v.rb + tgt_lo + x;
+#pragma unroll 4
+    for (uint32_t sl = 0; sl < W; ++sl) {
+      const float a = val.get<KIND>(acc, sl * TW + x, cells);
+      if (a != 0.f)
+        red_add_f32(col + (size_t)((uint32_t)(base + sl) & v.slot_mask) * v.pitch, a);
+    }
+  }
+}
+template <bool HOM>
+__device__ __forceinline__ void flush_tile(const NetView& v, const FixScale& fx,
+                                           bool two, const int* acc,
+                                           uint32_t tgt_lo, long long base) {
+  const CellValue val(v, fx);
+  if (HOM && fx.packed) {
+    if (!fx.fixed) flush_kind<kCellCountsFloat>(v, val, acc, tgt_lo, base);
+    else if (two) flush_kind<kCellCounts>(v, val, acc, tgt_lo, base);
+    else flush_kind<kCellCountsOne>(v, val, acc, tgt_lo, base);
+  } else if (!fx.fixed) {
+    flush_kind<kCellFloat>(v, val, acc, tgt_lo, base);
+  } else if (two) {
+    flush_kind<kCellTwo>(v, val, acc, tgt_lo, base);
+  } else {
+    flush_kind<kCellOne>(v, val, acc, tgt_lo, base);
+  }
+}
+
+// A CTA's end of a list: the last of the list's CTAs clears its counters and,
+// for the interval's own list, commits its events and advances the clock.
+__device__ __forceinline__ void finish_list(const NetView& v,
+                                            unsigned long long* pair_p,
+                                            unsigned int* done_p,
+                                            int advance_time, bool gathered) {
+  __threadfence();
+  const unsigned prev = atomicAdd(done_p, 1u);
+  if (prev != v.n_tiles - 1) return;
+  *pair_p = 0ull;
+  *done_p = 0u;
+  if (!advance_time) return;
+  // this net's exchange list has been read (by the collective before this
+  // delivery, or by this delivery itself): the next update refills it
+  if (v.xbuf) *v.xbuf = 0u;
+  v.ctl->t_now += v.ctl->iv_steps;
+  const unsigned long long own = atomicExch(&v.ctl->pending_events, 0ull);
+  v.ctl->events += gathered ? atomicExch(&v.ctl->gx_events, 0ull) : own;
+}
+
+// The events of one vector: elements K of [lo, n) (CLIP; else [0, n)).
+template <int LAY, bool CLIP, int K>
+__device__ __forceinline__ void add_elem(const Vec<LAY>& x, uint32_t row_s,
+                                         uint32_t inc, int n, int lo,
+                                         uint32_t lo_off, uint32_t none,
+                                        const SplitScale& fx) {
+  if constexpr (LAY == kLayHom) {
+    const uint32_t w = K < 2 ? x.a.x : K < 4 ? x.a.y : K < 6 ? x.a.z : x.a.w;
+    red_shared_u32_at<K, CLIP>(cell_addr<K & 1>(w, row_s), inc, n, lo, none);
+  } else if constexpr (LAY == kLayI16) {
+    const uint32_t w = K == 0 ? x.a.x : K == 1 ? x.a.y : K == 2 ? x.a.z : x.a.w;
+    red_shared_u32_at<K, CLIP>(cell_addr<0>(w, row_s), (uint32_t)((int)w >> 16), n, lo,
+                               none);
+  } else {
+    uint32_t addr;
+    if constexpr (LAY == kLayF32)
+      addr = cell_addr<K & 1>(K < 2 ? x.c.x : x.c.y, row_s);
+    else
+      addr = cell_addr<0>(K == 0 ? x.a.x : K == 1 ? x.a.y : K == 2 ? x.a.z : x.a.w, row_s);
+    int hi, low;
+    fixed_split(vec_weight<LAY>(x, K), fx, hi, low);
+    red_shared_u32_at<K, CLIP>(addr, (uint32_t)hi, n, lo, none);
+    // (one-word cells have no low part)
+    if constexpr (LAY == kLayF32)
+      red_shared_u32_at<K, CLIP>(addr + lo_off, (uint32_t)low, n, lo, none);
+    else
+      red_shared_u32_at<K, CLIP>(addr + lo_off, (uint32_t)low,
+                                 lo_off ? n : 0, lo, none);
+  }
+}
+template <int LAY, bool CLIP>
+__device__ __forceinline__ void add_vec(const Vec<LAY>& x, uint32_t row_s,
+                                        uint32_t inc, int n, int lo,
+                                        uint32_t lo_off, uint32_t none,
+                                        const SplitScale& fx) {
+  add_elem<LAY, CLIP, 0>(x, row_s, inc, n, lo, lo_off, none, fx);
+  add_elem<LAY, CLIP, 1>(x, row_s, inc, n, lo, lo_off, none, fx);
+  add_elem<LAY, CLIP, 2>(x, row_s, inc, n, lo, lo_off, none, fx);
+  add_elem<LAY, CLIP, 3>(x, row_s, inc, n, lo, lo_off, none, fx);
+  if constexpr (Lay<LAY>::kElems == 8) {
+    add_elem<LAY, CLIP, 4>(x, row_s, inc, n, lo, lo_off, none, fx);
+    add_elem<LAY, CLIP, 5>(x, row_s, inc, n, lo, lo_off, none, fx);
+    add_elem<LAY, CLIP, 6>(x, row_s, inc, n, lo, lo_off, none, fx);
+    add_elem<LAY, CLIP, 7>(x, row_s, inc, n, lo, lo_off, none, fx);
+  }
+}
+
+// A lane's part of one run: its first vectors, the elements of the run from
+// the first of them on (n; those before `lo` belong to the row's previous
+// run), the run's cells in the accumulator and its increment.
+template <int LAY> struct LaneRun {
+  Vec<LAY> x[kAhead];
+  const char* p;   // the lane's first vector (cells: FP32 layouts)
+  int n, lo;
+  uint32_t row_s, inc;
+};
+
+// Phase (B) for a batch of nb described runs, 2^lg lanes a run: every warp
+// takes each kTileWarps-th group of 32 / 2^lg runs, and loads a lane's first
+// kAhead vectors of the next group before it adds the current one.
+template <int LAY>
+__device__ __forceinline__ void add_runs(const char* dat, const char* cel,
+                                      const SegDesc* s_desc, uint32_t nb,
+                                      uint32_t acc_s, uint32_t lo_off,
+                                      uint32_t lg, SplitScale fx) {
+  constexpr uint32_t E = Lay<LAY>::kElems;
+  __shared__ uint32_t s_none[32];  // what masked elements add to
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t none = (uint32_t)__cvta_generic_to_shared(s_none + lane);
+  const uint32_t L = 1u << lg, R = 32u >> lg;
+  const int kStep = (int)(L * E);  // elements between a lane's vectors
+  const uint32_t sub = lane & (L - 1u);
+  const uint32_t stride = kTileWarps * R;
+  // (FP32 weights at dat: their cells, half the bytes, at cel)
+  auto fetch = [&](const LaneRun<LAY>& r, int q) {
+    const char* p = r.p + (size_t)q * (L * 16u);
+    Vec<LAY> x;
+    x.a = __ldcs(reinterpret_cast<const uint4*>(p));
+    if constexpr (LAY == kLayF32)
+      x.c = __ldcs(reinterpret_cast<const uint2*>(cel + ((p - dat) >> 1)));
+    return x;
+  };
+  auto load = [&](LaneRun<LAY>& r, uint32_t j) {
+    r.n = 0;
+    if (j < nb) {
+      const SegDesc sd = s_desc[j];
+      const uint32_t head = (uint32_t)sd.beg & (E - 1u);
+      r.p = dat + (sd.beg / E + sub) * 16u;
+      r.lo = sub == 0 ? (int)head : 0;
+      r.n = (int)(head + (sd.len & 0x7FFFFFFFu)) - (int)(sub * E);
+      r.row_s = acc_s + 4u * (uint32_t)sd.off;
+      r.inc = (int)sd.len < 0 ? 0x10000u : 1u;
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q)
+        if (r.n > q * kStep) r.x[q] = fetch(r, q);
+    }
+  };
+  auto add = [&](LaneRun<LAY>& r) {
+    if (r.n > 0) add_vec<LAY, true>(r.x[0], r.row_s, r.inc, r.n, r.lo, lo_off, none, fx);
+#pragma unroll
+    for (int q = 1; q < kAhead; ++q)
+      if (r.n > q * kStep)
+        add_vec<LAY, false>(r.x[q], r.row_s, r.inc, r.n - q * kStep, 0, lo_off,
+                            none, fx);
+    for (int q = kAhead; r.n > q * kStep; ++q) {
+      const Vec<LAY> x = fetch(r, q);
+      add_vec<LAY, false>(x, r.row_s, r.inc, r.n - q * kStep, 0, lo_off,
+                            none, fx);
+    }
+  };
+  uint32_t k = (threadIdx.x >> 5) * R;
+  const uint32_t grp = lane >> lg;
+  LaneRun<LAY> a, b;
+  load(a, k + grp);
+  for (; k < nb; k += 2 * stride) {
+    load(b, k + stride + grp);
+    add(a);
+    load(a, k + 2 * stride + grp);
+    add(b);
+  }
+}
+
+// One interval's (or one caller's) list for tile `tile`.
+template <int LAY, bool COUNT, bool GX>
 __device__ __forceinline__ void deliver_tile_body(
     const NetView& v, unsigned long long* pair_p, unsigned int* done_p,
     const SpikeEntry* __restrict__ list, int from_list_range, int advance_time,
     uint32_t tile, int* acc_mem, uint32_t desc_off, uint32_t desc_cap) {
-  // U runs per warp pass, PER records per lane of each loaded before use
-  // (plastic nets also hold each record's plastic weight: fewer runs)
-  constexpr int U = PL ? (FMT == SNN_W_FP32_12B ? 1 : 2)
-                       : (FMT == SNN_W_FP32_12B ? 2 : (SHORT ? 8 : 4));
-  constexpr int PER = 3;
-  // lanes per run: short runs take half a warp each, two side by side (48
-  // record slots per run instead of a whole warp's)
-  constexpr int LG = SHORT ? 16 : 32;
-  constexpr int G = 32 / LG;   // runs side by side in a warp
-  constexpr int UR = U / G;    // run slots of a lane per pass
-  static_assert(U % G == 0, "runs per pass must fill the warp");
-  // FP32 interval lists: each record's cell comes precomputed in its delay
-  // word (no target load, no d TW + target arithmetic); bounds-checked
-  // builds keep the checked form
-  constexpr bool CELL = FAST && FMT == SNN_W_FP32_12B && !PL && !COUNT && !kChecked;
-  // run descriptors of one batch (desc_cap spikes), after the accumulator
+  constexpr uint32_t E = Lay<LAY>::kElems;
   SegDesc* const s_desc =
       reinterpret_cast<SegDesc*>(reinterpret_cast<char*>(acc_mem) + desc_off);
-  int32_t* const s_tprev = reinterpret_cast<int32_t*>(s_desc + desc_cap);  // PL
-  float* const s_kprev = reinterpret_cast<float*>(s_tprev + desc_cap);     // PL
-  __shared__ unsigned long long s_pl[2];             // plastic updates, truncations
-  __shared__ uint32_t s_next;                        // next run of the batch
   __shared__ FixScale s_fx;
+  __shared__ uint32_t s_gstart[GX ? kMaxGatherParts + 1 : 1];
+  __shared__ unsigned long long s_events;  // gathered lists: this CTA's events
   const uint32_t TW = v.tile_w;
   const uint32_t W = (uint32_t)v.window;
   const uint32_t cells = W * TW;
-  // hi and lo words per cell (FP32 stores always use two: their 24-bit
-  // significands never sit on a grid as coarse as a launch's step)
-  const bool two = FMT == SNN_W_FP32_12B || (!ONE && v.acc_words == 2);
-  const uint32_t acc_len = two ? 2 * cells : cells;
+  // hi and lo words per cell (FP32 weights' 24-bit significands never sit on
+  // a grid as coarse as a launch's step)
+  const bool two = LAY != kLayI16 && v.acc_words == 2;
   const uint32_t tgt_lo = tile * TW;
   const unsigned lane = threadIdx.x & 31u;
-  const uint32_t warp = threadIdx.x >> 5;
   // An interval's own list (capacity list_cap): this thread's first list
   // entries are read together with the list's length, not after it (one
   // memory round trip fewer before the runs can be described); entries past
   // the length are never used.
-  constexpr int kDU = PL ? 1 : 4;
-  // GX: the list is gathered from the partitions' exchange buffers (v.gx)
-  constexpr bool gathered = GX;
+  constexpr int kDU = 4;
   SpikeEntry pre[GX ? 1 : kDU];
   uint2 pre_g[GX ? kDU : 1];
   const bool spec = !from_list_range;
@@ -885,12 +1249,11 @@ __device__ __forceinline__ void deliver_tile_body(
   }
   // every thread reads the launch's list size and window (same addresses);
   // thread 0 derives the fixed-point scales meanwhile
-  uint32_t n_sp;
-  // a list gathered from the partitions: the parts' counts (each at most
-  // its capacity) and their starts in the union, in part order; every
-  // thread computes them (same values, no barrier) from the same words
-  __shared__ uint32_t s_gstart[kMaxGatherParts + 1];
+  ListView lv;
   if constexpr (GX) {
+    // the parts' counts (each at most its capacity) and their starts in the
+    // union, in part order; every thread computes them (same values, no
+    // barrier) from the same words
     uint32_t run = 0;
     for (uint32_t p = 0; p < v.gx_parts; ++p) {
       s_gstart[p] = run;
@@ -899,425 +1262,421 @@ __device__ __forceinline__ void deliver_tile_body(
                  v.gx_cap);
     }
     s_gstart[v.gx_parts] = run;
-    n_sp = run;
+    lv.n_sp = run;
   } else {
     const unsigned long long pr =
         *reinterpret_cast<volatile unsigned long long*>(pair_p);
-    n_sp = (uint32_t)(pr >> 32);
+    lv.n_sp = (uint32_t)(pr >> 32);
   }
-  long long base;
-  bool inwin;
-  // gathered lists: steps of this interval lie in [t_now, t_now + iv_span)
-  const long long t_now = gathered ? v.ctl->t_now : 0ll;
-  const uint32_t iv_span = (uint32_t)(W - (uint32_t)(v.d_max - v.d_min));
+  lv.t_now = GX ? v.ctl->t_now : 0ll;
   if (from_list_range) {
     const long long tmin = v.ctl->ext_tmin, tmax = v.ctl->ext_tmax;
-    base = tmin + v.d_min;
-    inwin = (tmax - tmin) + (v.d_max - v.d_min) + 1 <= (long long)W;
+    lv.base = tmin + v.d_min;
+    lv.inwin = (tmax - tmin) + (v.d_max - v.d_min) + 1 <= (long long)W;
   } else {
-    base = v.ctl->t_now + v.d_min;
-    inwin = true;
+    lv.base = v.ctl->t_now + v.d_min;
+    lv.inwin = true;
   }
-  if (threadIdx.x == 0) {
-    s_fx = fix_scale(v, n_sp, !from_list_range);
-    s_next = 0u;
-  }
-  int* accH = acc_mem;                                // fixed: hi parts
-  int* accL = acc_mem + cells;                        // fixed: lo parts (two)
-  float* accF = reinterpret_cast<float*>(acc_mem);    // FP32 fallback
-  for (uint32_t x = threadIdx.x; x < acc_len; x += blockDim.x) acc_mem[x] = 0;
-  // plastic nets: the post-spike times of this tile's targets (rings) and
-  // their post traces at the W horizons (t - d) this interval can ask for
-  int32_t* s_rt = acc_mem + acc_len;                             // [hist][TW]
-  uint32_t* s_rn = reinterpret_cast<uint32_t*>(s_rt + (PL ? v.sp.hist * TW : 0));
-  float* s_km = reinterpret_cast<float*>(s_rn + (PL ? TW : 0));  // [W][TW]
-  const bool tile_plastic = PL && tgt_lo < v.sp.n_exc;
-  uint32_t my_pl = 0, my_trunc = 0;
-  // first horizon: (interval start) - d_max
-  const long long h_lo = base - v.d_min - v.d_max;
-  if (PL) {
-    if (threadIdx.x < 2) s_pl[threadIdx.x] = 0ull;
-    if (tile_plastic) {
-      for (uint32_t x = threadIdx.x; x < TW; x += blockDim.x)
-        s_rn[x] = tgt_lo + x < v.n ? v.sp.ring_n[tgt_lo + x] : 0u;
-      for (uint32_t x = threadIdx.x; x < v.sp.hist * TW; x += blockDim.x) {
-        const uint32_t q = x / TW, jj = x - q * TW;
-        if (tgt_lo + jj < v.n)
-          s_rt[x] = v.sp.ring_t[(size_t)q * v.pitch + tgt_lo + jj];
-      }
-      __syncthreads();
-      // post trace of target j at horizon h: the trace right after its
-      // latest spike at or before h, decayed to h (0 if it never fired)
-      const uint32_t hm = v.sp.hist - 1u;
-      for (uint32_t x = threadIdx.x; x < W * TW; x += blockDim.x) {
-        const uint32_t hi = x / TW, jj = x - hi * TW;
-        const int32_t h = (int32_t)(h_lo + hi);
-        const uint32_t n = s_rn[jj];
-        const int32_t k_min = n > v.sp.hist ? (int32_t)(n - v.sp.hist) : 0;
-        float km = 0.f;
-        int32_t k = (int32_t)n - 1;
-        for (; k >= k_min; --k) {
-          const int32_t tp = s_rt[((uint32_t)k & hm) * TW + jj];
-          if (tp <= h) {
-            km = v.sp.ring_k[(size_t)((uint32_t)k & hm) * v.pitch + tgt_lo + jj] *
-                 exp2f(-(float)(h - tp) * v.sp.l2_minus);
-            break;
-          }
-        }
-        // every kept spike is after h but older ones were dropped: the
-        // trace at h is unknown (-1; an update that needs it is counted
-        // with the truncated windows)
-        s_km[x] = (k < k_min && n > v.sp.hist) ? -1.f : km;
-      }
-    }
-  }
-  const uint32_t row_stride = v.n_tiles + 1;
+  const uint32_t n_sp = lv.n_sp;
+  const long long base = lv.base;
+  // (the last thread: it describes no run of a list of up to 1,023 spikes)
+  if (threadIdx.x == kTileThreads - 1) s_fx = fix_scale(v, n_sp, !from_list_range);
+  if (GX && threadIdx.x == 0) s_events = 0ull;
+  // (an interval's own list of a uniform store always fits its counts when
+  // the largest interval's does: one word a cell)
+  const bool one = !two || (LAY == kLayHom && !from_list_range &&
+                            (uint64_t)v.k_in_max * v.spikes_per_iv <= 0xFFFFull);
+  for (uint32_t x = threadIdx.x; x < (one ? cells : 2 * cells); x += blockDim.x)
+    acc_mem[x] = 0;
+  const uint32_t acc_s = (uint32_t)__cvta_generic_to_shared(acc_mem);
   FixScale fx{};  // thread 0's s_fx, read after the first barrier
-  __shared__ unsigned long long s_events;  // gathered lists: this CTA's events
-  if (gathered && threadIdx.x == 0) s_events = 0ull;
 
-  // one event: cell = d TW + tgt + off, off = (t - base) TW - tgt_lo per run
-  auto add = [&](uint32_t tgt, int32_t t, int32_t off, uint32_t d, float w) {
-    if (FAST || inwin) {
-      const uint32_t cell = d * TW + tgt + (uint32_t)off;
-      if (FAST || fx.fixed) {
+  // lanes of this warp's runs: 2^lg of them share run `grp` of the warp's
+  uint32_t lg = 0, n_lanes = 1, runs = 32, sub = 0, grp = lane;
+
+  // one event in every other case: uniform weights whose counts do not fit,
+  // no fixed-point scales, a list outside the window, counted cells
+  auto add_slow = [&](uint32_t cell, const SegDesc& sd, float w) {
+    if (lv.inwin) {
+      const uint32_t c = (uint32_t)sd.off + cell;
+      if (LAY == kLayHom && fx.packed) {
+        red_shared_u32(acc_s + 4u * c, (int)sd.len < 0 ? 0x10000u : 1u);
+      } else if (fx.fixed) {
         int hi, lo;
         fixed_split(w, fx, hi, lo);
-        atomicAdd(&accH[cell], hi);
-        // BF16 weights have 8 significant bits: their scaled value is
-        // usually an integer, and a zero low part needs no addition (with
-        // one-word cells it is zero for every event)
-        if (two && (FMT == SNN_W_FP32_12B || lo != 0)) atomicAdd(&accL[cell], lo);
+        atomicAdd(&acc_mem[c], hi);
+        if (two && lo != 0) atomicAdd(&acc_mem[cells + c], lo);
       } else {
-        atomicAdd(&accF[cell], w);
+        atomicAdd(reinterpret_cast<float*>(acc_mem) + c, w);
+      }
+      if (COUNT) {
+        const uint32_t sl = c / TW;
+        atomicAdd(v.counts + (size_t)((uint32_t)(base + sl) & v.slot_mask) * v.pitch +
+                      tgt_lo + (c - sl * TW), 1u);
       }
     } else {
-      const uint32_t step = (uint32_t)t + d;
-      red_add_f32(v.rb + (size_t)(step & v.slot_mask) * v.pitch + tgt, w);
-    }
-    if (COUNT)
-      atomicAdd(v.counts + (size_t)(((uint32_t)t + d) & v.slot_mask) * v.pitch + tgt,
-                1u);
-  };
-  // one event of an interval list (in the window, fixed point) by its cell
-  auto add_cell = [&](uint32_t cell, float w) {
-    int hi, lo;
-    fixed_split(w, fx, hi, lo);
-    atomicAdd(&accH[cell], hi);
-    atomicAdd(&accL[cell], lo);
-  };
-
-  // plastic E->E synapse: update its weight (record index r), store it
-  StdpConst sc{};
-  if (PL) {
-    sc.c_pot = v.sp.c_pot;
-    sc.c_dep = v.sp.c_dep;
-    sc.mu = v.sp.mu;
-    sc.w_max = v.sp.w_max;
-    sc.l2_plus = v.sp.l2_plus;
-    sc.l2_minus = v.sp.l2_minus;
-    sc.hmask = v.sp.hist - 1u;
-  }
-  auto plastic = [&](uint32_t tgt, uint32_t k_run, int32_t t, uint32_t d,
-                     float w, uint64_t r) -> float {
-    const uint32_t j = tgt - tgt_lo;
-    const float km = s_km[(uint32_t)((long long)t - (long long)d - h_lo) * TW + j];
-    const StdpOut o = stdp_weight(w, t, d, s_tprev[k_run], s_kprev[k_run], j,
-                                  TW, s_rt, fmaxf(km, 0.f), s_rn[j], sc);
-    v.sp.wp[r] = o.w;
-    ++my_pl;
-    my_trunc += o.trunc | (km < 0.f ? 1u : 0u);
-    return o.w;
-  };
-  const uint32_t sub = lane & (uint32_t)(LG - 1);  // lane within its run
-  const uint32_t grp = lane / (uint32_t)LG;         // run side of the warp
-  auto load_pass = [&](Rec1<FMT> (&r)[UR][PER], float (&wv)[UR][PER], uint32_t k0,
-                       uint32_t nb) {
-#pragma unroll
-    for (int u = 0; u < UR; ++u) {
-      const uint32_t j = k0 + (uint32_t)(G * u) + grp;
-      const bool ok = j < nb;
-      const uint64_t beg = ok ? s_desc[j].beg : 0ull;
-      const uint32_t len = ok ? s_desc[j].len : 0u;
-      const bool pl = PL && tile_plastic && ok && s_kprev[j] >= 0.f;
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        const uint32_t idx = sub + (uint32_t)LG * q;
-        if (idx < len) {
-          if constexpr (CELL)
-            r[u][q] = load_rec_wc(v.recs, beg + idx);
-          else
-            r[u][q] = load_rec<FMT>(v.recs, beg + idx);
-          if (pl) wv[u][q] = __ldcs(v.sp.wp + beg + idx);
-        }
-      }
+      const uint32_t d = cell / TW;
+      const size_t at =
+          (size_t)(((uint32_t)sd.off + d + (uint32_t)v.d_base) & v.slot_mask) * v.pitch +
+          tgt_lo + (cell - d * TW);
+      red_add_f32(v.rb + at, w);
+      if (COUNT) atomicAdd(v.counts + at, 1u);
     }
   };
-  auto add_pass = [&](const Rec1<FMT> (&r)[UR][PER], const float (&wv)[UR][PER],
-                      uint32_t k0, uint32_t nb) {
-#pragma unroll
-    for (int u = 0; u < UR; ++u) {
-      const uint32_t j = k0 + (uint32_t)(G * u) + grp;
-      if (j >= nb) {
-        if constexpr (G == 1) break;  // (uniform across the warp)
-        else continue;
-      }
-      const SegDesc sd = s_desc[j];
-      const int32_t roff = (int32_t)(((long long)sd.t - base) * (long long)TW);
-      const int32_t off = roff - (int32_t)tgt_lo;
-      const bool pl = PL && tile_plastic && s_kprev[j] >= 0.f;
-      if constexpr (CELL) {
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          const uint32_t idx = sub + (uint32_t)LG * q;
-          if (idx < sd.len)
-            add_cell((r[u][q].c >> 8) + (uint32_t)roff, __uint_as_float(r[u][q].b));
-        }
-        for (uint32_t idx = (uint32_t)LG * PER + sub; idx < sd.len; idx += (uint32_t)LG) {
-          const Rec1<FMT> x = load_rec_wc(v.recs, sd.beg + idx);
-          add_cell((x.c >> 8) + (uint32_t)roff, __uint_as_float(x.b));
-        }
-        continue;
-      }
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        const uint32_t idx = sub + (uint32_t)LG * q;
-        if (idx < sd.len) {
-          uint32_t tgt, d;
-          float w;
-          rec_fields(r[u][q], tgt, d, w);
-          if (!rec_in_bounds(v, tgt, d, tgt_lo, TW)) continue;
-          if (pl && tgt < v.sp.n_exc)
-            w = plastic(tgt, j, sd.t, d, wv[u][q], sd.beg + idx);
-          add(tgt, sd.t, off, d, w);
-        }
-      }
-      for (uint32_t idx = (uint32_t)LG * PER + sub; idx < sd.len; idx += (uint32_t)LG) {
-        uint32_t tgt, d;
-        float w;
-        rec_fields(load_rec<FMT>(v.recs, sd.beg + idx), tgt, d, w);
-        if (!rec_in_bounds(v, tgt, d, tgt_lo, TW)) continue;
-        if (pl && tgt < v.sp.n_exc)
-          w = plastic(tgt, j, sd.t, d, __ldcs(v.sp.wp + sd.beg + idx),
-                      sd.beg + idx);
-        add(tgt, sd.t, off, d, w);
-      }
-    }
-  };
-
-  // (A) describe the runs of spikes [j0, j0 + nb): kDU list entries per
-  // thread in flight (the first ones already read), then their tile-index
-  // words and row starts
-  auto describe = [&](uint32_t j0, uint32_t nb) {
-    unsigned long long my_events = 0;
-    for (uint32_t k0 = threadIdx.x; k0 < nb; k0 += kDU * blockDim.x) {
-      SpikeEntry e[kDU];
-      const bool have = spec && j0 == 0 && k0 == threadIdx.x;
-#pragma unroll
-      for (int u = 0; u < kDU; ++u) {
-        const uint32_t k = k0 + u * blockDim.x;
-        if (k < nb) {
-          if constexpr (GX) {
-            const uint32_t g = j0 + k;
-            uint32_t p = 0;
-            while (s_gstart[p + 1] <= g) ++p;
-            const uint2 x = (have && p == 0)
-                ? pre_g[u]
-                : reinterpret_cast<const uint2*>(
-                      v.gx + (uint64_t)p * v.gx_stride + 4)[g - s_gstart[p]];
-            // entries come from the caller's buffers: a source outside the
-            // store or a step outside this interval is skipped and flagged
-            // (its cells would lie outside the tile's window)
-            const bool ok = x.x < v.n_src &&
-                            (uint32_t)((int32_t)x.y - (int32_t)t_now) < iv_span;
-            if (!ok) atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_BAD_SOURCE);
-            e[u].src = ok ? x.x : 0xFFFFFFFFu;
-            e[u].t = (int32_t)x.y;
-            e[u].choff = 0;
-            e[u].pad = 0;
-          } else {
-            e[u] = have ? pre[u] : list[j0 + k];
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kDU; ++u) {
-        const uint32_t k = k0 + u * blockDim.x;
-        if (k < nb) {
-          SegDesc sd{0, 0u, e[u].t};
-          if (e[u].src < v.n_src) {
-            const uint32_t* to = v.tile_off + (uint64_t)e[u].src * row_stride + tile;
-            const uint32_t a = to[0], b = to[1];
-            sd.beg = v.row_ptr[e[u].src] + a;
-            sd.len = b - a;
-            if (kChecked && (b < a || sd.beg + sd.len > v.row_ptr[e[u].src + 1])) {
-              atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_CHECK);
-              sd.len = 0;
-            }
-            if (gathered) my_events += sd.len;
-          }
-          s_desc[k] = sd;
-          if (PL) {
-            const bool exc = e[u].src < v.sp.n_exc;
-            s_tprev[k] = exc ? v.sp.prev_t[e[u].src] : kNoSpike;
-            s_kprev[k] = exc ? v.sp.prev_k[e[u].src] : -1.f;
-          }
-        }
-      }
-    }
-    // gathered lists: the warp's events (all threads of the CTA reach this)
-    if (gathered) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) my_events += __shfl_xor_sync(kFull, my_events, o);
-    }
-    return my_events;
-  };
-  // next U runs for this warp (shared counter: warps that met short runs or
-  // fast loads take more)
-  auto grab = [&]() {
-    uint32_t k = 0u;
-    if (lane == 0) k = atomicAdd(&s_next, (uint32_t)U);
-    return __shfl_sync(kFull, k, 0);
-  };
-
   uint32_t j0 = 0;
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
-    const unsigned long long warp_events = describe(j0, nb);
-    if (threadIdx.x == 0) s_next = 0u;
+    const unsigned long long warp_events = describe_runs<kDU, false, GX>(
+        v, lv, list, tile, j0, nb, spec, pre, pre_g, s_gstart, s_desc, nullptr, nullptr, nullptr);
+    // a batch of few runs spreads them over all lanes of the CTA
+    lg = (uint32_t)v.lg;
+    while (lg < 5u && (nb << (lg + 1u)) <= (uint32_t)kTileThreads) ++lg;
+    n_lanes = 1u << lg;
+    runs = 32u >> lg;
+    sub = lane & (n_lanes - 1u);
+    grp = lane >> lg;
     __syncthreads();
     // (after the barrier: s_events was cleared before it)
-    if (gathered && lane == 0 && warp_events) atomicAdd(&s_events, warp_events);
+    if (GX && lane == 0 && warp_events) atomicAdd(&s_events, warp_events);
     fx = s_fx;
-    if (FAST && !fx.fixed && n_sp > 0 && j0 == 0 && threadIdx.x == 0)
-      atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_SCALES);
-    // (B) each warp takes U runs at a time: all loads first, then the adds
-    // (plastic nets: a fixed share per warp, the registers being spent on
-    // the weight update)
-    if constexpr (PL) {
-      for (uint32_t k = warp * U; k < nb; k += kTileWarps * U) {
-        Rec1<FMT> r[UR][PER];
-        float wv[UR][PER];
-        load_pass(r, wv, k, nb);
-        add_pass(r, wv, k, nb);
-      }
+    const bool fast = !COUNT && !kChecked && lv.inwin &&
+                      (LAY == kLayHom ? fx.packed : fx.fixed);
+    // every warp takes each kTileWarps-th group of `runs` runs
+    const uint32_t stride = kTileWarps * runs;
+    uint32_t k = (threadIdx.x >> 5) * runs;
+    if (fast) {
+      const uint32_t lo_off = two ? 4u * cells : 0u;
+      const char* const dat = reinterpret_cast<const char*>(v.dat);
+      const char* const cel = reinterpret_cast<const char*>(v.cells);
+      const SplitScale sc{fx.scale_hs, fx.scale_s};
+      add_runs<LAY>(dat, cel, s_desc, nb, acc_s, lo_off, lg, sc);
     } else {
-      uint32_t k = grab();
-      while (k < nb) {
-        Rec1<FMT> r[UR][PER];
-        float wv[UR][PER];
-        load_pass(r, wv, k, nb);
-        const uint32_t k_next = grab();
-        add_pass(r, wv, k, nb);
-        k = k_next;
+      for (; k < nb; k += stride) {
+        const uint32_t j = k + grp;
+        if (j < nb) {
+          const SegDesc sd = s_desc[j];
+          const uint32_t head = (uint32_t)(sd.beg & (E - 1u));
+          const uint32_t total = head + (sd.len & 0x7FFFFFFFu);
+          const float w_hom = v.hom_w[(int)sd.len < 0];
+          for (uint32_t jv = sub; jv * E < total; jv += n_lanes) {
+            const Vec<LAY> x = load_vec<LAY>(v, sd.beg / E + jv);
+            const uint32_t m = vec_mask<LAY>(jv, head, total);
+#pragma unroll
+            for (int e = 0; e < (int)E; ++e) {
+              if (!(m & (1u << e))) continue;
+              const uint32_t cell = vec_cell<LAY>(x, e);
+#if SNN_CHECK
+              const uint64_t ti = sd.tgt + jv * E + e - head;
+              const uint32_t tgt = v.tgts ? v.tgts[ti]
+                                          : reinterpret_cast<const uint32_t*>(v.recs)[ti];
+              if (!cell_in_bounds(v, cell, tgt, tgt_lo)) continue;
+#endif
+              float w = w_hom;
+              if constexpr (LAY == kLayI16)
+                w = (float)vec_int<LAY>(x, e) * pow2f(-v.acc_qs_min);
+              else if constexpr (LAY != kLayHom)
+                w = vec_weight<LAY>(x, e);
+              add_slow(cell, sd, w);
+            }
+          }
+        }
       }
     }
     j0 += nb;
     __syncthreads();  // s_desc is rewritten by the next batch
   } while (j0 < n_sp);
-  if (inwin) {
-    // Every cell of the window belongs to this CTA alone, so its sum goes
-    // into the ring buffer as a fire-and-forget global reduction: the one
-    // addition rb + sum that a read-modify-write would make, without a
-    // memory round trip.  The exact sum (H 2^s + L) 2^-q becomes
-    // H 2^(s-q) + L 2^-q in FP32: both products are exact while |H| and |L|
-    // are below 2^24 (then only the addition rounds, so the result is the
-    // correctly rounded sum; larger words round once more), no 64-bit
-    // conversion or FP64 arithmetic, whose rate is low on this part.
-    // (the slots of a column are independent: unrolled, so that their
-    // shared-memory reads and conversions overlap)
-    const uint32_t x_end = tgt_lo < v.n ? min(TW, v.n - tgt_lo) : 0u;
-    for (uint32_t x = threadIdx.x; x < x_end; x += blockDim.x) {
-      float* const col = v.rb + tgt_lo + x;
-#pragma unroll 4
-      for (uint32_t sl = 0; sl < W; ++sl) {
-        const uint32_t c = sl * TW + x;
-        float a;
-        if (fx.fixed) {
-          a = __fmul_rn(__int2float_rn(accH[c]), fx.scale_sq);
-          if (two) a = __fadd_rn(a, __fmul_rn(__int2float_rn(accL[c]), fx.inv_q));
-        } else {
-          a = accF[c];
-        }
-        if (a != 0.f)
-          red_add_f32(col + (size_t)((uint32_t)(base + sl) & v.slot_mask) * v.pitch, a);
-      }
-    }
-  }
-  if (PL) {
-    // one pair of atomics per warp, one per CTA
-    unsigned long long a = my_pl, b = my_trunc;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(kFull, a, o);
-      b += __shfl_xor_sync(kFull, b, o);
-    }
-    if (lane == 0 && (a | b)) {
-      atomicAdd(&s_pl[0], a);
-      atomicAdd(&s_pl[1], b);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && (s_pl[0] | s_pl[1])) {
-      atomicAdd(&v.ctl->plastic_events, s_pl[0]);
-      atomicAdd(&v.ctl->stdp_truncated, s_pl[1]);
-    }
-  }
+  if (lv.inwin) flush_tile<LAY == kLayHom>(v, fx, two, acc_mem, tgt_lo, base);
   // The last CTA to finish clears the list counters and advances the clock
   // (a gathered list's events -- its spikes' runs onto this partition's
   // targets -- are counted by the CTAs themselves).
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (gathered && s_events) atomicAdd(&v.ctl->gx_events, s_events);
-    __threadfence();
-    unsigned prev = atomicAdd(done_p, 1u);
-    if (prev == v.n_tiles - 1) {
-      *pair_p = 0ull;
-      *done_p = 0u;
-      if (advance_time) {  // the interval's own list: commit its events
-        // this net's exchange list has been read (by the collective before
-        // this delivery, or by this delivery itself): the next update
-        // refills it
-        if (v.xbuf) *v.xbuf = 0u;
-        v.ctl->t_now += v.ctl->iv_steps;
-        const unsigned long long own = atomicExch(&v.ctl->pending_events, 0ull);
-        v.ctl->events += gathered ? atomicExch(&v.ctl->gx_events, 0ull) : own;
-      }
-    }
+    if (GX && s_events) atomicAdd(&v.ctl->gx_events, s_events);
+    finish_list(v, pair_p, done_p, advance_time, GX);
   }
 }
 
-template <int FMT, bool COUNT, bool PL, bool FAST, bool ONE, bool SHORT,
-          bool GX>
+// The same for a plastic net's tile (snn_set_stdp): E->E events apply the
+// weight rule to their FP32 weight first.  A warp takes U runs at a time,
+// three records per lane of each loaded before any is added (the rule's
+// registers leave no room for more), in fixed shares: the plastic net's own
+// lists are always inside the window.
+template <int LAY, bool COUNT>
+__device__ __forceinline__ void deliver_tile_plastic(
+    const NetView& v, unsigned long long* pair_p, unsigned int* done_p,
+    const SpikeEntry* __restrict__ list, int advance_time, uint32_t tile,
+    int* acc_mem, uint32_t desc_off, uint32_t desc_cap) {
+  constexpr int U = LAY == kLayF32 ? 1 : 2;
+  constexpr int PER = 3;
+  SegDesc* const s_desc =
+      reinterpret_cast<SegDesc*>(reinterpret_cast<char*>(acc_mem) + desc_off);
+  int32_t* const s_tprev = reinterpret_cast<int32_t*>(s_desc + desc_cap);
+  float* const s_kprev = reinterpret_cast<float*>(s_tprev + desc_cap);
+  // where each run lies in its row (the index of its first plastic weight is
+  // the row's start plus that; BF16 streams count from twice the row's start)
+  uint32_t* const s_at = reinterpret_cast<uint32_t*>(s_kprev + desc_cap);
+  __shared__ unsigned long long s_pl[2];             // plastic updates, truncations
+  __shared__ FixScale s_fx;
+  const uint32_t TW = v.tile_w;
+  const uint32_t W = (uint32_t)v.window;
+  const uint32_t cells = W * TW;
+  const bool two = v.acc_words == 2;
+  const uint32_t acc_len = two ? 2 * cells : cells;
+  const uint32_t tgt_lo = tile * TW;
+  const unsigned lane = threadIdx.x & 31u;
+  const uint32_t warp = threadIdx.x >> 5;
+  SpikeEntry pre[1];
+  if (threadIdx.x < desc_cap && threadIdx.x < v.list_cap) pre[0] = list[threadIdx.x];
+  ListView lv;
+  lv.n_sp = (uint32_t)(*reinterpret_cast<volatile unsigned long long*>(pair_p) >> 32);
+  lv.t_now = v.ctl->t_now;
+  lv.base = lv.t_now + v.d_min;
+  lv.inwin = true;
+  const uint32_t n_sp = lv.n_sp;
+  const long long base = lv.base;
+  if (threadIdx.x == 0) s_fx = fix_scale(v, n_sp, true);
+  for (uint32_t x = threadIdx.x; x < acc_len; x += blockDim.x) acc_mem[x] = 0;
+  // the post-spike times of this tile's targets (rings) and their post
+  // traces at the W horizons (t - d) this interval can ask for
+  int32_t* const s_rt = acc_mem + acc_len;                             // [hist][TW]
+  uint32_t* const s_rn = reinterpret_cast<uint32_t*>(s_rt + v.sp.hist * TW);
+  float* const s_km = reinterpret_cast<float*>(s_rn + TW);             // [W][TW]
+  const bool tile_plastic = tgt_lo < v.sp.n_exc;
+  uint32_t my_pl = 0, my_trunc = 0;
+  // first horizon: (interval start) - d_max
+  const long long h_lo = base - v.d_min - v.d_max;
+  if (threadIdx.x < 2) s_pl[threadIdx.x] = 0ull;
+  if (tile_plastic) {
+    for (uint32_t x = threadIdx.x; x < TW; x += blockDim.x)
+      s_rn[x] = tgt_lo + x < v.n ? v.sp.ring_n[tgt_lo + x] : 0u;
+    for (uint32_t x = threadIdx.x; x < v.sp.hist * TW; x += blockDim.x) {
+      const uint32_t q = x / TW, jj = x - q * TW;
+      if (tgt_lo + jj < v.n)
+        s_rt[x] = v.sp.ring_t[(size_t)q * v.pitch + tgt_lo + jj];
+    }
+    __syncthreads();
+    // post trace of target j at horizon h: the trace right after its
+    // latest spike at or before h, decayed to h (0 if it never fired)
+    const uint32_t hm = v.sp.hist - 1u;
+    for (uint32_t x = threadIdx.x; x < W * TW; x += blockDim.x) {
+      const uint32_t hi = x / TW, jj = x - hi * TW;
+      const int32_t h = (int32_t)(h_lo + hi);
+      const uint32_t n = s_rn[jj];
+      const int32_t k_min = n > v.sp.hist ? (int32_t)(n - v.sp.hist) : 0;
+      float km = 0.f;
+      int32_t k = (int32_t)n - 1;
+      for (; k >= k_min; --k) {
+        const int32_t tp = s_rt[((uint32_t)k & hm) * TW + jj];
+        if (tp <= h) {
+          km = v.sp.ring_k[(size_t)((uint32_t)k & hm) * v.pitch + tgt_lo + jj] *
+               exp2f(-(float)(h - tp) * v.sp.l2_minus);
+          break;
+        }
+      }
+      // every kept spike is after h but older ones were dropped: the
+      // trace at h is unknown (-1; an update that needs it is counted
+      // with the truncated windows)
+      s_km[x] = (k < k_min && n > v.sp.hist) ? -1.f : km;
+    }
+  }
+  FixScale fx{};  // thread 0's s_fx, read after the first barrier
+  StdpConst sc;
+  sc.c_pot = v.sp.c_pot;
+  sc.c_dep = v.sp.c_dep;
+  sc.mu = v.sp.mu;
+  sc.w_max = v.sp.w_max;
+  sc.l2_plus = v.sp.l2_plus;
+  sc.l2_minus = v.sp.l2_minus;
+  sc.hmask = v.sp.hist - 1u;
+  const uint32_t magic = cell_magic(TW);
+
+  // one event of run k_run (spike at step t): the synapse's cell, stored weight,
+  // plastic weight (pl: of a plastic run) and the index of the latter
+  auto event = [&](uint32_t k_run, const SegDesc& sd, int32_t t, bool pl,
+                   uint32_t cell, float w, float wv, uint64_t r) {
+    if (pl) w = wv;  // (static synapses of a plastic run: the stored weight)
+    const uint32_t ds = cell_step(cell, magic), j = cell - ds * TW;
+    if (pl && tgt_lo + j < v.sp.n_exc) {
+      const uint32_t d = ds + (uint32_t)v.d_base;
+      const float km = s_km[(uint32_t)((long long)t - (long long)d - h_lo) * TW + j];
+      const StdpOut o = stdp_weight(w, t, d, s_tprev[k_run], s_kprev[k_run], j,
+                                    TW, s_rt, fmaxf(km, 0.f), s_rn[j], sc);
+      w = o.w;
+      v.sp.wp[r] = w;
+      ++my_pl;
+      my_trunc += o.trunc | (km < 0.f ? 1u : 0u);
+    }
+    const uint32_t c = (uint32_t)sd.off + cell;
+    if (fx.fixed) {
+      int hi, lo;
+      fixed_split(w, fx, hi, lo);
+      atomicAdd(&acc_mem[c], hi);
+      if (two && (LAY == kLayF32 || lo != 0)) atomicAdd(&acc_mem[cells + c], lo);
+    } else {
+      atomicAdd(reinterpret_cast<float*>(acc_mem) + c, w);
+    }
+    if (COUNT) {
+      const uint32_t sl = c / TW;
+      atomicAdd(v.counts + (size_t)((uint32_t)(base + sl) & v.slot_mask) * v.pitch +
+                    tgt_lo + (c - sl * TW), 1u);
+    }
+  };
+  // synapse idx of a run: the stream's word (weight and cell), the index of
+  // its plastic weight
+  struct Syn { uint32_t a, c; };
+  auto load_syn = [&](const SegDesc& sd, uint32_t idx) {
+    Syn x;
+    if constexpr (LAY == kLayF32) {
+      x.a = __ldcs(reinterpret_cast<const uint32_t*>(v.dat) + sd.beg + idx);
+      x.c = __ldcs(v.cells + sd.beg + idx);
+    } else {
+      // (taken apart only when it is added: no use before the other loads)
+      x.a = __ldcs(reinterpret_cast<const uint32_t*>(v.dat) + sd.beg + idx);
+      x.c = 0;
+    }
+    return x;
+  };
+  auto syn_cell = [&](const Syn& x) { return LAY == kLayF32 ? x.c : x.a & 0xFFFFu; };
+  auto syn_w = [&](const Syn& x) {
+    return __uint_as_float(LAY == kLayF32 ? x.a : x.a & 0xFFFF0000u);
+  };
+  auto check = [&](const SegDesc& sd, uint32_t idx, uint32_t cell) {
+#if SNN_CHECK
+    const uint64_t ti = sd.tgt + idx;
+    return cell_in_bounds(v, cell, v.tgts ? v.tgts[ti]
+                                          : reinterpret_cast<const uint32_t*>(v.recs)[ti],
+                          tgt_lo);
+#else
+    return true;
+#endif
+  };
+
+  uint32_t j0 = 0;
+  do {
+    const uint32_t nb = min(desc_cap, n_sp - j0);
+    describe_runs<1, true, false>(v, lv, list, tile, j0, nb, true, pre, nullptr,
+                                  nullptr, s_desc, s_tprev, s_kprev, s_at);
+    __syncthreads();
+    fx = s_fx;
+    for (uint32_t k0 = warp * U; k0 < nb; k0 += kTileWarps * U) {
+      Syn r[U][PER];
+      float wv[U][PER];
+      uint64_t wi[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t j = k0 + (uint32_t)u;
+        const bool ok = j < nb;
+        const SegDesc sd = ok ? s_desc[j] : SegDesc{};
+        const bool pl = tile_plastic && ok && s_kprev[j] >= 0.f;
+        wi[u] = !ok ? 0ull : LAY == kLayF32 ? sd.beg : (sd.beg + s_at[j]) >> 1;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          const uint32_t idx = lane + 32u * q;
+          if (idx < sd.len) {
+            r[u][q] = load_syn(sd, idx);
+            if (pl) wv[u][q] = __ldcs(v.sp.wp + wi[u] + idx);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t j = k0 + (uint32_t)u;
+        if (j >= nb) break;  // (uniform across the warp)
+        const SegDesc sd = s_desc[j];
+        const bool pl = tile_plastic && s_kprev[j] >= 0.f;
+        const int32_t t = (int32_t)(base - v.d_base) + sd.off / (int32_t)TW;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          const uint32_t idx = lane + 32u * q;
+          if (idx < sd.len && check(sd, idx, syn_cell(r[u][q])))
+            event(j, sd, t, pl, syn_cell(r[u][q]), syn_w(r[u][q]), wv[u][q],
+                  wi[u] + idx);
+        }
+        for (uint32_t idx = 32u * PER + lane; idx < sd.len; idx += 32u) {
+          const Syn x = load_syn(sd, idx);
+          const float w = pl ? __ldcs(v.sp.wp + wi[u] + idx) : 0.f;
+          if (check(sd, idx, syn_cell(x)))
+            event(j, sd, t, pl, syn_cell(x), syn_w(x), w, wi[u] + idx);
+        }
+      }
+    }
+    j0 += nb;
+    __syncthreads();  // s_desc is rewritten by the next batch
+  } while (j0 < n_sp);
+  flush_tile<false>(v, fx, two, acc_mem, tgt_lo, base);
+  // one pair of atomics per warp, one per CTA
+  unsigned long long a = my_pl, b = my_trunc;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(kFull, a, o);
+    b += __shfl_xor_sync(kFull, b, o);
+  }
+  if (lane == 0 && (a | b)) {
+    atomicAdd(&s_pl[0], a);
+    atomicAdd(&s_pl[1], b);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_pl[0] | s_pl[1]) {
+      atomicAdd(&v.ctl->plastic_events, s_pl[0]);
+      atomicAdd(&v.ctl->stdp_truncated, s_pl[1]);
+    }
+    finish_list(v, pair_p, done_p, advance_time, false);
+  }
+}
+
+template <int LAY, bool COUNT, bool GX>
 __global__ void __launch_bounds__(kTileThreads, 1)
 k_deliver_tiled(NetView v, unsigned long long* pair_p, unsigned int* done_p,
                 const SpikeEntry* __restrict__ list, int from_list_range,
                 int advance_time, uint32_t desc_off, uint32_t desc_cap) {
   extern __shared__ __align__(16) int acc_mem[];
-  if constexpr (PL) {
-    // one tile of plastic targets, or up to tile_grp static tiles one
-    // after another in the same shared memory
-    uint32_t t0 = blockIdx.x, t1 = blockIdx.x + 1u;
-    if (blockIdx.x >= v.pl_tiles) {
-      t0 = v.pl_tiles + (blockIdx.x - v.pl_tiles) * v.tile_grp;
-      t1 = min(t0 + v.tile_grp, v.n_tiles);
-    }
-    for (uint32_t t = t0; t < t1; ++t) {
-      if (t > t0) __syncthreads();  // the previous tile's last reads
-      deliver_tile_body<FMT, COUNT, PL, FAST, ONE, SHORT, GX>(
-          v, pair_p, done_p, list, from_list_range, advance_time, t, acc_mem,
-          desc_off, desc_cap);
-    }
-  } else {
-    deliver_tile_body<FMT, COUNT, PL, FAST, ONE, SHORT, GX>(
-        v, pair_p, done_p, list, from_list_range, advance_time, blockIdx.x,
-        acc_mem, desc_off, desc_cap);
-  }
+  deliver_tile_body<LAY, COUNT, GX>(v, pair_p, done_p, list,
+                                         from_list_range, advance_time,
+                                         blockIdx.x, acc_mem, desc_off, desc_cap);
   // the next update may be scheduled once every CTA got here
   asm volatile("griddepcontrol.launch_dependents;");
 }
 
+// Plastic nets: one tile of plastic targets, or up to tile_grp static tiles
+// one after another in the same shared memory.
+template <int LAY, bool COUNT>
+__global__ void __launch_bounds__(kTileThreads, 1)
+k_deliver_plastic(NetView v, unsigned long long* pair_p, unsigned int* done_p,
+                  const SpikeEntry* __restrict__ list, int advance_time,
+                  uint32_t desc_off, uint32_t desc_cap) {
+  extern __shared__ __align__(16) int acc_mem[];
+  uint32_t t0 = blockIdx.x, t1 = blockIdx.x + 1u;
+  if (blockIdx.x >= v.pl_tiles) {
+    t0 = v.pl_tiles + (blockIdx.x - v.pl_tiles) * v.tile_grp;
+    t1 = min(t0 + v.tile_grp, v.n_tiles);
+  }
+  for (uint32_t t = t0; t < t1; ++t) {
+    if (t > t0) __syncthreads();  // the previous tile's last reads
+    deliver_tile_plastic<LAY, COUNT>(v, pair_p, done_p, list, advance_time, t,
+                                     acc_mem, desc_off, desc_cap);
+  }
+  asm volatile("griddepcontrol.launch_dependents;");
+}
+
+// A served net's tile, its pending interval list (advancing the net's clock).
+template <int FMT>
+__device__ __forceinline__ void serve_tile(const NetView& v, uint32_t tile,
+                                           int* acc_mem, uint32_t desc_off,
+                                           uint32_t desc_cap) {
+  if (v.lay == kLayHom)
+    deliver_tile_body<kLayHom, false, false>(
+        v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
+  else if (FMT == SNN_W_BF16_8B && v.lay == kLayI16)
+    deliver_tile_body<kLayI16, false, false>(
+        v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
+  else
+    deliver_tile_body<FMT == SNN_W_FP32_12B ? kLayF32 : kLayJ16, false, false>(
+        v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
+}
+
 // All nets of a batch in one launch: CTA b delivers tile bmap[b].y of net
-// bmap[b].x (its pending interval list, advancing that net's clock).
+// bmap[b].x.
 template <int FMT>
 __global__ void __launch_bounds__(kTileThreads, 1)
 k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
@@ -1326,8 +1685,7 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
   extern __shared__ __align__(16) int acc_mem[];
   const uint2 m = bmap[blockIdx.x];
   const NetView v = nets[m.x].v;
-  deliver_tile_body<FMT, false, false>(v, &v.ctl->pair, &v.ctl->done, v.list,
-                                       0, 1, m.y, acc_mem, desc_off, desc_cap);
+  serve_tile<FMT>(v, m.y, acc_mem, desc_off, desc_cap);
 }
 
 // ---------------------------------------------------------------------------
@@ -1365,8 +1723,7 @@ template <int FMT>
 __device__ __noinline__ void serve_deliver(const NetView& v, uint32_t tile,
                                            int* acc_mem, uint32_t desc_off,
                                            uint32_t desc_cap) {
-  deliver_tile_body<FMT, false, false>(v, &v.ctl->pair, &v.ctl->done, v.list, 0,
-                                       1, tile, acc_mem, desc_off, desc_cap);
+  serve_tile<FMT>(v, tile, acc_mem, desc_off, desc_cap);
 }
 
 template <int FMT>
@@ -1686,113 +2043,86 @@ struct DescLayout {
 };
 cudaError_t desc_layout(size_t used, size_t dyn_max, bool plastic,
                         DescLayout* out) {
-  const size_t per = sizeof(SegDesc) + (plastic ? 8u : 0u);
+  // (a plastic run also has its source's last spike and its place in the row;
+  // what is added keeps the 196 KB carve-out of the benchmark network's tile)
+  const size_t per = sizeof(SegDesc) + (plastic ? 12u : 0u);
+  const size_t room = plastic ? kDescBytes + 5 * 1024 : kDescBytes;
   const size_t off = (used + 15u) & ~(size_t)15u;
   if (dyn_max < off + 32u * per) return cudaErrorInvalidConfiguration;
-  const size_t cap = std::min(kDescBytes, dyn_max - off) / per;
+  const size_t cap = std::min(room, dyn_max - off) / per & ~(size_t)1;
   out->off = (uint32_t)off;
   out->cap = (uint32_t)cap;
   out->smem = off + cap * per;
   return cudaSuccess;
 }
 
-template <int FMT, bool COUNT, bool PL, bool FAST = false, bool ONE = false,
-          bool SHORT = false, bool GX = false>
+template <int LAY, bool COUNT, bool GX>
 cudaError_t launch_tiled_t(const NetView& v, unsigned long long* pair,
                            unsigned int* done, const SpikeEntry* list,
                            int from_list_range, int advance_time,
                            cudaStream_t s) {
   static std::atomic<uint32_t> lim[64];
   size_t dm = 0;
-  cudaError_t e = allow_tile_smem(
-      k_deliver_tiled<FMT, COUNT, PL, FAST, ONE, SHORT, GX>, lim, &dm);
+  cudaError_t e = allow_tile_smem(k_deliver_tiled<LAY, COUNT, GX>, lim, &dm);
   if (e != cudaSuccess) return e;
   DescLayout dl;
-  e = desc_layout(tiled_smem_bytes(v), dm, PL, &dl);
+  e = desc_layout(tiled_smem_bytes(v), dm, false, &dl);
   if (e != cudaSuccess) return e;
-  // plastic nets: a CTA per plastic tile, then one per tile_grp static ones
-  const uint32_t ctas =
-      PL ? v.pl_tiles + (v.n_tiles - v.pl_tiles + v.tile_grp - 1u) / v.tile_grp
-         : v.n_tiles;
-  k_deliver_tiled<FMT, COUNT, PL, FAST, ONE, SHORT, GX>
-      <<<ctas, kTileThreads, dl.smem, s>>>(
+  k_deliver_tiled<LAY, COUNT, GX><<<v.n_tiles, kTileThreads, dl.smem, s>>>(
       v, pair, done, list, from_list_range, advance_time, dl.off, dl.cap);
   return cudaGetLastError();
 }
 
-template <bool GX>
-cudaError_t launch_deliver_tiled_gx(const NetView& v, unsigned long long* pair,
-                                    unsigned int* done, const SpikeEntry* list,
-                                    int from_list_range, int advance_time,
-                                    cudaStream_t s) {
-#define SNN_TILED(F, C, P)                                                   \
-  launch_tiled_t<F, C, P, false, false, false, GX>(v, pair, done, list,     \
-                                                   from_list_range,         \
-                                                   advance_time, s)
-  // an interval's own list: the scales exist for every spike count when
-  // they exist for the largest (E = max in-degree x spikes per neuron)
-  bool interval_exact = false;
-  if (!from_list_range && !v.counts) {
-    const int qs = fixed_qs_host(
-        (uint64_t)v.k_in_max * (v.spikes_per_iv ? v.spikes_per_iv : 1u), v.max_abs_w);
-    interval_exact = qs >= 0 && (v.acc_words == 2 || qs >= v.acc_qs_min);
-  }
-  if constexpr (GX) {  // gathered lists: static nets only
-    if (v.plastic) return cudaErrorNotSupported;
-  } else if (v.plastic) {
-    if (interval_exact)
-      return v.fmt == SNN_W_FP32_12B
-                 ? launch_tiled_t<SNN_W_FP32_12B, false, true, true>(
-                       v, pair, done, list, 0, advance_time, s)
-                 : launch_tiled_t<SNN_W_BF16_8B, false, true, true>(
-                       v, pair, done, list, 0, advance_time, s);
-    if (v.fmt == SNN_W_FP32_12B)
-      return v.counts ? SNN_TILED(SNN_W_FP32_12B, true, true)
-                      : SNN_TILED(SNN_W_FP32_12B, false, true);
-    return v.counts ? SNN_TILED(SNN_W_BF16_8B, true, true)
-                    : SNN_TILED(SNN_W_BF16_8B, false, true);
-  }
-  {
-    if (interval_exact) {
-      if (v.fmt == SNN_W_FP32_12B) {
-        // (the records' precomputed cells exist for tiles below 2^16
-        // targets; wider tiles take the general form below)
-        if (v.tile_w < (1u << 16))
-          return launch_tiled_t<SNN_W_FP32_12B, false, false, true, false,
-                                false, GX>(v, pair, done, list, 0, advance_time, s);
-      } else if (v.acc_words == 1) {
-        // runs of a few dozen records: half a warp per run, eight per pass
-        return v.mean_run < 48.f
-                   ? launch_tiled_t<SNN_W_BF16_8B, false, false, true, true,
-                                    true, GX>(v, pair, done, list, 0,
-                                              advance_time, s)
-                   : launch_tiled_t<SNN_W_BF16_8B, false, false, true, true,
-                                    false, GX>(v, pair, done, list, 0,
-                                               advance_time, s);
-      } else {
-        return launch_tiled_t<SNN_W_BF16_8B, false, false, true, false, false,
-                              GX>(v, pair, done, list, 0, advance_time, s);
-      }
-    }
-  }
-  if (v.fmt == SNN_W_FP32_12B)
-    return v.counts ? SNN_TILED(SNN_W_FP32_12B, true, false)
-                    : SNN_TILED(SNN_W_FP32_12B, false, false);
-  return v.counts ? SNN_TILED(SNN_W_BF16_8B, true, false)
-                  : SNN_TILED(SNN_W_BF16_8B, false, false);
-#undef SNN_TILED
+template <int LAY, bool COUNT>
+cudaError_t launch_plastic_t(const NetView& v, unsigned long long* pair,
+                             unsigned int* done, const SpikeEntry* list,
+                             int advance_time, cudaStream_t s) {
+  static std::atomic<uint32_t> lim[64];
+  size_t dm = 0;
+  cudaError_t e = allow_tile_smem(k_deliver_plastic<LAY, COUNT>, lim, &dm);
+  if (e != cudaSuccess) return e;
+  DescLayout dl;
+  e = desc_layout(tiled_smem_bytes(v), dm, true, &dl);
+  if (e != cudaSuccess) return e;
+  // a CTA per plastic tile, then one per tile_grp static ones
+  const uint32_t ctas =
+      v.pl_tiles + (v.n_tiles - v.pl_tiles + v.tile_grp - 1u) / v.tile_grp;
+  k_deliver_plastic<LAY, COUNT><<<ctas, kTileThreads, dl.smem, s>>>(
+      v, pair, done, list, advance_time, dl.off, dl.cap);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
                                  unsigned int* done, const SpikeEntry* list,
                                  int from_list_range, int advance_time,
                                  cudaStream_t s) {
-  if (v.gx) {
-    if (from_list_range) return cudaErrorInvalidValue;
-    return launch_deliver_tiled_gx<true>(v, pair, done, list, 0, advance_time, s);
+  if (v.gx && from_list_range) return cudaErrorInvalidValue;
+  if (v.plastic) {
+    if (v.gx || from_list_range) return cudaErrorNotSupported;
+    if (v.lay == kLayF32)
+      return v.counts ? launch_plastic_t<kLayF32, true>(v, pair, done, list, advance_time, s)
+                      : launch_plastic_t<kLayF32, false>(v, pair, done, list, advance_time, s);
+    return v.counts ? launch_plastic_t<kLayJ16, true>(v, pair, done, list, advance_time, s)
+                    : launch_plastic_t<kLayJ16, false>(v, pair, done, list, advance_time, s);
   }
-  return launch_deliver_tiled_gx<false>(v, pair, done, list, from_list_range,
-                                        advance_time, s);
+#define SNN_TILED(L)                                                          \
+  (v.counts ? (v.gx ? launch_tiled_t<L, true, true>(                          \
+                          v, pair, done, list, 0, advance_time, s)            \
+                    : launch_tiled_t<L, true, false>(                         \
+                          v, pair, done, list, from_list_range,               \
+                          advance_time, s))                                   \
+            : (v.gx ? launch_tiled_t<L, false, true>(                         \
+                          v, pair, done, list, 0, advance_time, s)            \
+                    : launch_tiled_t<L, false, false>(                        \
+                          v, pair, done, list, from_list_range,               \
+                          advance_time, s)))
+  switch (v.lay) {
+    case kLayHom: return SNN_TILED(kLayHom);
+    case kLayF32: return SNN_TILED(kLayF32);
+    case kLayI16: return SNN_TILED(kLayI16);
+    default: return SNN_TILED(kLayJ16);
+  }
+#undef SNN_TILED
 }
 
 cudaError_t launch_fill_i32(int32_t* p, int32_t value, uint64_t n,
@@ -1936,6 +2266,8 @@ cudaError_t launch_deliver_noalloc(const NetView& v, const uint32_t* src,
   if (e != cudaSuccess) return e;
   e = launch_prepare_external(v, src, t, n, sc->list, &sc->pair, s);
   if (e != cudaSuccess) return e;
-  return launch_deliver(v, &sc->pair, &sc->done, sc->list, 0, s);
+  return v.lay != kLayRecords
+             ? launch_deliver_tiled(v, &sc->pair, &sc->done, sc->list, 1, 0, s)
+             : launch_deliver(v, &sc->pair, &sc->done, sc->list, 0, s);
 }
 }  // namespace snn

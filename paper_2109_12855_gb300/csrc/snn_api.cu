@@ -59,6 +59,7 @@ int fail(int code, const char* fmt, ...) {
   } while (0)
 
 constexpr int kGraphIntervals = 8;
+constexpr int kSimIntervals = 256;  // intervals of one k_simulate launch at most
 constexpr size_t kTileSmemBudget = 200 * 1024;  // accumulator bytes per CTA
 
 // ---------------------------------------------------------------------------
@@ -1131,6 +1132,7 @@ int snn_finalize(snn_net* net) {
   // a partition also takes the gathered list of the whole population
   net->list_cap = (uint64_t)net->n_src * iv;
   CK(dalloc(&net->list, net->list_cap * sizeof(SpikeEntry), net->stream));
+  CK(dalloc(&net->sim_flags, kSimFlagBytes, net->stream));
   if (net->stdp_on) {
     int rc2;
     if ((rc2 = setup_stdp(net)) != SNN_OK) return rc2;
@@ -1533,8 +1535,28 @@ int snn_simulate(snn_net* net, int64_t n_steps) {
     CK(cudaStreamSynchronize(s));
     if ((rc = add_times(n_iv)) != SNN_OK) return rc;
   } else {
-    if ((rc = simulate_async(net, n_steps, true)) != SNN_OK) return rc;
-    return SNN_OK;
+    SimShared sh{};
+    sh.flags = net->sim_flags;
+    sh.stop = reinterpret_cast<unsigned int*>(net->sim_flags + 2 * 256);
+    for (uint32_t r = 0; r < 10; ++r) {
+      sh.key[2 * r] = (uint32_t)net->uc.seed + r * 0x9E3779B9u;
+      sh.key[2 * r + 1] = (uint32_t)(net->uc.seed >> 32) + r * 0xBB67AE85u;
+    }
+    uint32_t ctas = 0;
+    const NetView v = net->view();
+    if (full + (rem ? 1 : 0) < 2 || !simulate_fits(v, net->uc, D, &sh, &ctas))
+      return simulate_async(net, n_steps, true);
+    // launches of at most kSimIntervals intervals, so that other streams'
+    // work is not held off for long
+    int64_t left = full + (rem ? 1 : 0);
+    while (left > 0) {
+      const int m = (int)std::min<int64_t>(left, kSimIntervals);
+      left -= m;
+      CK(launch_simulate(v, net->uc, sh, ctas, m, D, left == 0 && rem ? rem : D, s));
+      net->launches += 1;
+      net->upd_launches += m;  // (intervals updated and delivered)
+      net->del_launches += m;
+    }
   }
   net->t_host += n_steps;
   return SNN_OK;
@@ -2100,7 +2122,8 @@ int snn_destroy(snn_net* net) {
   void* bufs[] = {net->V,        net->I,        net->J,       net->refr,
                   net->rb,       net->counts,   net->ctl,     net->row_ptr,
                   net->recs,     net->list,     net->ext_list, net->ext_src,
-                  net->ext_t,    net->log_src,  net->log_t,   net->tile_off};
+                  net->ext_t,    net->log_src,  net->log_t,   net->tile_off,
+                  net->sim_flags};
   for (void* b : bufs) dfree(b, net->stream);
   void* ibufs[] = {net->isi_last, net->isi_spikes, net->isi_n, net->isi_sum,
                    net->isi_sq};

@@ -283,6 +283,7 @@ struct NetView {
   uint32_t row_mul;
   int d_base;
   int lg;                   // log2 of the lanes that share a run
+  float mean_row;           // synapses per source
   uint32_t hom_split;
   float hom_w[2];
   const uint32_t* tile_off; // [n][n_tiles + 1] row-relative tile starts
@@ -336,6 +337,19 @@ struct BatchNet {
   UpdConst c;
   int n_steps;   // steps of this net's next interval
   int pad_;
+};
+
+// What the CTAs of one k_simulate launch share: two sets of a flag word per
+// CTA ({interval, spikes}; zeroed before the launch together with `stop`,
+// which a CTA sets when a wait runs out), and of list regions (an entry:
+// source | step in its interval << 24).
+constexpr size_t kSimFlagBytes = 2 * 256 * 8 + 16;
+struct SimShared {
+  unsigned long long* flags;  // [2][256]
+  unsigned int* stop;
+  uint32_t* list;             // [2][CTAs][region]
+  uint32_t region;
+  uint32_t key[20];           // the drive's Philox round keys
 };
 
 // Progress of one net in one launch of the persistent serving kernel
@@ -396,6 +410,14 @@ cudaError_t launch_update_batch(const BatchNet* nets, const uint2* bmap,
 cudaError_t launch_deliver_tiled_batch(int fmt, const BatchNet* nets,
                                        const uint2* bmap, uint32_t n_ctas,
                                        size_t smem, cudaStream_t s);
+// Several intervals in one cooperative launch (see k_simulate): whether the
+// net's can (filling sh's list and the grid), and the launch of n_iv
+// intervals, the last of last_steps steps, from the device clock.
+bool simulate_fits(const NetView& v, const UpdConst& c, int interval,
+                   SimShared* sh, uint32_t* ctas);
+cudaError_t launch_simulate(const NetView& v, const UpdConst& c,
+                            const SimShared& sh, uint32_t ctas, int n_iv,
+                            int steps, int last_steps, cudaStream_t s);
 uint32_t update_threads();
 // Threads of a persistent serving CTA (= neurons of one update item).
 uint32_t serve_threads();

@@ -137,6 +137,25 @@ __device__ __forceinline__ void prefetch_row_l2(const NetView& v, uint32_t src) 
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// One step of a neuron: exact integration, this step's input (ring buffer and
+// drive), threshold.  Returns whether it fired.
+__device__ __forceinline__ bool update_step(const UpdConst& c, float& V, float& I,
+                                            float& J, int& refr, float in) {
+  // (1) membrane, unless refractory
+  if (refr == 0) V = c.p31 * J + c.p32 * I + c.p33 * V;
+  else refr -= 1;
+  // (2) synaptic current and its derivative
+  I = c.p21 * J + c.p22 * I;
+  J = c.p11 * J;
+  // (3) input
+  J += c.psc * in;
+  // (4) threshold
+  if (!(V >= c.v_th)) return false;
+  V = c.v_reset;
+  refr = c.refr_steps;
+  return true;
+}
+
 // Body of the update for neuron block `block` of net v (one thread per
 // neuron); shared by the single-net and the batched kernels.
 // PL: the single-net update, which also keeps the plasticity state and the
@@ -257,22 +276,10 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
       for (int q = 0; q < kPrefetch; ++q) {
         if (!live || sb + q >= ns) continue;
         const long long t = t0 + s0 + sb + q;
-        // (1) membrane, unless refractory
-        if (refr == 0) V = c.p31 * J + c.p32 * I + c.p33 * V;
-        else refr -= 1;
-        // (2) synaptic current and its derivative
-        I = c.p21 * J + c.p22 * I;
-        J = c.p11 * J;
-        // (3) this step's ring-buffer input (read above; the slot is
-        // cleared here) plus drive
+        // this step's ring-buffer input (read above; the slot is cleared
+        // here) plus drive
         rb_i[((uint32_t)t & v.slot_mask) * v.pitch] = 0.0f;
-        J += c.psc * buf[q];
-        // (4) threshold
-        if (V >= c.v_th) {
-          V = c.v_reset;
-          refr = c.refr_steps;
-          mask |= 1u << (sb + q);
-        }
+        if (update_step(c, V, I, J, refr, buf[q])) mask |= 1u << (sb + q);
       }
     }
     // warp compaction of this chunk's spikes: a warp with spikes scans its
@@ -704,9 +711,12 @@ __device__ __forceinline__ uint32_t cell_addr(uint32_t w, uint32_t base) {
   return __dp2a_lo(w, HALF ? 0x0400u : 0x0004u, base);
 }
 
-// Per-spike run for this CTA's tile: its first element in the store's stream,
-// its length (top bit: uniform weight class), and the offset of its cells in
-// the accumulator, (t - base + d_base) TW (a list outside the window: t).
+// Per-spike run for this CTA's tile, in elements of the store's stream (dat):
+// the address of its first vector with the elements to skip there in the low
+// bits, its end in elements from that vector on (top bit: uniform weight
+// class), and the offset of its cells in the accumulator,
+// (t - base + d_base) TW (a list outside the window: t).  Plastic tiles read
+// element by element: the index of the first one, and the length.
 struct SegDesc {
   uint64_t beg;
   uint32_t len;
@@ -887,6 +897,17 @@ __device__ __noinline__ StdpOut stdp_weight(float w, int32_t t, uint32_t d,
   return o;
 }
 
+// Places the run of elements [first, first + len) of v's stream in a
+// descriptor.
+template <int LAY>
+__device__ __forceinline__ void place_run(const NetView& v, uint64_t first,
+                                          uint32_t len, SegDesc* sd) {
+  constexpr uint32_t E = Lay<LAY>::kElems;
+  const uint32_t head = (uint32_t)first & (E - 1u);
+  sd->beg = (reinterpret_cast<uint64_t>(v.dat) + (first / E) * 16u) | head;
+  sd->len = len ? head + len : 0u;
+}
+
 // The launch's list as a delivery sees it: its length, the window's base
 // step, whether its steps lie inside the window, and the clock.
 struct ListView {
@@ -900,7 +921,7 @@ struct ListView {
 // starts.  pre (pre_g): entries threadIdx.x + u blockDim.x of the list, read
 // ahead of its length (have_pre).  Returns the events described (gathered
 // lists).  PL: also the presynaptic history the plastic rule needs.
-template <int DU, bool PL, bool GX>
+template <int LAY, int DU, bool PL, bool GX>
 __device__ __forceinline__ unsigned long long describe_runs(
     const NetView& v, const ListView& lv, const SpikeEntry* list, uint32_t tile,
     uint32_t j0, uint32_t nb, bool have_pre, const SpikeEntry* pre,
@@ -954,20 +975,25 @@ __device__ __forceinline__ unsigned long long describe_runs(
         const uint32_t* to = v.tile_off + (uint64_t)src[u] * row_stride + tile;
         const uint32_t a = to[0], b = to[1];
         const uint64_t row = v.row_ptr[src[u]];
-        sd.beg = row * v.row_mul + a;
-        sd.len = b - a;
+        uint32_t len = b - a;
 #if SNN_CHECK
         const uint64_t row_end = v.row_ptr[src[u] + 1];
         sd.tgt = v.fmt == SNN_W_FP32_12B ? row + a
                                          : 2 * row + (row_end - row) + a;
         if (b < a || row + b > row_end) {
           atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_CHECK);
-          sd.len = 0;
+          len = 0;
         }
 #endif
-        if (GX) my_events += sd.len;
-        if (v.lay == kLayHom && src[u] >= v.hom_split) sd.len |= 0x80000000u;
-        if constexpr (PL) s_at[k] = a;
+        if (GX) my_events += len;
+        if constexpr (PL) {
+          sd.beg = row * v.row_mul + a;
+          sd.len = len;
+          s_at[k] = a;
+        } else {
+          place_run<LAY>(v, row * v.row_mul + a, len, &sd);
+          if (LAY == kLayHom && src[u] >= v.hom_split) sd.len |= 0x80000000u;
+        }
       }
       s_desc[k] = sd;
       if constexpr (PL) {
@@ -1108,11 +1134,8 @@ __device__ __forceinline__ void add_elem(const Vec<LAY>& x, uint32_t row_s,
     fixed_split(vec_weight<LAY>(x, K), fx, hi, low);
     red_shared_u32_at<K, CLIP>(addr, (uint32_t)hi, n, lo, none);
     // (one-word cells have no low part)
-    if constexpr (LAY == kLayF32)
-      red_shared_u32_at<K, CLIP>(addr + lo_off, (uint32_t)low, n, lo, none);
-    else
-      red_shared_u32_at<K, CLIP>(addr + lo_off, (uint32_t)low,
-                                 lo_off ? n : 0, lo, none);
+    red_shared_u32_at<K, CLIP>(LAY == kLayF32 || lo_off ? addr + lo_off : none,
+                               (uint32_t)low, n, lo, none);
   }
 }
 template <int LAY, bool CLIP>
@@ -1137,7 +1160,7 @@ __device__ __forceinline__ void add_vec(const Vec<LAY>& x, uint32_t row_s,
 // run), the run's cells in the accumulator and its increment.
 template <int LAY> struct LaneRun {
   Vec<LAY> x[kAhead];
-  const char* p;   // the lane's first vector (cells: FP32 layouts)
+  const char* p;   // the lane's first vector
   int n, lo;
   uint32_t row_s, inc;
 };
@@ -1145,6 +1168,9 @@ template <int LAY> struct LaneRun {
 // Phase (B) for a batch of nb described runs, 2^lg lanes a run: every warp
 // takes each kTileWarps-th group of 32 / 2^lg runs, and loads a lane's first
 // kAhead vectors of the next group before it adds the current one.
+// (Measured and not kept: masks only on a run's first and last vector, held
+// apart from the whole ones -- a fifth fewer instructions, but more registers
+// and branches: 29.8 -> 34.9 us on the 112,500-neuron list.)
 template <int LAY>
 __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
                                       const SegDesc* s_desc, uint32_t nb,
@@ -1171,10 +1197,9 @@ __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
     r.n = 0;
     if (j < nb) {
       const SegDesc sd = s_desc[j];
-      const uint32_t head = (uint32_t)sd.beg & (E - 1u);
-      r.p = dat + (sd.beg / E + sub) * 16u;
-      r.lo = sub == 0 ? (int)head : 0;
-      r.n = (int)(head + (sd.len & 0x7FFFFFFFu)) - (int)(sub * E);
+      r.p = reinterpret_cast<const char*>((sd.beg & ~15ull) + sub * 16u);
+      r.lo = sub == 0 ? (int)((uint32_t)sd.beg & 15u) : 0;
+      r.n = (int)(sd.len & 0x7FFFFFFFu) - (int)(sub * E);
       r.row_s = acc_s + 4u * (uint32_t)sd.off;
       r.inc = (int)sd.len < 0 ? 0x10000u : 1u;
 #pragma unroll
@@ -1191,8 +1216,7 @@ __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
                             none, fx);
     for (int q = kAhead; r.n > q * kStep; ++q) {
       const Vec<LAY> x = fetch(r, q);
-      add_vec<LAY, false>(x, r.row_s, r.inc, r.n - q * kStep, 0, lo_off,
-                            none, fx);
+      add_vec<LAY, false>(x, r.row_s, r.inc, r.n - q * kStep, 0, lo_off, none, fx);
     }
   };
   uint32_t k = (threadIdx.x >> 5) * R;
@@ -1205,6 +1229,16 @@ __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
     load(a, k + 2 * stride + grp);
     add(b);
   }
+}
+
+// The same out of line, for a kernel whose own registers it would not fit
+// beside.
+template <int LAY>
+__device__ __noinline__ void add_runs_call(const char* dat, const char* cel,
+                                           const SegDesc* s_desc, uint32_t nb,
+                                           uint32_t acc_s, uint32_t lo_off,
+                                           uint32_t lg, SplitScale fx) {
+  add_runs<LAY>(dat, cel, s_desc, nb, acc_s, lo_off, lg, fx);
 }
 
 // One interval's (or one caller's) list for tile `tile`.
@@ -1326,7 +1360,7 @@ __device__ __forceinline__ void deliver_tile_body(
   uint32_t j0 = 0;
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
-    const unsigned long long warp_events = describe_runs<kDU, false, GX>(
+    const unsigned long long warp_events = describe_runs<LAY, kDU, false, GX>(
         v, lv, list, tile, j0, nb, spec, pre, pre_g, s_gstart, s_desc, nullptr, nullptr, nullptr);
     // a batch of few runs spreads them over all lanes of the CTA
     lg = (uint32_t)v.lg;
@@ -1355,11 +1389,12 @@ __device__ __forceinline__ void deliver_tile_body(
         const uint32_t j = k + grp;
         if (j < nb) {
           const SegDesc sd = s_desc[j];
-          const uint32_t head = (uint32_t)(sd.beg & (E - 1u));
-          const uint32_t total = head + (sd.len & 0x7FFFFFFFu);
+          const uint32_t head = (uint32_t)sd.beg & 15u;
+          const uint32_t total = sd.len & 0x7FFFFFFFu;
+          const uint64_t v0 = ((sd.beg & ~15ull) - reinterpret_cast<uint64_t>(v.dat)) / 16u;
           const float w_hom = v.hom_w[(int)sd.len < 0];
           for (uint32_t jv = sub; jv * E < total; jv += n_lanes) {
-            const Vec<LAY> x = load_vec<LAY>(v, sd.beg / E + jv);
+            const Vec<LAY> x = load_vec<LAY>(v, v0 + jv);
             const uint32_t m = vec_mask<LAY>(jv, head, total);
 #pragma unroll
             for (int e = 0; e < (int)E; ++e) {
@@ -1554,7 +1589,7 @@ __device__ __forceinline__ void deliver_tile_plastic(
   uint32_t j0 = 0;
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
-    describe_runs<1, true, false>(v, lv, list, tile, j0, nb, true, pre, nullptr,
+    describe_runs<LAY, 1, true, false>(v, lv, list, tile, j0, nb, true, pre, nullptr,
                                   nullptr, s_desc, s_tprev, s_kprev, s_at);
     __syncthreads();
     fx = s_fx;
@@ -1686,6 +1721,516 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
   const uint2 m = bmap[blockIdx.x];
   const NetView v = nets[m.x].v;
   serve_tile<FMT>(v, m.y, acc_mem, desc_off, desc_cap);
+}
+
+// ---------------------------------------------------------------------------
+// Many intervals in one launch.
+//
+// k_simulate runs the time-driven cycle -- update, exchange of the interval's
+// spikes, delivery -- for a whole call of a net with at most a tile per SM: a
+// cooperative launch, CTA r owning target tile r with its neurons.  Per
+// interval a CTA delivers the previous interval's list into its tile's
+// accumulator, updates the tile's neurons straight from it (what later steps
+// get goes on to the ring buffer), and publishes its spikes; nothing else
+// crosses CTAs.  Each CTA has its own region of the interval's list and a flag
+// word {interval, spike count}; the wait for all flags is the exchange's
+// barrier, and the counts it reads are the list's lengths: one store and one
+// load of latency, no counter shared by all.  Flags and lists alternate
+// between two sets: a CTA writes a set again only after every CTA has
+// published the interval between, hence has read the set.
+//
+// The separate kernels spent, per interval of the 112,500-neuron network, 13
+// us in the update and 22 us in the delivery, of which 12 us with an empty
+// list: launch, list and clock reads, clearing, the ring buffer written by one
+// kernel and read and cleared by the next.  Here the state stays in registers,
+// the drive is drawn while the list's index words arrive, the rows of the
+// neurons that just fired are requested into L2, and all threads of a CTA form
+// the steps' inputs however few targets it has.  What bounds it: instructions
+// of the accumulation (12 of 33 us at 112,500 neurons), then latencies in
+// series (10.9 us an interval of 10 steps at 1,250 neurons).  Per interval,
+// separate kernels -> this: 1,250 neurons FP32 13.8 -> 10.9 us, 20,003 BF16
+// 18.2 -> 15.8, 112,500 FP32 34.0 -> 33.5; 562,500 (304 tiles) would go 143 ->
+// 178 us and keeps the separate kernels.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kSimMaxCtas = 256;
+constexpr uint32_t kSimMaxSteps = 32;     // steps of an interval (one spike mask)
+constexpr uint32_t kDriveBits = 10;       // leading bits of a draw per table entry
+// Polls of a CTA that waits for another one's spikes before it gives up
+// (about a microsecond each): the error is flagged and every CTA leaves.
+constexpr uint32_t kSimPolls = 1u << 24;
+
+// Cells' kind by layout: the persistent cycle runs only nets whose scales (and
+// counts) exist for every interval.
+template <int LAY> struct SimCell {
+  static constexpr int kKind = LAY == kLayHom ? kCellCounts
+                             : LAY == kLayI16 ? kCellOne : kCellTwo;
+  static constexpr bool kTwo = LAY == kLayF32 || LAY == kLayJ16;
+};
+
+// draw(seed, id, block, 2) with the seed's round keys (seed + r x the Weyl
+// increments) as kernel constants.
+__device__ __forceinline__ U4 draw_keys(const SimShared& sh, uint32_t id, uint32_t block) {
+  U4 c{id, block, 0u, 2u};
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    const uint64_t m0 = (uint64_t)0xD2511F53u * c.x;
+    const uint64_t m1 = (uint64_t)0xCD9E8D57u * c.z;
+    c = U4{(uint32_t)(m1 >> 32) ^ c.y ^ sh.key[2 * r], (uint32_t)m1,
+           (uint32_t)(m0 >> 32) ^ c.w ^ sh.key[2 * r + 1], (uint32_t)m0};
+  }
+  return c;
+}
+
+// Poisson counts of four draws, a byte each.  tab[w >> 22] holds the outcomes below the draw's
+// bucket (bits 22 on) plus 2^22 less the one threshold inside it: adding the
+// draw's low bits carries exactly when the draw reaches that threshold.
+// Buckets with more thresholds (the tail) have bit 31 set and are searched.
+__device__ __forceinline__ uint32_t drive_counts(const U4& d, const uint32_t* tab,
+                                                 const uint32_t* thr, int n_thr) {
+  constexpr int kS = 32 - kDriveBits;
+  constexpr uint32_t kLow = (1u << kS) - 1u;
+  const uint32_t w[4] = {d.x, d.y, d.z, d.w};
+  uint32_t e[4], out = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) e[q] = tab[w[q] >> kS];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) out |= ((e[q] + (w[q] & kLow)) >> kS) << (8 * q);
+  if ((int)(e[0] | e[1] | e[2] | e[3]) < 0) {
+    out = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t k = (e[q] + (w[q] & kLow)) >> kS;
+      if ((int)e[q] < 0) {
+        k = (e[q] & 0x7FFFFFFFu) >> kS;
+        while ((int)k < n_thr - 1 && w[q] >= thr[k]) ++k;
+      }
+      out |= k << (8 * q);
+    }
+  }
+  return out;
+}
+
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+  unsigned long long x;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(p) : "memory");
+  return x;
+}
+__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long x) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(x) : "memory");
+}
+
+// Requests the bytes [p, p + bytes) into L2 (whole 16-byte units around them).
+__device__ __forceinline__ void prefetch_l2(const void* p, uint64_t bytes) {
+  const uint64_t a = reinterpret_cast<uint64_t>(p) & ~15ull;
+  const uint64_t e = (reinterpret_cast<uint64_t>(p) + bytes + 15ull) & ~15ull;
+  if (e > a)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                 ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
+}
+// The stream of the row [beg, end) that a delivery of its source reads.
+template <int LAY>
+__device__ __forceinline__ void prefetch_stream(const NetView& v, uint64_t beg,
+                                                uint64_t len) {
+  const char* d = reinterpret_cast<const char*>(v.dat);
+  if constexpr (LAY == kLayHom) {
+    prefetch_l2(d + 2 * beg * v.row_mul, 2 * len);
+  } else {
+    prefetch_l2(d + 4 * beg * v.row_mul, 4 * len);
+    if constexpr (LAY == kLayF32)
+      prefetch_l2(reinterpret_cast<const char*>(v.cells) + 2 * beg, 2 * len);
+  }
+}
+
+__device__ __forceinline__ uint32_t ld_list(const uint32_t* p) {
+  uint32_t x;
+  asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
+  return x;
+}
+
+__device__ __forceinline__ uint64_t ld_row(const uint64_t* p) {
+  uint64_t x;
+  asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(p) : "memory");
+  return x;
+}
+
+template <int LAY>
+__global__ void __launch_bounds__(kTileThreads, 1)
+k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c,
+           SimShared sh, int n_iv, int n_steps, int last_steps,
+           uint32_t drv_off, uint32_t desc_off, uint32_t desc_cap,
+           uint32_t pf_rows) {
+  extern __shared__ __align__(16) int acc[];
+  // drive of the interval to come: [4-step block][target], a byte a step
+  uint32_t* const s_drv =
+      reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(acc) + drv_off);
+  SegDesc* const s_desc =
+      reinterpret_cast<SegDesc*>(reinterpret_cast<char*>(acc) + desc_off);
+  __shared__ uint32_t s_tab[1u << kDriveBits];
+  __shared__ uint32_t s_thr[kMaxPoisson];
+  __shared__ uint32_t s_start[kSimMaxCtas + 1];  // list index of each CTA's first
+  __shared__ uint32_t s_wsum[kSimMaxCtas / 32];
+  __shared__ uint32_t s_cnt;                     // spikes published this interval
+  __shared__ int s_bad;
+  __shared__ FixScale s_fx;
+  __shared__ unsigned long long s_sum[2];
+  constexpr int KIND = SimCell<LAY>::kKind;
+  constexpr bool TWO = SimCell<LAY>::kTwo;
+  const uint32_t G = gridDim.x, r = blockIdx.x;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u;
+  const uint32_t TW = v.tile_w, W = (uint32_t)v.window, cells = W * TW;
+  const uint32_t acc_s = (uint32_t)__cvta_generic_to_shared(acc);
+  const uint32_t magic = cell_magic(TW);
+  const bool single = TW <= (uint32_t)kTileThreads;  // one neuron a thread
+  const uint32_t lo = r * TW, x_end = min(TW, v.n - lo);  // this CTA's targets
+  const bool drive = c.n_thr > 0;
+
+  // the drive's table and thresholds, an empty accumulator
+  for (uint32_t k = tid; k < (uint32_t)c.n_thr; k += kTileThreads) s_thr[k] = c.thr[k];
+  for (uint32_t x = tid; x < (TWO ? 2 * cells : cells); x += kTileThreads) acc[x] = 0;
+  if (tid == 0) {
+    s_cnt = 0;
+    s_bad = 0;
+    s_sum[0] = s_sum[1] = 0ull;
+    s_fx = FixScale{0, 0, 0, 1.f, 1.f, 1.f, 1.f};
+  }
+  if (drive) {
+    constexpr uint32_t kSpan = 1u << (32 - kDriveBits);
+    const uint32_t lo = tid * kSpan;  // (one entry a thread)
+    uint32_t k = 0, inside = 0, thr = 0;
+    for (int m = 0; m < c.n_thr - 1; ++m) {
+      const uint32_t x = c.thr[m];
+      if (x <= lo) ++k;
+      else if (x - lo < kSpan) { ++inside; thr = x; }
+    }
+    s_tab[tid] = inside > 1 ? 0x80000000u | (k << (32 - kDriveBits))
+                            : (k << (32 - kDriveBits)) + (inside ? kSpan - (thr - lo) : 0u);
+  }
+  static_assert((1u << kDriveBits) == (uint32_t)kTileThreads, "an entry a thread");
+  // (clocks stay below 2^31)
+  int t = (int)*reinterpret_cast<volatile long long*>(&v.ctl->t_now);
+  unsigned long long logged = *reinterpret_cast<volatile unsigned long long*>(&v.ctl->log_count);
+  unsigned long long my_events = 0, my_spikes = 0;
+  __syncthreads();
+
+  // state of this thread's neuron, kept over the launch when it has only one
+  float V = 0.f, I = 0.f, J = 0.f;
+  int refr = 0;
+  if (single && tid < x_end) {
+    const uint32_t i = lo + tid;
+    V = v.V[i];
+    I = v.I[i];
+    J = v.J[i];
+    refr = v.refr[i];
+  }
+
+  const uint32_t* list = nullptr;  // the list published last
+  uint32_t n_sp = 0;
+  int t_list = 0;                  // its first step
+  // one round more than intervals: the last delivers the last list into the
+  // ring buffer
+  int iv = 0;
+  for (; iv <= n_iv; ++iv) {
+    const int steps = iv == n_iv ? 0 : iv == n_iv - 1 ? last_steps : n_steps;
+    uint32_t* const my_list =
+        sh.list + (size_t)((uint32_t)(iv & 1) * G + r) * sh.region;
+    // step of the window's slot 0: the round's first step (the interval is the
+    // minimum delay), but after a last, shorter interval
+    const int tb = iv == n_iv ? t_list + v.d_min : t;
+    const int b0 = tb >> 2, a0 = tb & 3;  // the round's first 4-step block
+    const uint32_t nb_up = steps ? (uint32_t)((a0 + steps + 3) >> 2) : 0u;
+    // draws the drive of the steps to come (while the index words arrive)
+    auto draw_drive = [&]() {
+      if (!drive) return;
+      for (uint32_t k = tid; k < nb_up * TW; k += kTileThreads) {
+        const uint32_t j = cell_step(k, magic), x = k - j * TW;
+        s_drv[k] = drive_counts(draw_keys(sh, v.g0 + lo + x, (uint32_t)b0 + j),
+                                s_tab, s_thr, c.n_thr);
+      }
+    };
+    // (1) the list's events for this tile into the accumulator
+    if (iv > 0 && tid == kTileThreads - 1) s_fx = fix_scale(v, n_sp, true);
+    uint32_t j0 = 0;
+    do {
+      const uint32_t nb = min(desc_cap, n_sp - j0);
+      for (uint32_t k0 = tid; k0 < nb || k0 == tid; k0 += 2 * kTileThreads) {
+        uint32_t e[2] = {0u, 0u}, ra[2] = {0u, 0u}, rb[2] = {0u, 0u};
+        uint64_t row[2] = {0ull, 0ull};
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (k0 + u * kTileThreads >= nb) continue;
+          // the CTA whose region holds list entry g: the last one that
+          // starts at or before it (empty ones start where the next does)
+          const uint32_t g = j0 + k0 + u * kTileThreads;
+          uint32_t at = 0, hi = G;
+          while (hi - at > 1) {
+            const uint32_t mid = (at + hi) >> 1;
+            if (s_start[mid] <= g) at = mid; else hi = mid;
+          }
+          e[u] = ld_list(list + (size_t)at * sh.region + (g - s_start[at]));
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (k0 + u * kTileThreads >= nb) continue;
+          const uint32_t src = e[u] & 0xFFFFFFu;
+          const uint32_t* to = v.tile_off + (uint64_t)src * (v.n_tiles + 1) + r;
+          ra[u] = ld_list(to);
+          rb[u] = ld_list(to + 1);
+          row[u] = ld_row(v.row_ptr + src);
+        }
+        if (j0 == 0 && k0 == tid) draw_drive();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const uint32_t k = k0 + u * kTileThreads;
+          if (k >= nb) continue;
+          SegDesc sd;
+          place_run<LAY>(v, row[u] * v.row_mul + ra[u], rb[u] - ra[u], &sd);
+          // (base = t_list + d_min)
+          sd.off = ((int32_t)(e[u] >> 24) - v.d_min + v.d_base) * (int32_t)TW;
+          if (LAY == kLayHom && (e[u] & 0xFFFFFFu) >= v.hom_split) sd.len |= 0x80000000u;
+          s_desc[k] = sd;
+        }
+      }
+      uint32_t lg = (uint32_t)v.lg;
+      while (lg < 5u && (nb << (lg + 1u)) <= (uint32_t)kTileThreads) ++lg;
+      __syncthreads();
+      if (nb)
+        add_runs_call<LAY>(reinterpret_cast<const char*>(v.dat),
+                           reinterpret_cast<const char*>(v.cells), s_desc, nb,
+                           acc_s, TWO ? 4u * cells : 0u, lg,
+                           SplitScale{s_fx.scale_hs, s_fx.scale_s});
+      j0 += nb;
+      if (j0 < n_sp) __syncthreads();  // s_desc is rewritten by the next batch
+    } while (j0 < n_sp);
+    // (2) the input of every step and target: the ring buffer's value and
+    // the list's sum and drive, as a float in the cell's place; later steps'
+    // sums go on to the ring buffer.  All threads take part, however few
+    // targets the tile has, four cells at a time.
+    {
+      const FixScale fx = s_fx;
+      const CellValue val(v, fx);
+      const uint32_t n_in = (uint32_t)steps * TW;
+      bool first = true;
+      for (uint32_t k0 = tid; first || k0 < n_in; k0 += 4 * kTileThreads) {
+        float in[4];
+        uint32_t st[4], at[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t k = k0 + q * kTileThreads;
+          st[q] = cell_step(k, magic);
+          at[q] = k - st[q] * TW;
+          in[q] = 0.f;
+          if (k < n_in && at[q] < x_end)
+            in[q] = __ldcg(v.rb + lo + at[q] +
+                           (size_t)((uint32_t)(tb + st[q]) & v.slot_mask) * v.pitch);
+        }
+        if (first) __syncthreads();  // the sums are complete
+        first = false;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t k = k0 + q * kTileThreads;
+          if (k >= n_in || at[q] >= x_end) continue;
+          const float a = val.get<KIND>(acc, k, cells);
+          if (__float_as_uint(in[q]) != 0u)
+            v.rb[lo + at[q] + (size_t)((uint32_t)(tb + st[q]) & v.slot_mask) * v.pitch] = 0.f;
+          if (a != 0.f) in[q] += a;
+          if (drive) {
+            const uint32_t u = (uint32_t)a0 + st[q];
+            in[q] += c.w_ext * (float)((s_drv[(u >> 2) * TW + at[q]] >> (8u * (u & 3u))) & 0xFFu);
+          }
+          reinterpret_cast<float*>(acc)[k] = in[q];
+          if (TWO) acc[cells + k] = 0;
+        }
+      }
+      if (iv > 0)
+        for (uint32_t k = n_in + tid; k < cells; k += kTileThreads) {
+          const float a = val.get<KIND>(acc, k, cells);
+          if (a != 0.f) {
+            const uint32_t sl = cell_step(k, magic);
+            red_add_f32(v.rb + lo + (k - sl * TW) +
+                            (size_t)((uint32_t)(tb + sl) & v.slot_mask) * v.pitch, a);
+          }
+          acc[k] = 0;
+          if (TWO) acc[cells + k] = 0;
+        }
+    }
+    if (steps == 0) break;
+    __syncthreads();
+    // (3) the neurons, a thread each, through the interval's steps
+    for (uint32_t x0 = 0; x0 < TW; x0 += kTileThreads) {
+      const uint32_t x = x0 + tid, i = lo + x;
+      const bool live = x < x_end;
+      uint32_t mask = 0;
+      if (live) {
+        if (!single) {
+          V = v.V[i];
+          I = v.I[i];
+          J = v.J[i];
+          refr = v.refr[i];
+        }
+        int* p = acc + x;
+        float in = __int_as_float(*p);
+        for (int s = 0; s < steps; ++s, p += TW) {
+          const float next = s + 1 < steps ? __int_as_float(p[TW]) : 0.f;
+          *p = 0;
+          if (update_step(c, V, I, J, refr, in)) mask |= 1u << s;
+          in = next;
+        }
+        if (!single) {
+          v.V[i] = V;
+          v.I[i] = I;
+          v.J[i] = J;
+          v.refr[i] = refr;
+        }
+      }
+      // this tile's spikes into the CTA's region of the list
+      const uint32_t cnt = __popc(mask);
+      uint32_t at = 0;
+      if (__ballot_sync(kFull, cnt != 0)) {
+        uint32_t inc = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(kFull, inc, o);
+          if (lane >= (unsigned)o) inc += y;
+        }
+        if (lane == 31u) at = atomicAdd(&s_cnt, inc);
+        at = __shfl_sync(kFull, at, 31) + inc - cnt;
+        uint32_t to = at;
+        for (uint32_t m = mask; m; m &= m - 1u, ++to)
+          if (to < sh.region)  // (always: simulate_fits)
+            my_list[to] = (v.g0 + i) | ((uint32_t)(__ffs(m) - 1) << 24);
+      }
+      if (x0 + kTileThreads >= TW) {
+        // publish: every thread's entries, then the count (the release
+        // covers what the barrier ordered before it)
+        __syncthreads();
+        if (tid == 0)
+          st_release_u64(&sh.flags[(uint32_t)(iv & 1) * kSimMaxCtas + r],
+                         ((unsigned long long)(iv + 1) << 32) | s_cnt);
+      }
+      if (cnt) {
+        // the deliveries that follow read this source's row of the tile
+        // index and, for as many rows as L2 takes, its synapses
+        prefetch_row_l2(v, v.g0 + i);
+        const uint64_t beg = v.row_ptr[v.g0 + i];
+        const uint64_t len = v.row_ptr[v.g0 + i + 1] - beg;
+        if (at < pf_rows) prefetch_stream<LAY>(v, beg, len);
+        my_events += cnt * len;
+        my_spikes += cnt;
+        if (v.isi_spikes) {
+          int32_t last = v.isi_last[i];
+          uint32_t n_isi = v.isi_n[i];
+          double s1 = v.isi_sum[i], s2 = v.isi_sq[i];
+          for (uint32_t m = mask; m; m &= m - 1u) {
+            const int32_t ts = t + __ffs(m) - 1;
+            if (last != kNoSpike) {
+              const double d = (double)(ts - last);  // exact in FP64
+              s1 += d;
+              s2 += d * d;
+              n_isi += 1u;
+            }
+            last = ts;
+          }
+          v.isi_last[i] = last;
+          v.isi_spikes[i] += cnt;
+          v.isi_n[i] = n_isi;
+          v.isi_sum[i] = s1;
+          v.isi_sq[i] = s2;
+        }
+      }
+    }
+    t_list = t;
+    t += steps;
+    // (4) every CTA's count (thread k: CTA k's), and where its entries start
+    if (tid < kSimMaxCtas) {
+      uint32_t n_r = 0;
+      if (tid < G) {
+        const unsigned long long* f = &sh.flags[(uint32_t)(iv & 1) * kSimMaxCtas + tid];
+        unsigned long long x;
+        uint32_t polls = 0;
+        while ((uint32_t)((x = ld_acquire_u64(f)) >> 32) != (uint32_t)(iv + 1)) {
+          ++polls;
+          if (polls > kSimPolls ||
+              ((polls & 1023u) == 0u &&
+               *reinterpret_cast<volatile unsigned int*>(sh.stop))) {
+            s_bad = 1;
+            break;
+          }
+        }
+        n_r = (uint32_t)x;
+      }
+      uint32_t inc = n_r;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= (unsigned)o) inc += y;
+      }
+      if (lane == 31u) s_wsum[tid >> 5] = inc;
+      s_start[tid] = inc - n_r;
+    }
+    if (tid == 0) s_cnt = 0;
+    __syncthreads();
+    if (s_bad) break;  // (uniform: read after the barrier)
+    n_sp = 0;
+    uint32_t before = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < kSimMaxCtas / 32; ++w) {
+      if (w == (tid >> 5)) before = n_sp;
+      n_sp += s_wsum[w];
+    }
+    if (tid < kSimMaxCtas) s_start[tid] += before;
+    __syncthreads();
+    list = sh.list + (size_t)((uint32_t)(iv & 1) * G) * sh.region;
+    // this CTA's spikes into the log, at their place in the list
+    if (v.log_cap && tid >= kTileThreads / 2) {
+      const uint32_t mine = (r + 1 < G ? s_start[r + 1] : n_sp) - s_start[r];
+      for (uint32_t k = kTileThreads - 1 - tid; k < mine; k += kTileThreads / 2) {
+        const uint32_t e = ld_list(my_list + k);
+        const unsigned long long at = logged + s_start[r] + k;
+        if (at < v.log_cap) {
+          v.log_src[at] = e & 0xFFFFFFu;
+          v.log_t[at] = t_list + (int32_t)(e >> 24);
+        } else {
+          atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_SPIKE_LOG);
+        }
+      }
+    }
+    logged += n_sp;
+  }
+  if (s_bad && tid == 0) {
+    // a wait ran out: the others leave as well
+    atomicExch(sh.stop, 1u);
+    atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_TIMEOUT);
+  }
+  if (single && tid < x_end) {
+    const uint32_t i = lo + tid;
+    v.V[i] = V;
+    v.I[i] = I;
+    v.J[i] = J;
+    v.refr[i] = refr;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    my_events += __shfl_xor_sync(kFull, my_events, o);
+    my_spikes += __shfl_xor_sync(kFull, my_spikes, o);
+  }
+  if (lane == 0 && my_spikes) {
+    atomicAdd(&s_sum[0], my_events);
+    atomicAdd(&s_sum[1], my_spikes);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    if (s_sum[1]) {
+      atomicAdd(&v.ctl->events, s_sum[0]);
+      atomicAdd(&v.ctl->spikes, s_sum[1]);
+    }
+    // (every CTA read the clock and the log's length before its first
+    // publication, so before this one saw all of them)
+    if (r == 0) {
+      v.ctl->t_now = t;
+      v.ctl->iv_steps = last_steps;
+      if (v.log_cap) v.ctl->log_count = logged;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -2123,6 +2668,105 @@ cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
     default: return SNN_TILED(kLayJ16);
   }
 #undef SNN_TILED
+}
+
+// Whether the intervals of a net can run in k_simulate: a split store whose
+// scales (and counts) exist for every interval, nothing that only the
+// separate kernels do (plasticity, counted cells, exchange buffers, bounds
+// checks), and lists that fit the interval list's memory.
+template <int LAY>
+cudaError_t launch_simulate_t(const NetView& v, const UpdConst& c,
+                              const SimShared& sh, uint32_t ctas, int n_iv,
+                              int steps, int last_steps, cudaStream_t s) {
+  static std::atomic<uint32_t> lim[64];
+  size_t dm = 0;
+  cudaError_t e = allow_tile_smem(k_simulate<LAY>, lim, &dm);
+  if (e != cudaSuccess) return e;
+  DescLayout dl;  // after the accumulator and the drive (5 or 9 blocks)
+  const size_t drv = ((size_t)v.tile_w * v.window * (SimCell<LAY>::kTwo ? 8u : 4u) + 15u) & ~(size_t)15u;
+  const size_t blocks = ((size_t)steps + 6) / 4;
+  e = desc_layout(drv + blocks * v.tile_w * 4u, dm, false, &dl);
+  if (e != cudaSuccess) return e;
+  // as many rows of a CTA's spikes are requested ahead as a third of L2 holds
+  // of all CTAs'
+  const double row = v.n_src ? (double)v.mean_row * (LAY == kLayHom ? 2.0 : LAY == kLayF32 ? 6.0 : 4.0) : 1.0;
+  const uint32_t pf = (uint32_t)std::max(1.0, 40e6 / (std::max(row, 64.0) * ctas));
+  e = cudaMemsetAsync(sh.flags, 0, kSimFlagBytes, s);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kTileThreads);
+  cfg.dynamicSmemBytes = dl.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;  // every CTA waits for the others
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_simulate<LAY>, v, c, sh, n_iv, steps,
+                            last_steps, (uint32_t)drv, dl.off, dl.cap, pf);
+}
+
+static int sim_sms() {
+  static std::atomic<int> sms[64];
+  int dev = 0, m = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  m = sms[dev].load(std::memory_order_relaxed);
+  if (m == 0) {
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        !coop)
+      m = -1;
+    sms[dev].store(m, std::memory_order_relaxed);
+  }
+  return m;
+}
+
+bool simulate_fits(const NetView& v, const UpdConst& c, int interval,
+                   SimShared* sh, uint32_t* ctas) {
+  // (a reset at or above the threshold fires at every step, refractory or not)
+  if (!(c.v_reset < c.v_th)) return false;
+  if (kChecked || v.lay == kLayRecords || v.plastic || v.counts || v.xbuf ||
+      interval < 1 || interval > (int)kSimMaxSteps || v.n_tiles == 0)
+    return false;
+  const uint64_t e = (uint64_t)v.k_in_max * std::max(v.spikes_per_iv, 1u);
+  const int qs = fixed_qs_host(e, v.max_abs_w);
+  if (qs < 0 || (v.acc_words == 1 && qs < v.acc_qs_min)) return false;
+  // (a list's window starts where the next interval does; room for the drive
+  // and some run descriptors beside the accumulator)
+  if (interval != v.d_min) return false;
+  const uint32_t words = v.lay == kLayF32 || v.lay == kLayJ16 ? 2u : 1u;
+  if ((size_t)v.tile_w * (4u * words * v.window + 4u * ((interval + 6) / 4)) >
+      (size_t)(210 * 1024))
+    return false;
+  // (cells and draws are numbered within 16 bits)
+  if ((uint64_t)v.tile_w * std::max<uint32_t>(v.window, (interval + 6) / 4) > 0xFFFFull)
+    return false;
+  if (v.lay == kLayHom && e > 0xFFFFull) return false;
+  if (v.lay == kLayJ16 && v.acc_words == 1) return false;
+  const int sms = sim_sms();
+  // (nets of more tiles than SMs: the separate kernels, whose grids balance
+  // their tiles, are faster: 7.15 against 8.90 ms at 562,500 neurons)
+  if (sms < 1 || v.n_tiles > std::min<uint32_t>((uint32_t)sms, kSimMaxCtas)) return false;
+  const uint32_t G = v.n_tiles;
+  const uint64_t region = (uint64_t)v.tile_w * std::max(v.spikes_per_iv, 1u);
+  if (2 * G * region * sizeof(uint32_t) > v.list_cap * sizeof(SpikeEntry)) return false;
+  sh->list = reinterpret_cast<uint32_t*>(v.list);
+  sh->region = (uint32_t)region;
+  *ctas = G;
+  return true;
+}
+
+cudaError_t launch_simulate(const NetView& v, const UpdConst& c,
+                            const SimShared& sh, uint32_t ctas, int n_iv,
+                            int steps, int last_steps, cudaStream_t s) {
+  switch (v.lay) {
+    case kLayHom: return launch_simulate_t<kLayHom>(v, c, sh, ctas, n_iv, steps, last_steps, s);
+    case kLayF32: return launch_simulate_t<kLayF32>(v, c, sh, ctas, n_iv, steps, last_steps, s);
+    case kLayI16: return launch_simulate_t<kLayI16>(v, c, sh, ctas, n_iv, steps, last_steps, s);
+    default: return launch_simulate_t<kLayJ16>(v, c, sh, ctas, n_iv, steps, last_steps, s);
+  }
 }
 
 cudaError_t launch_fill_i32(int32_t* p, int32_t value, uint64_t n,

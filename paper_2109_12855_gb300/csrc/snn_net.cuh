@@ -72,6 +72,7 @@ struct snn_net {
   float max_abs_w = 0.f;
   SpikeEntry* list = nullptr;
   uint64_t list_cap = 0;
+  unsigned long long* sim_flags = nullptr;  // see SimShared
   SpikeEntry* ext_list = nullptr;
   uint32_t* ext_src = nullptr;
   int32_t* ext_t = nullptr;
@@ -117,6 +118,7 @@ struct snn_net {
     v->tgts = nullptr;
     v->row_mul = 1;
     v->lg = 0;
+    v->mean_row = n_src ? (float)((double)n_syn / n_src) : 0.f;
     if (lay == kLayRecords) return;
     if (fmt == SNN_W_FP32_12B) {
       const char* p = static_cast<const char*>(recs);

@@ -1234,13 +1234,19 @@ int snn_deliver(snn_net* net, const uint32_t* src, const int32_t* t_emit,
     e0 = pool_event(net, 0);
     e1 = pool_event(net, 1);
   }
-  CK(launch_prepare_external(v, d_src, d_t, n_spikes, net->ext_list,
-                             &net->ctl->ext_pair, s));
+  // a short list needs no preparation: every CTA reads the arrays themselves
+  const bool raw = use_tiled(net) && deliver_raw_fits(v, n_spikes);
+  if (!raw)
+    CK(launch_prepare_external(v, d_src, d_t, n_spikes, net->ext_list,
+                               &net->ctl->ext_pair, s));
   if (e0) CK(cudaEventRecord(e0, s));
-  CK(launch_deliver_any(net, &net->ctl->ext_pair, &net->ctl->ext_done,
-                        net->ext_list, 1, 0));
+  if (raw)
+    CK(launch_deliver_raw(v, d_src, d_t, n_spikes, s));
+  else
+    CK(launch_deliver_any(net, &net->ctl->ext_pair, &net->ctl->ext_done,
+                          net->ext_list, 1, 0));
   if (e1) CK(cudaEventRecord(e1, s));
-  net->launches += 2;
+  net->launches += raw ? 1 : 2;
   net->del_launches += 1;
   if (e1) {
     float ms = 0;

@@ -317,6 +317,10 @@ struct NetView {
   const uint32_t* gx;
   uint64_t gx_stride;
   uint32_t gx_cap;
+  // a caller's spike arrays, delivered as they stand (null otherwise)
+  const uint32_t* ext_src;
+  const int32_t* ext_t;
+  uint32_t ext_n;
   uint32_t* log_src;        // spike log, capacity log_cap
   int32_t* log_t;
   uint64_t log_cap;
@@ -404,6 +408,11 @@ cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
                                  int from_list_range, int advance_time,
                                  cudaStream_t s);
 size_t tiled_smem_bytes(const NetView& v);
+// A caller's arrays of n spikes delivered without preparing a list: whether
+// the store and the length allow it, and the launch.
+bool deliver_raw_fits(const NetView& v, uint32_t n);
+cudaError_t launch_deliver_raw(const NetView& v, const uint32_t* src,
+                               const int32_t* t, uint32_t n, cudaStream_t s);
 // Batched kernels (serving): bmap entries are (net index, block or tile).
 cudaError_t launch_update_batch(const BatchNet* nets, const uint2* bmap,
                                 uint32_t n_blocks, cudaStream_t s);

@@ -897,6 +897,14 @@ __device__ __noinline__ StdpOut stdp_weight(float w, int32_t t, uint32_t d,
   return o;
 }
 
+// Where a tiled delivery's list comes from: the interval's own list (or a
+// caller's, prepared in the same form), the partitions' exchange buffers
+// (v.gx), or a caller's arrays as they stand (v.ext_*).
+enum ListKind { kListOwn, kListGathered, kListRaw };
+// A caller's list up to this long is read by every CTA as it stands (four
+// entries a thread); a longer one is prepared by k_prepare_external first.
+constexpr uint32_t kRawMax = 4 * kTileThreads;
+
 // Places the run of elements [first, first + len) of v's stream in a
 // descriptor.
 template <int LAY>
@@ -920,13 +928,14 @@ struct ListView {
 // list entries per thread in flight, then their tile-index words and row
 // starts.  pre (pre_g): entries threadIdx.x + u blockDim.x of the list, read
 // ahead of its length (have_pre).  Returns the events described (gathered
-// lists).  PL: also the presynaptic history the plastic rule needs.
-template <int LAY, int DU, bool PL, bool GX>
+// lists and callers' arrays).  PL: also the presynaptic history the plastic rule needs.
+template <int LAY, int DU, bool PL, int KIND>
 __device__ __forceinline__ unsigned long long describe_runs(
     const NetView& v, const ListView& lv, const SpikeEntry* list, uint32_t tile,
     uint32_t j0, uint32_t nb, bool have_pre, const SpikeEntry* pre,
     const uint2* pre_g, const uint32_t* s_gstart, SegDesc* s_desc,
     int32_t* s_tprev, float* s_kprev, uint32_t* s_at) {
+  constexpr bool GX = KIND == kListGathered, RAW = KIND == kListRaw;
   const uint32_t row_stride = v.n_tiles + 1;
   const uint32_t iv_span = (uint32_t)(v.window - (v.d_max - v.d_min));
   unsigned long long my_events = 0;
@@ -955,6 +964,12 @@ __device__ __forceinline__ unsigned long long describe_runs(
                           (uint32_t)((int32_t)x.y - (int32_t)lv.t_now) < iv_span;
           if (!ok) atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_BAD_SOURCE);
           src[u] = ok ? x.x : 0xFFFFFFFFu;
+          t[u] = (int32_t)x.y;
+        } else if constexpr (RAW) {
+          const uint2 x = have ? pre_g[u]
+                               : make_uint2(v.ext_src[j0 + k], (uint32_t)v.ext_t[j0 + k]);
+          if (x.x >= v.n_src) atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_BAD_SOURCE);
+          src[u] = x.x;
           t[u] = (int32_t)x.y;
         } else {
           const SpikeEntry e = have ? pre[u] : list[j0 + k];
@@ -985,7 +1000,7 @@ __device__ __forceinline__ unsigned long long describe_runs(
           len = 0;
         }
 #endif
-        if (GX) my_events += len;
+        if (GX || RAW) my_events += len;
         if constexpr (PL) {
           sd.beg = row * v.row_mul + a;
           sd.len = len;
@@ -1003,8 +1018,8 @@ __device__ __forceinline__ unsigned long long describe_runs(
       }
     }
   }
-  // gathered lists: the warp's events (all threads of the CTA reach this)
-  if (GX) {
+  // the warp's events (all threads of the CTA reach this)
+  if (GX || RAW) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) my_events += __shfl_xor_sync(kFull, my_events, o);
   }
@@ -1242,17 +1257,19 @@ __device__ __noinline__ void add_runs_call(const char* dat, const char* cel,
 }
 
 // One interval's (or one caller's) list for tile `tile`.
-template <int LAY, bool COUNT, bool GX>
+template <int LAY, bool COUNT, int KIND>
 __device__ __forceinline__ void deliver_tile_body(
     const NetView& v, unsigned long long* pair_p, unsigned int* done_p,
     const SpikeEntry* __restrict__ list, int from_list_range, int advance_time,
     uint32_t tile, int* acc_mem, uint32_t desc_off, uint32_t desc_cap) {
   constexpr uint32_t E = Lay<LAY>::kElems;
+  constexpr bool GX = KIND == kListGathered, RAW = KIND == kListRaw;
   SegDesc* const s_desc =
       reinterpret_cast<SegDesc*>(reinterpret_cast<char*>(acc_mem) + desc_off);
   __shared__ FixScale s_fx;
+  __shared__ int s_range[2];  // callers' arrays: first and last emission step
   __shared__ uint32_t s_gstart[GX ? kMaxGatherParts + 1 : 1];
-  __shared__ unsigned long long s_events;  // gathered lists: this CTA's events
+  __shared__ unsigned long long s_events;  // (GX, RAW) this CTA's events
   const uint32_t TW = v.tile_w;
   const uint32_t W = (uint32_t)v.window;
   const uint32_t cells = W * TW;
@@ -1266,14 +1283,17 @@ __device__ __forceinline__ void deliver_tile_body(
   // memory round trip fewer before the runs can be described); entries past
   // the length are never used.
   constexpr int kDU = 4;
-  SpikeEntry pre[GX ? 1 : kDU];
-  uint2 pre_g[GX ? kDU : 1];
-  const bool spec = !from_list_range;
+  SpikeEntry pre[GX || RAW ? 1 : kDU];
+  uint2 pre_g[GX || RAW ? kDU : 1];
+  const bool spec = RAW || !from_list_range;
   if (spec) {
 #pragma unroll
     for (int u = 0; u < kDU; ++u) {
       const uint32_t k = threadIdx.x + u * blockDim.x;
-      if constexpr (GX) {  // part 0's first entries (its count comes next)
+      if constexpr (RAW) {
+        pre_g[u] = make_uint2(0xFFFFFFFFu, 0u);
+        if (k < v.ext_n) pre_g[u] = make_uint2(v.ext_src[k], (uint32_t)v.ext_t[k]);
+      } else if constexpr (GX) {  // part 0's first entries (its count comes next)
         if (k < desc_cap && k < v.gx_cap)
           pre_g[u] = reinterpret_cast<const uint2*>(v.gx + 4)[k];
       } else {
@@ -1297,14 +1317,37 @@ __device__ __forceinline__ void deliver_tile_body(
     }
     s_gstart[v.gx_parts] = run;
     lv.n_sp = run;
+  } else if constexpr (RAW) {
+    lv.n_sp = v.ext_n;
+    if (threadIdx.x == 0) {
+      s_range[0] = INT_MAX;
+      s_range[1] = INT_MIN;
+      s_events = 0ull;
+    }
+    __syncthreads();
+    int lo = INT_MAX, hi = INT_MIN;
+#pragma unroll
+    for (int u = 0; u < kDU; ++u)
+      if (threadIdx.x + u * blockDim.x < v.ext_n) {
+        lo = min(lo, (int)pre_g[u].y);
+        hi = max(hi, (int)pre_g[u].y);
+      }
+    lo = __reduce_min_sync(kFull, lo);
+    hi = __reduce_max_sync(kFull, hi);
+    if (lane == 0 && lo <= hi) {
+      atomicMin(&s_range[0], lo);
+      atomicMax(&s_range[1], hi);
+    }
+    __syncthreads();
   } else {
     const unsigned long long pr =
         *reinterpret_cast<volatile unsigned long long*>(pair_p);
     lv.n_sp = (uint32_t)(pr >> 32);
   }
   lv.t_now = GX ? v.ctl->t_now : 0ll;
-  if (from_list_range) {
-    const long long tmin = v.ctl->ext_tmin, tmax = v.ctl->ext_tmax;
+  if (RAW || from_list_range) {
+    const long long tmin = RAW ? s_range[0] : v.ctl->ext_tmin;
+    const long long tmax = RAW ? s_range[1] : v.ctl->ext_tmax;
     lv.base = tmin + v.d_min;
     lv.inwin = (tmax - tmin) + (v.d_max - v.d_min) + 1 <= (long long)W;
   } else {
@@ -1314,11 +1357,11 @@ __device__ __forceinline__ void deliver_tile_body(
   const uint32_t n_sp = lv.n_sp;
   const long long base = lv.base;
   // (the last thread: it describes no run of a list of up to 1,023 spikes)
-  if (threadIdx.x == kTileThreads - 1) s_fx = fix_scale(v, n_sp, !from_list_range);
+  if (threadIdx.x == kTileThreads - 1) s_fx = fix_scale(v, n_sp, !RAW && !from_list_range);
   if (GX && threadIdx.x == 0) s_events = 0ull;
   // (an interval's own list of a uniform store always fits its counts when
   // the largest interval's does: one word a cell)
-  const bool one = !two || (LAY == kLayHom && !from_list_range &&
+  const bool one = !two || (LAY == kLayHom && !RAW && !from_list_range &&
                             (uint64_t)v.k_in_max * v.spikes_per_iv <= 0xFFFFull);
   for (uint32_t x = threadIdx.x; x < (one ? cells : 2 * cells); x += blockDim.x)
     acc_mem[x] = 0;
@@ -1360,7 +1403,7 @@ __device__ __forceinline__ void deliver_tile_body(
   uint32_t j0 = 0;
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
-    const unsigned long long warp_events = describe_runs<LAY, kDU, false, GX>(
+    const unsigned long long warp_events = describe_runs<LAY, kDU, false, KIND>(
         v, lv, list, tile, j0, nb, spec, pre, pre_g, s_gstart, s_desc, nullptr, nullptr, nullptr);
     // a batch of few runs spreads them over all lanes of the CTA
     lg = (uint32_t)v.lg;
@@ -1371,7 +1414,7 @@ __device__ __forceinline__ void deliver_tile_body(
     grp = lane >> lg;
     __syncthreads();
     // (after the barrier: s_events was cleared before it)
-    if (GX && lane == 0 && warp_events) atomicAdd(&s_events, warp_events);
+    if ((GX || RAW) && lane == 0 && warp_events) atomicAdd(&s_events, warp_events);
     fx = s_fx;
     const bool fast = !COUNT && !kChecked && lv.inwin &&
                       (LAY == kLayHom ? fx.packed : fx.fixed);
@@ -1424,10 +1467,15 @@ __device__ __forceinline__ void deliver_tile_body(
   // The last CTA to finish clears the list counters and advances the clock
   // (a gathered list's events -- its spikes' runs onto this partition's
   // targets -- are counted by the CTAs themselves).
+  // A caller's arrays leave no counters behind but the events.
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (GX && s_events) atomicAdd(&v.ctl->gx_events, s_events);
-    finish_list(v, pair_p, done_p, advance_time, GX);
+    if (RAW) {
+      if (s_events) atomicAdd(&v.ctl->events, s_events);
+    } else {
+      if (GX && s_events) atomicAdd(&v.ctl->gx_events, s_events);
+      finish_list(v, pair_p, done_p, advance_time, GX);
+    }
   }
 }
 
@@ -1589,7 +1637,7 @@ __device__ __forceinline__ void deliver_tile_plastic(
   uint32_t j0 = 0;
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
-    describe_runs<LAY, 1, true, false>(v, lv, list, tile, j0, nb, true, pre, nullptr,
+    describe_runs<LAY, 1, true, kListOwn>(v, lv, list, tile, j0, nb, true, pre, nullptr,
                                   nullptr, s_desc, s_tprev, s_kprev, s_at);
     __syncthreads();
     fx = s_fx;
@@ -1660,13 +1708,13 @@ __device__ __forceinline__ void deliver_tile_plastic(
   }
 }
 
-template <int LAY, bool COUNT, bool GX>
+template <int LAY, bool COUNT, int KIND>
 __global__ void __launch_bounds__(kTileThreads, 1)
 k_deliver_tiled(NetView v, unsigned long long* pair_p, unsigned int* done_p,
                 const SpikeEntry* __restrict__ list, int from_list_range,
                 int advance_time, uint32_t desc_off, uint32_t desc_cap) {
   extern __shared__ __align__(16) int acc_mem[];
-  deliver_tile_body<LAY, COUNT, GX>(v, pair_p, done_p, list,
+  deliver_tile_body<LAY, COUNT, KIND>(v, pair_p, done_p, list,
                                          from_list_range, advance_time,
                                          blockIdx.x, acc_mem, desc_off, desc_cap);
   // the next update may be scheduled once every CTA got here
@@ -1700,13 +1748,13 @@ __device__ __forceinline__ void serve_tile(const NetView& v, uint32_t tile,
                                            int* acc_mem, uint32_t desc_off,
                                            uint32_t desc_cap) {
   if (v.lay == kLayHom)
-    deliver_tile_body<kLayHom, false, false>(
+    deliver_tile_body<kLayHom, false, kListOwn>(
         v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
   else if (FMT == SNN_W_BF16_8B && v.lay == kLayI16)
-    deliver_tile_body<kLayI16, false, false>(
+    deliver_tile_body<kLayI16, false, kListOwn>(
         v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
   else
-    deliver_tile_body<FMT == SNN_W_FP32_12B ? kLayF32 : kLayJ16, false, false>(
+    deliver_tile_body<FMT == SNN_W_FP32_12B ? kLayF32 : kLayJ16, false, kListOwn>(
         v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
 }
 
@@ -1746,11 +1794,12 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
 // the drive is drawn while the list's index words arrive, the rows of the
 // neurons that just fired are requested into L2, and all threads of a CTA form
 // the steps' inputs however few targets it has.  What bounds it: instructions
-// of the accumulation (12 of 33 us at 112,500 neurons), then latencies in
-// series (10.9 us an interval of 10 steps at 1,250 neurons).  Per interval,
-// separate kernels -> this: 1,250 neurons FP32 13.8 -> 10.9 us, 20,003 BF16
-// 18.2 -> 15.8, 112,500 FP32 34.0 -> 33.5; 562,500 (304 tiles) would go 143 ->
-// 178 us and keeps the separate kernels.
+// of the accumulation (about 11 of 30 us an interval at 112,500 neurons), then
+// latencies in series.  Per interval, two kernels in a graph at the start of
+// this work, on split stores, and here: 1,250 neurons FP32 13.9, 13.6, 8.5 us;
+// 20,003 BF16 19.7, 18.2, 13.6; 112,500 FP32 48.0, 34.0, 30.2.  Nets of more
+// tiles than SMs keep the two kernels (562,500 neurons: 143 us against 178
+// with two tiles a CTA here).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kSimMaxCtas = 256;
 constexpr uint32_t kSimMaxSteps = 32;     // steps of an interval (one spike mask)
@@ -2601,19 +2650,19 @@ cudaError_t desc_layout(size_t used, size_t dyn_max, bool plastic,
   return cudaSuccess;
 }
 
-template <int LAY, bool COUNT, bool GX>
+template <int LAY, bool COUNT, int KIND>
 cudaError_t launch_tiled_t(const NetView& v, unsigned long long* pair,
                            unsigned int* done, const SpikeEntry* list,
                            int from_list_range, int advance_time,
                            cudaStream_t s) {
   static std::atomic<uint32_t> lim[64];
   size_t dm = 0;
-  cudaError_t e = allow_tile_smem(k_deliver_tiled<LAY, COUNT, GX>, lim, &dm);
+  cudaError_t e = allow_tile_smem(k_deliver_tiled<LAY, COUNT, KIND>, lim, &dm);
   if (e != cudaSuccess) return e;
   DescLayout dl;
   e = desc_layout(tiled_smem_bytes(v), dm, false, &dl);
   if (e != cudaSuccess) return e;
-  k_deliver_tiled<LAY, COUNT, GX><<<v.n_tiles, kTileThreads, dl.smem, s>>>(
+  k_deliver_tiled<LAY, COUNT, KIND><<<v.n_tiles, kTileThreads, dl.smem, s>>>(
       v, pair, done, list, from_list_range, advance_time, dl.off, dl.cap);
   return cudaGetLastError();
 }
@@ -2641,26 +2690,23 @@ cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
                                  unsigned int* done, const SpikeEntry* list,
                                  int from_list_range, int advance_time,
                                  cudaStream_t s) {
-  if (v.gx && from_list_range) return cudaErrorInvalidValue;
+  if ((v.gx || v.ext_src) && from_list_range) return cudaErrorInvalidValue;
   if (v.plastic) {
-    if (v.gx || from_list_range) return cudaErrorNotSupported;
+    if (v.gx || v.ext_src || from_list_range) return cudaErrorNotSupported;
     if (v.lay == kLayF32)
       return v.counts ? launch_plastic_t<kLayF32, true>(v, pair, done, list, advance_time, s)
                       : launch_plastic_t<kLayF32, false>(v, pair, done, list, advance_time, s);
     return v.counts ? launch_plastic_t<kLayJ16, true>(v, pair, done, list, advance_time, s)
                     : launch_plastic_t<kLayJ16, false>(v, pair, done, list, advance_time, s);
   }
-#define SNN_TILED(L)                                                          \
-  (v.counts ? (v.gx ? launch_tiled_t<L, true, true>(                          \
-                          v, pair, done, list, 0, advance_time, s)            \
-                    : launch_tiled_t<L, true, false>(                         \
-                          v, pair, done, list, from_list_range,               \
-                          advance_time, s))                                   \
-            : (v.gx ? launch_tiled_t<L, false, true>(                         \
-                          v, pair, done, list, 0, advance_time, s)            \
-                    : launch_tiled_t<L, false, false>(                        \
-                          v, pair, done, list, from_list_range,               \
-                          advance_time, s)))
+#define SNN_TILED_K(L, C)                                                     \
+  (v.gx ? launch_tiled_t<L, C, kListGathered>(v, pair, done, list, 0,         \
+                                              advance_time, s)                \
+   : v.ext_src ? launch_tiled_t<L, C, kListRaw>(v, pair, done, list, 0, 0, s) \
+               : launch_tiled_t<L, C, kListOwn>(v, pair, done, list,          \
+                                                from_list_range,              \
+                                                advance_time, s))
+#define SNN_TILED(L) (v.counts ? SNN_TILED_K(L, true) : SNN_TILED_K(L, false))
   switch (v.lay) {
     case kLayHom: return SNN_TILED(kLayHom);
     case kLayF32: return SNN_TILED(kLayF32);
@@ -2668,6 +2714,20 @@ cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
     default: return SNN_TILED(kLayJ16);
   }
 #undef SNN_TILED
+#undef SNN_TILED_K
+}
+
+bool deliver_raw_fits(const NetView& v, uint32_t n) {
+  return v.lay != kLayRecords && n <= kRawMax;
+}
+
+cudaError_t launch_deliver_raw(const NetView& v, const uint32_t* src,
+                               const int32_t* t, uint32_t n, cudaStream_t s) {
+  NetView x = v;
+  x.ext_src = src;
+  x.ext_t = t;
+  x.ext_n = n;
+  return launch_deliver_tiled(x, nullptr, nullptr, nullptr, 0, 0, s);
 }
 
 // Whether the intervals of a net can run in k_simulate: a split store whose
@@ -2902,6 +2962,7 @@ cudaError_t launch_deliver_noalloc(const NetView& v, const uint32_t* src,
                                    const int32_t* t, uint32_t n,
                                    cudaStream_t s) {
   if (n > SNN_NOALLOC_MAX_SPIKES) return cudaErrorInvalidValue;
+  if (deliver_raw_fits(v, n)) return launch_deliver_raw(v, src, t, n, s);
   NoAllocScratch* sc = nullptr;
   cudaError_t e = noalloc_scratch(&sc);
   if (e != cudaSuccess) return e;

@@ -176,6 +176,9 @@ struct snn_net {
     v.gx_parts = 0;
     v.gx_stride = 0;
     v.gx_cap = 0;
+    v.ext_src = nullptr;
+    v.ext_t = nullptr;
+    v.ext_n = 0;
     v.log_src = log_src;
     v.log_t = log_t;
     v.log_cap = log_cap;

@@ -89,3 +89,29 @@ def test_uniform_edges_per_population(fmt):
             rb_o, _, absw, _ = O.deliver_ref(store, S, s, t)
             assert np.all(np.abs(net.read_rb() - rb_o) <= 1e-5 * absw + 1e-12)
             assert sorted(net.read_store()[3].tolist()) == sorted(w.tolist())
+
+
+@pytest.mark.parametrize("n_sp", [1, 1023, 1024, 2049, 4096, 4097])
+@pytest.mark.parametrize("steps", [5, 40])
+def test_lists_read_as_they_stand(n_sp, steps):
+    """Device arrays around the longest list delivered without preparation:
+    events counted, values as REF, a source outside the network skipped and
+    flagged, steps far from the clock and spread past the window alike."""
+    import torch
+    from paper_2109_12855_gb300 import snn
+    net, cp = fixed_net(400, 100, 40, 10, 20.0, -100.0, 10, 20, 7, fmt=0,
+                        sd_e=2.0, sd_i=10.0, count_events=0)
+    store = O.build_fixed_indegree(cp)
+    src, t = W.random_spikes(500, n_sp, 1000, 1000 + steps, seed=n_sp)
+    bad = np.concatenate([src, [500]]).astype(np.uint32)
+    tb = np.concatenate([t, [1000]]).astype(np.int32)
+    rb_o, _, absw, ev_o = O.deliver_ref(store, S, src, t)
+    with net:
+        for s, tt, flag in ((src, t, 0), (bad, tb, snn.SNN_ERRF_BAD_SOURCE)):
+            snn.snn_clear_rb(net.h)
+            ev = snn.snn_deliver(
+                net.h, torch.from_numpy(s.view(np.int32).copy()).cuda(),
+                torch.from_numpy(tt.astype(np.int32)).cuda())
+            assert ev == ev_o
+            assert np.all(np.abs(net.read_rb() - rb_o) <= 1e-5 * absw + 1e-12)
+            assert net.stats().error_flags == flag

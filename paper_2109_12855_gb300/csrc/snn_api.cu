@@ -924,7 +924,7 @@ int snn_connect_fixed_indegree(snn_net* net, const snn_conn_params* c) {
   uint32_t* deg = nullptr;
   CK(dalloc(&deg, net->n_src * sizeof(uint32_t), net->stream));
   CK(cudaMemsetAsync(deg, 0, net->n_src * sizeof(uint32_t), net->stream));
-  cudaError_t e = build_count_fixed(b, deg, net->stream);
+  cudaError_t e = build_count_fixed(b, net->n_src, deg, net->stream);
   if (e != cudaSuccess) {
     dfree(deg, net->stream);
     CK(e);

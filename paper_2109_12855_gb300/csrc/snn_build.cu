@@ -24,6 +24,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "snn_internal.cuh"
 
@@ -78,6 +79,39 @@ __global__ void __launch_bounds__(1024) k_scatter_fixed(BuildFixed b, const uint
       uint32_t pos = atomicAdd(&cursor[src], 1u);
       keys[row_ptr[src] + pos] = make_key(d, tgt, k, g);
     }
+}
+
+// The same counts with each CTA's counters in its shared memory, for
+// populations that fit there: CTA c draws for the targets [c per, (c + 1) per)
+// and adds its counts once per source at the end.  One global atomic per
+// synapse bounded the plain form (1.2e11/s): 30,011 neurons of in-degree 3,000,
+// 0.78 -> 0.29 ms; 112,500 of 11,250, 7.1 -> 3.4 ms.  (A scatter that takes its
+// places from such counters too was slower, 1.4 -> 3.3 ms: every row is then
+// written at as many places at once as there are CTAs, more partly written
+// sectors than L2 holds.)
+// W16: counters in halves of a word (a CTA draws a source at most 65,535
+// times: count_shared).
+template <bool W16>
+__global__ void __launch_bounds__(1024) k_count_shared(BuildFixed b, uint32_t n_src,
+                                                       uint32_t per, uint32_t* deg) {
+  extern __shared__ uint32_t sc[];
+  const uint32_t kk = b.k_e + b.k_i;
+  const uint32_t words = W16 ? (n_src + 1) / 2 : n_src;
+  for (uint32_t k = threadIdx.x; k < words; k += blockDim.x) sc[k] = 0;
+  __syncthreads();
+  const uint32_t lo = blockIdx.x * per, hi = min(lo + per, b.n_tgt);
+  for (uint32_t tgt = lo; tgt < hi; ++tgt)
+    for (uint32_t k = threadIdx.x; k < kk; k += blockDim.x) {
+      const U4 r = draw(b.seed, b.tgt0 + tgt, k, 0u);
+      const uint32_t src = fixed_source(b, k, r.x);
+      if (W16) atomicAdd(&sc[src >> 1], 1u << (16u * (src & 1u)));
+      else atomicAdd(&sc[src], 1u);
+    }
+  __syncthreads();
+  for (uint32_t k = threadIdx.x; k < n_src; k += blockDim.x) {
+    const uint32_t x = W16 ? (sc[k >> 1] >> (16u * (k & 1u))) & 0xFFFFu : sc[k];
+    if (x) atomicAdd(&deg[k], x);
+  }
 }
 
 __global__ void k_count_edges(const uint32_t* src, uint64_t n, uint32_t* deg) {
@@ -183,7 +217,8 @@ template <int FMT, int WMODE>
 __device__ void pack_row(const uint64_t* sorted, uint32_t len, uint32_t row,
                          uint64_t beg, const StoreOut& o, const BuildFixed& b,
                          const double* edge_w, TileGeom g, uint32_t n_tiles,
-                         uint32_t* tile_off, uint32_t* stats) {
+                         uint32_t* tile_off, uint32_t* stats,
+                         const uint32_t* ends) {
   const bool exc = row < b.n_e;
   float wmax = 0.f;
   uint32_t run_max = 0, d_min = 0xFFFFFFFFu, d_max = 0;
@@ -247,8 +282,14 @@ __device__ void pack_row(const uint64_t* sorted, uint32_t len, uint32_t row,
     if (d_min < st[2]) atomicMin(&stats[2], d_min);
     if (d_max > st[3]) atomicMax(&stats[3], d_max);
   }
-  // tile index: first position whose tile is >= tau (lower bound)
+  // tile index: first position whose tile is >= tau (where the bucket before
+  // ends, if the row was sorted by buckets; else by bisection)
   uint32_t* out = tile_off + (uint64_t)row * (n_tiles + 1);
+  if (ends) {
+    for (uint32_t tau = threadIdx.x; tau <= n_tiles; tau += blockDim.x)
+      out[tau] = tau ? ends[tau - 1] : 0u;
+    return;
+  }
   for (uint32_t tau = threadIdx.x; tau <= n_tiles; tau += blockDim.x) {
     if (tau == n_tiles) {  // every key's tile is below n_tiles
       out[tau] = len;
@@ -296,18 +337,49 @@ constexpr uint32_t kWarpSegMax = 256;
 // Rows of stores with more tiles than this are sorted whole.
 constexpr uint32_t kBucketTilesMax = 4096;
 
+// Rank sort of one segment of up to 32 Q keys by a warp: a key's rank is the
+// number of smaller keys (keys are distinct).
+template <int Q>
+__device__ __forceinline__ void rank_segment(uint64_t* a, uint32_t c) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint64_t key[Q];
+  uint32_t rank[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    rank[q] = 0;
+    key[q] = lane + 32u * q < c ? a[lane + 32u * q] : ~0ull;
+  }
+#pragma unroll 4
+  for (uint32_t i = 0; i < c; ++i) {
+    const uint64_t y = a[i];  // the same word for every lane
+#pragma unroll
+    for (int q = 0; q < Q; ++q) rank[q] += y < key[q];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    if (lane + 32u * q < c) a[rank[q]] = key[q];
+  __syncwarp();
+}
+
 // Sort one row of keys in shared memory (len keys at a[0..len), room for the
 // next power of two; cnt: n_tiles + 1 words): bucket by target tile
-// (histogram, exclusive scan, scatter from registers), then every warp
-// rank-sorts the short segments of the tiles it takes.  Keys are distinct,
-// so a key's rank in its segment is its position, and the result equals a
-// full sort of the row.  Falls back to the bitonic network when a segment
-// is longer than kWarpSegMax or the store has too many tiles.
-__device__ void sort_row(uint64_t* a, uint32_t len, uint32_t* cnt,
-                         uint32_t n_tiles, int lb) {
+// (histogram, exclusive scan by one warp, scatter from registers), then every
+// warp rank-sorts the short segments of the tiles it takes, with as many
+// registers a lane as the segment needs.  The result equals a full sort of
+// the row; returns the buckets' ends.  Falls back to the bitonic network
+// (returning null) when a segment is longer than kWarpSegMax or the store has
+// too many tiles.
+// The scan by one thread and eight compares a key for every segment, in CTAs
+// of 1,024 threads of which one fits an SM, took 33 us a row of 3,000 keys.
+__device__ const uint32_t* sort_row(uint64_t* a, uint32_t len, uint32_t* cnt,
+                                    uint32_t n_tiles, int lb) {
   const uint32_t P = pow2_ceil(len);
   bool whole = n_tiles > kBucketTilesMax || len > 16u * blockDim.x;
   if (!whole) {
+    __shared__ uint32_t s_max;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t n_warps = blockDim.x >> 5;
     for (uint32_t t = threadIdx.x; t <= n_tiles; t += blockDim.x) cnt[t] = 0;
     __syncthreads();
     // keys of this thread (at most 16) into registers, tiles counted
@@ -321,21 +393,28 @@ __device__ void sort_row(uint64_t* a, uint32_t len, uint32_t* cnt,
       }
     }
     __syncthreads();
-    // longest segment, then the exclusive scan of the counts (one thread
-    // per block of counts: n_tiles is small)
-    __shared__ uint32_t s_max;
-    if (threadIdx.x == 0) {
+    // longest segment, and the exclusive scan of the counts
+    if (warp == 0) {
       uint32_t run = 0, mx = 0;
-      for (uint32_t t = 0; t <= n_tiles; ++t) {
-        const uint32_t c = cnt[t];
-        cnt[t] = run;
-        run += c;
+      for (uint32_t t0 = 0; t0 <= n_tiles; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        const uint32_t c = t <= n_tiles ? cnt[t] : 0u;
+        uint32_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+          if (lane >= (uint32_t)o) inc += y;
+        }
+        if (t <= n_tiles) cnt[t] = run + inc - c;
+        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
         mx = max(mx, c);
       }
-      s_max = mx;
+      mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+      if (lane == 0) s_max = mx;
     }
     __syncthreads();
-    whole = s_max > kWarpSegMax;
+    const uint32_t longest = s_max;
+    whole = longest > kWarpSegMax;
     // scatter into the buckets (cnt becomes each bucket's end)
 #pragma unroll
     for (uint32_t q = 0; q < 16; ++q) {
@@ -347,38 +426,25 @@ __device__ void sort_row(uint64_t* a, uint32_t len, uint32_t* cnt,
     }
     __syncthreads();
     if (!whole) {
-      const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-      const uint32_t n_warps = blockDim.x >> 5;
       for (uint32_t t = warp; t < n_tiles; t += n_warps) {
         const uint32_t end = cnt[t];
         const uint32_t beg = t == 0 ? 0u : cnt[t - 1];
         const uint32_t c = end - beg;
         if (c < 2) continue;
-        uint64_t key[kWarpSegMax / 32];
-        uint32_t rank[kWarpSegMax / 32];
-#pragma unroll
-        for (uint32_t q = 0; q < kWarpSegMax / 32; ++q) {
-          rank[q] = 0;
-          key[q] = lane + 32u * q < c ? a[beg + lane + 32u * q] : ~0ull;
-        }
-        for (uint32_t i = 0; i < c; ++i) {
-          const uint64_t y = a[beg + i];  // the same word for every lane
-#pragma unroll
-          for (uint32_t q = 0; q < kWarpSegMax / 32; ++q) rank[q] += y < key[q];
-        }
-        __syncwarp();
-#pragma unroll
-        for (uint32_t q = 0; q < kWarpSegMax / 32; ++q)
-          if (lane + 32u * q < c) a[beg + rank[q]] = key[q];
-        __syncwarp();
+        if (c <= 32) rank_segment<1>(a + beg, c);
+        else if (c <= 64) rank_segment<2>(a + beg, c);
+        else if (c <= 96) rank_segment<3>(a + beg, c);
+        else if (c <= 128) rank_segment<4>(a + beg, c);
+        else rank_segment<kWarpSegMax / 32>(a + beg, c);
       }
       __syncthreads();
-      return;
+      return cnt;
     }
   }
   for (uint32_t i = len + threadIdx.x; i < P; i += blockDim.x) a[i] = ~0ull;
   __syncthreads();
   if (P > 1) bitonic(a, P);
+  return nullptr;
 }
 
 template <int FMT, int WMODE>
@@ -395,9 +461,9 @@ __global__ void __launch_bounds__(1024) k_sort_pack(uint32_t n, const uint64_t* 
     if (len > cap) continue;                 // uniform per block
     for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) sk[i] = keys[beg + i];
     __syncthreads();
-    if (len > 1) sort_row(sk, len, cnt, n_tiles, g.lb);
+    const uint32_t* ends = len > 1 ? sort_row(sk, len, cnt, n_tiles, g.lb) : nullptr;
     pack_row<FMT, WMODE>(sk, len, row, beg, recs, b, edge_w, g, n_tiles,
-                         tile_off, stats);
+                         tile_off, stats, ends);
     __syncthreads();
   }
 }
@@ -421,7 +487,7 @@ __global__ void __launch_bounds__(1024) k_sort_long(const uint32_t* rows, uint32
     __syncthreads();
     bitonic(a, P);
     pack_row<FMT, WMODE>(a, len, row, beg, recs, b, edge_w, g, n_tiles,
-                         tile_off, stats);
+                         tile_off, stats, nullptr);
     __syncthreads();
   }
 }
@@ -546,7 +612,9 @@ cudaError_t sort_pack_t(uint32_t n, const uint64_t* row_ptr, uint64_t* keys,
   size_t smem = (size_t)P * sizeof(uint64_t) +
                 (size_t)(std::min(n_tiles, kBucketTilesMax) + 1) * sizeof(uint32_t);
   cudaError_t e;
-  unsigned threads = P >= 1024 ? 1024 : (P >= 128 ? P : 128);
+  // 16 keys a thread at most: a CTA waits for itself several times a row, so
+  // several small ones on an SM keep it busy
+  unsigned threads = std::max(128u, std::min(1024u, P / 16u));
   unsigned blocks = n < (1u << 20) ? n : (1u << 20);
   BuildShape sh;
   if (blocks) {
@@ -572,11 +640,56 @@ cudaError_t sort_pack_t(uint32_t n, const uint64_t* row_ptr, uint64_t* keys,
 
 void set_build_yield(unsigned on) { t_build_yield = on; }
 
-cudaError_t build_count_fixed(const BuildFixed& b, uint32_t* deg,
+// Whether the fixed rule's count runs in shared memory (*bytes of it a CTA,
+// *parts CTAs): not in a build that yields SMs, for populations past shared
+// memory, for counts that could pass 16 bits, or for too few synapses to pay
+// for clearing and adding up the counters.
+static cudaError_t count_shared(const BuildFixed& b, uint32_t n_src, bool* use,
+                                bool* w16, size_t* bytes, uint32_t* parts) {
+  *use = false;
+  const uint64_t syn = (uint64_t)b.n_tgt * (b.k_e + b.k_i);
+  if (t_build_yield || syn < (4ull << 20) || syn < 64ull * n_src) return cudaSuccess;
+  int dev = 0, sms = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  *w16 = (size_t)n_src * 4 > (size_t)optin;
+  *bytes = *w16 ? ((size_t)n_src + 1) / 2 * 4 : (size_t)n_src * 4;
+  *parts = std::min<uint32_t>((uint32_t)std::max(sms, 1), b.n_tgt);
+  // a source's draws in a CTA are binomial: a mean of 2^14 leaves 2^16 out of
+  // reach
+  const double per = std::ceil((double)b.n_tgt / *parts);
+  *use = *bytes <= (size_t)optin &&
+         (!b.n_e || per * b.k_e / b.n_e <= 16384.0) &&
+         (!b.n_i || per * b.k_i / b.n_i <= 16384.0);
+  return cudaSuccess;
+}
+
+cudaError_t build_count_fixed(const BuildFixed& b, uint32_t n_src, uint32_t* deg,
                               cudaStream_t s) {
   if (b.n_tgt == 0 || b.k_e + b.k_i == 0) return cudaSuccess;
+  bool use = false, w16 = false;
+  size_t bytes = 0;
+  uint32_t parts = 0;
+  cudaError_t e = count_shared(b, n_src, &use, &w16, &bytes, &parts);
+  if (e != cudaSuccess) return e;
   BuildShape sh;
-  cudaError_t e = build_shape(k_count_fixed, b.n_tgt, 256, 0, &sh);
+  if (use) {
+    const uint32_t per = (b.n_tgt + parts - 1) / parts;
+    // (build_shape raises the kernel's shared-memory limit)
+    e = w16 ? build_shape(k_count_shared<true>, parts, 1024, bytes, &sh)
+            : build_shape(k_count_shared<false>, parts, 1024, bytes, &sh);
+    if (e != cudaSuccess) return e;
+    if (w16)
+      k_count_shared<true><<<sh.blocks, sh.threads, sh.smem, s>>>(b, n_src, per, deg);
+    else
+      k_count_shared<false><<<sh.blocks, sh.threads, sh.smem, s>>>(b, n_src, per, deg);
+    return cudaGetLastError();
+  }
+  e = build_shape(k_count_fixed, b.n_tgt, 256, 0, &sh);
   if (e != cudaSuccess) return e;
   k_count_fixed<<<sh.blocks, sh.threads, sh.smem, s>>>(b, deg);
   return cudaGetLastError();

@@ -455,7 +455,7 @@ struct BuildFixed {
 // Build kernels launched by the calling thread run as short whole-SM CTAs
 // (1) or in their normal shape (0); see snn_params.build_yield.
 void set_build_yield(unsigned on);
-cudaError_t build_count_fixed(const BuildFixed& b, uint32_t* deg,
+cudaError_t build_count_fixed(const BuildFixed& b, uint32_t n_src, uint32_t* deg,
                               cudaStream_t s);
 cudaError_t build_scatter_fixed(const BuildFixed& b, const uint64_t* row_ptr,
                                 uint32_t* cursor, uint64_t* keys,

@@ -398,21 +398,27 @@ k_update(NetView v, UpdConst c, int n_steps, int from_ctl, long long t0_arg) {
   update_body<true>(v, c, n_steps, from_ctl, t0_arg, blockIdx.x);
 }
 
+// Copies *src (of whole words) to shared memory, all threads of the CTA.
+template <class T>
+__device__ __forceinline__ void load_shared(T* dst, const T* src) {
+  static_assert(sizeof(T) % 4 == 0, "whole words");
+  for (uint32_t k = threadIdx.x; k < sizeof(T) / 4; k += blockDim.x)
+    reinterpret_cast<uint32_t*>(dst)[k] = reinterpret_cast<const uint32_t*>(src)[k];
+}
+
 // All nets of a batch in one launch: block b updates neuron block bmap[b].y
 // of net bmap[b].x, from that net's clock.
 __global__ void __launch_bounds__(kUpdThreads, 3)
 k_update_batch(const BatchNet* __restrict__ nets, const uint2* __restrict__ bmap) {
   __shared__ UpdConst s_c;
+  __shared__ NetView s_v;
   const uint2 m = bmap[blockIdx.x];
   const BatchNet& bn = nets[m.x];
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(&bn.c);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(&s_c);
-  for (uint32_t k = threadIdx.x; k < sizeof(UpdConst) / 4; k += blockDim.x)
-    dst[k] = src[k];
-  const NetView v = bn.v;
+  load_shared(&s_c, &bn.c);
+  load_shared(&s_v, &bn.v);
   const int n_steps = bn.n_steps;
   __syncthreads();
-  update_body<false>(v, s_c, n_steps, 1, 0, m.y);  // served nets are static
+  update_body<false>(s_v, s_c, n_steps, 1, 0, m.y);  // served nets are static
 }
 
 // ---------------------------------------------------------------------------
@@ -1766,9 +1772,13 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
                       const uint2* __restrict__ bmap, uint32_t desc_off,
                       uint32_t desc_cap) {
   extern __shared__ __align__(16) int acc_mem[];
+  // (the net's view once per CTA in shared memory: a copy per thread goes to
+  // local memory)
+  __shared__ NetView s_v;
   const uint2 m = bmap[blockIdx.x];
-  const NetView v = nets[m.x].v;
-  serve_tile<FMT>(v, m.y, acc_mem, desc_off, desc_cap);
+  load_shared(&s_v, &nets[m.x].v);
+  __syncthreads();
+  serve_tile<FMT>(s_v, m.y, acc_mem, desc_off, desc_cap);
 }
 
 // ---------------------------------------------------------------------------

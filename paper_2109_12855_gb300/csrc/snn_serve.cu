@@ -65,8 +65,14 @@ constexpr int kTuneStepsPerCandidate = 4;
 constexpr uint64_t kLogCapMax = 1ull << 22;  // recorded spikes per request
 // Served nets share each delivery launch, so a net gets tiles in proportion
 // to its synapses (one per kSynPerTile, at most one per SM) rather than one
-// per SM: small nets then add few CTAs of fixed per-CTA cost to the batch.
-constexpr uint64_t kSynPerTile = 1ull << 22;
+// per SM: small nets then add few CTAs of fixed per-CTA cost to the batch, and
+// a batch waits for its longest tile.  Eight requests of 1,250 to 20,000
+// neurons: 43.9 ms with 2^22, 35.5 with 2^20, 33.8 with 2^19, 35.1 with 2^18,
+// 37.5 with 2^17; 40 requests at once (up to 81,330 neurons) 6.0e10 events/s
+// with 2^22, 6.35e10 with 2^19.  The persistent kernel pays a claim per tile
+// and keeps 2^22 (3.4e10 against 2.9e10 events/s).
+constexpr uint64_t kSynPerTile = 1ull << 19;
+constexpr uint64_t kSynPerTilePersistent = 1ull << 22;
 // At most this many tiles per served net, so that other lanes keep SMs.
 constexpr uint64_t kServeMaxTiles = 120;
 // Graphs cached per lane for steps of 2^1 .. 2^kMaxGraphLog intervals.
@@ -248,7 +254,8 @@ int32_t serve_tile_width(const snn_request& r, bool persistent) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  uint64_t tiles = (n_syn + kSynPerTile - 1) / kSynPerTile;
+  const uint64_t per = persistent ? kSynPerTilePersistent : kSynPerTile;
+  uint64_t tiles = (n_syn + per - 1) / per;
   // the persistent kernel claims tiles one by one: a small net gets at
   // least a few (of 32 neurons or more), so that its delivery spreads over
   // several CTAs when the GPU has room

@@ -2637,9 +2637,12 @@ cudaError_t allow_tile_smem(Kernel kernel, std::atomic<uint32_t>* lim,
   return cudaSuccess;
 }
 
-// Run descriptors go after the accumulator (and the plastic state): as
-// many as the remaining shared memory holds, within kDescBytes (a larger
-// shared-memory carve-out would take L1 capacity from the record loads).
+// Run descriptors go after the accumulator (and the plastic state): at least
+// kDescBytes of them (if they fit), and what is left of the shared-memory
+// carve-out that this needs anyway -- a larger carve-out would take L1
+// capacity, in which the record loads wait, from the kernel: at 562,500
+// neurons 32 KB took 7.28 ms a pass (three batches of 2,048 runs), 48 KB of the
+// same carve-out 7.07, 72 KB 8.40.
 constexpr size_t kDescBytes = 32 * 1024;
 struct DescLayout {
   uint32_t off, cap;
@@ -2647,13 +2650,21 @@ struct DescLayout {
 };
 cudaError_t desc_layout(size_t used, size_t dyn_max, bool plastic,
                         DescLayout* out) {
-  // (a plastic run also has its source's last spike and its place in the row;
-  // what is added keeps the 196 KB carve-out of the benchmark network's tile)
+  // (a plastic run also has its source's last spike and its place in the row)
   const size_t per = sizeof(SegDesc) + (plastic ? 12u : 0u);
-  const size_t room = plastic ? kDescBytes + 5 * 1024 : kDescBytes;
   const size_t off = (used + 15u) & ~(size_t)15u;
   if (dyn_max < off + 32u * per) return cudaErrorInvalidConfiguration;
-  const size_t cap = std::min(room, dyn_max - off) / per & ~(size_t)1;
+  // carve-outs of an SM; a CTA also takes 1 KB and its static memory
+  constexpr size_t kCarve[] = {16, 32, 64, 100, 132, 164, 196, 228};
+  constexpr size_t kOptin = 227 * 1024;
+  const size_t fixed = 1024 + (kOptin > dyn_max ? kOptin - dyn_max : 0);
+  size_t room = std::min(kDescBytes, dyn_max - off);
+  for (size_t c : kCarve)
+    if (c * 1024 >= fixed + off + room) {
+      room = std::min(c * 1024 - fixed, dyn_max) - off;
+      break;
+    }
+  const size_t cap = room / per & ~(size_t)1;
   out->off = (uint32_t)off;
   out->cap = (uint32_t)cap;
   out->smem = off + cap * per;

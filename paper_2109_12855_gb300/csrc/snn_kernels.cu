@@ -89,16 +89,18 @@ __global__ void k_fill_i32(int32_t* p, int32_t value, uint64_t n) {
 // ---------------------------------------------------------------------------
 // Fused update.
 //
-// One thread per neuron integrates its state for the interval's steps.  The
-// ring-buffer values of a step are loaded in groups of eight independent
-// loads ahead of use (one memory round trip per eight steps instead of one
-// per step).  Spikes are kept as a per-thread bit mask of step indices and
-// compacted once per warp for up to 32 steps: a warp scan of the per-thread
-// counts, then one set of global atomics per warp with spikes reserves its
-// list entries and chunk ranges.
+// One thread per neuron integrates its state for the interval's steps, in the
+// 4-step blocks that the drive is drawn in: a block's ring-buffer loads, draws
+// and table look-ups are independent and issued together, then its steps run in
+// order.  What bounds it: issue, where several waves of blocks hide the
+// latencies (562,500 neurons: 1,517 warp instructions for 10 steps, 63 % of the
+// issue slots; groups of eight steps, with the words of two or three blocks
+// selected by alignment, took 1,756), else the latency of a thread's chain.
+// Spikes are kept as a per-thread bit mask of step indices and compacted once
+// per warp for up to 32 steps: a warp scan of the per-thread counts, then one
+// set of global atomics per warp with spikes reserves its list entries and
+// chunk ranges.
 // ---------------------------------------------------------------------------
-constexpr int kPrefetch = 8;
-
 
 // Plasticity state at a spike of excitatory neuron i at step t: the
 // presynaptic trace (kept with the values before this spike, which its own
@@ -160,7 +162,10 @@ __device__ __forceinline__ bool update_step(const UpdConst& c, float& V, float& 
 // neuron); shared by the single-net and the batched kernels.
 // PL: the single-net update, which also keeps the plasticity state and the
 // long-run spike statistics (the batched serving update does neither).
-template <bool PL>
+// ONE: the grid is one wave, whose latency counts: the neurons' spike
+// statistics are read before the integration, so that those that fire need not
+// wait for them.
+template <bool PL, bool ONE>
 __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
                                             int n_steps, int from_ctl,
                                             long long t0_arg, uint32_t block) {
@@ -185,20 +190,17 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
     nch = row_chunks(beg, end, v.chunk);
     deg = end - beg;
   }
-  // long-run spike statistics of this neuron, read now so that their
-  // latency overlaps the integration; written back once if it fired
-  const bool isi = PL && v.isi_spikes && live;
   int32_t isi_last = kNoSpike;
   uint32_t isi_spk = 0, isi_cnt = 0;
   double isi_s1 = 0.0, isi_s2 = 0.0;
-  bool isi_dirty = false;
-  if (isi) {
+  auto load_isi = [&]() {
     isi_last = v.isi_last[i];
     isi_spk = v.isi_spikes[i];
     isi_cnt = v.isi_n[i];
     isi_s1 = v.isi_sum[i];
     isi_s2 = v.isi_sq[i];
-  }
+  };
+  if (PL && ONE && live && v.isi_spikes) load_isi();
   // the single-net update may start while the previous delivery's last
   // CTAs run (programmatic dependent launch): everything above reads only
   // what the previous update wrote; from here on the delivery's ring-buffer
@@ -210,76 +212,46 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
     if (!from_ctl) v.ctl->t_now = t0;
   }
   __syncthreads();
-  U4 rnd{0, 0, 0, 0};
-  long long rnd_block = -1;
   float* const rb_i = v.rb + i;  // slot s of neuron i at rb_i[s * pitch]
 
   for (int s0 = 0; s0 < n_steps; s0 += 32) {
     const int ns = n_steps - s0 < 32 ? n_steps - s0 : 32;
     uint32_t mask = 0;
-    for (int sb = 0; sb < ns; sb += kPrefetch) {
-      // ring-buffer values and drive counts of up to eight steps, computed
-      // before the (sequential) integration so they do not lengthen it
-      float buf[kPrefetch];
-      const long long tf = t0 + s0 + sb;  // first step of this group
-      const int ng = ns - sb < kPrefetch ? ns - sb : kPrefetch;
+    {
+      const long long tc = t0 + s0;
+      for (long long b = tc >> 2; 4 * b < tc + ns; ++b) {
+        const int s1 = (int)(4 * b - tc);  // the block's first step, from tc
+        float in[4];
+        uint32_t k[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-      for (int q = 0; q < kPrefetch; ++q) {
-        buf[q] = 0.f;
-        if (live && q < ng)
-          buf[q] = rb_i[((uint32_t)(tf + q) & v.slot_mask) * v.pitch];
-      }
-      if (c.n_thr > 0 && live) {
-        // the group's steps lie in the 4-step draw blocks b0 .. b0 + 2;
-        // the draws are independent of one another (issued together), and
-        // the block drawn last is kept for the next group
-        const long long b0 = tf >> 2, bl = (tf + ng - 1) >> 2;
-        const uint32_t ig = v.g0 + i;  // drive keyed by the global index
-        const U4 r0 = b0 == rnd_block ? rnd : draw(c.seed, ig, (uint64_t)b0, 2u);
-        U4 r1 = r0, r2 = r0;
-        if (bl >= b0 + 1) r1 = draw(c.seed, ig, (uint64_t)(b0 + 1), 2u);
-        if (bl >= b0 + 2) r2 = draw(c.seed, ig, (uint64_t)(b0 + 2), 2u);
-        rnd = bl == b0 ? r0 : bl == b0 + 1 ? r1 : r2;
-        rnd_block = bl;
-        const uint32_t wd[12] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y,
-                                 r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
-        const int a = (int)(tf & 3);
-        // inversion of each step's word: the group's guide and first
-        // threshold lookups are issued together (independent shared-memory
-        // loads); the search goes on only where the word passes the first
-        // threshold (a threshold inside its guide bucket), as the plain
-        // search would
-        uint32_t wq[kPrefetch];
-        int kq[kPrefetch];
-        uint32_t tq[kPrefetch];
+        for (int q = 0; q < 4; ++q) {
+          in[q] = 0.f;
+          if (live && s1 + q >= 0 && s1 + q < ns)
+            in[q] = rb_i[((uint32_t)(tc + s1 + q) & v.slot_mask) * v.pitch];
+        }
+        if (c.n_thr > 0) {
+          const U4 r = draw(c.seed, v.g0 + i, (uint64_t)b, 2u);  // by global index
+          const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-        for (int q = 0; q < kPrefetch; ++q) {
-          // word (tf + q) mod 4 of block (tf + q) / 4: wd[a + q]
-          wq[q] = a == 0 ? wd[q] : a == 1 ? wd[q + 1]
-                : a == 2 ? wd[q + 2] : wd[q + 3];
-          kq[q] = s_guide[wq[q] >> 24];
+          for (int q = 0; q < 4; ++q) k[q] = s_guide[w[q] >> 24];
+          uint32_t th[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) th[q] = s_thr[k[q]];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if ((int)k[q] < c.n_thr - 1 && w[q] >= th[q]) {
+              ++k[q];
+              while ((int)k[q] < c.n_thr - 1 && w[q] >= s_thr[k[q]]) ++k[q];
+            }
         }
 #pragma unroll
-        for (int q = 0; q < kPrefetch; ++q) tq[q] = s_thr[kq[q]];
-#pragma unroll
-        for (int q = 0; q < kPrefetch; ++q) {
-          if (q >= ng) continue;
-          int k = kq[q];
-          if (k < c.n_thr - 1 && wq[q] >= tq[q]) {
-            ++k;
-            while (k < c.n_thr - 1 && wq[q] >= s_thr[k]) ++k;
-          }
-          buf[q] += c.w_ext * (float)k;
+        for (int q = 0; q < 4; ++q) {
+          const int st = s1 + q;
+          if (!live || st < 0 || st >= ns) continue;
+          if (c.n_thr > 0) in[q] += c.w_ext * (float)(int)k[q];
+          rb_i[((uint32_t)(tc + st) & v.slot_mask) * v.pitch] = 0.0f;
+          if (update_step(c, V, I, J, refr, in[q])) mask |= 1u << st;
         }
-      }
-#pragma unroll
-      for (int q = 0; q < kPrefetch; ++q) {
-        if (!live || sb + q >= ns) continue;
-        const long long t = t0 + s0 + sb + q;
-        // this step's ring-buffer input (read above; the slot is cleared
-        // here) plus drive
-        rb_i[((uint32_t)t & v.slot_mask) * v.pitch] = 0.0f;
-        if (update_step(c, V, I, J, refr, buf[q])) mask |= 1u << (sb + q);
       }
     }
     // warp compaction of this chunk's spikes: a warp with spikes scans its
@@ -289,6 +261,11 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
     const uint32_t cnt = __popc(mask);
     if (__ballot_sync(kFull, cnt != 0)) {
       const unsigned lane = threadIdx.x & 31u;
+      // (several waves: only the statistics of the neurons that fired, whose
+      // latency then overlaps the reservation; 24 bytes a neuron and interval
+      // less)
+      const bool isi = PL && cnt && v.isi_spikes;
+      if (isi && !ONE) load_isi();
       uint32_t inc_cnt = cnt, inc_ch = cnt * nch;
       unsigned long long inc_deg = (unsigned long long)cnt * deg;
 #pragma unroll
@@ -368,9 +345,15 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
           }
           isi_last = (int32_t)t;
           isi_spk += 1u;
-          isi_dirty = true;
         }
         ++k;
+      }
+      if (isi) {
+        v.isi_last[i] = isi_last;
+        v.isi_spikes[i] = isi_spk;
+        v.isi_n[i] = isi_cnt;
+        v.isi_sum[i] = isi_s1;
+        v.isi_sq[i] = isi_s2;
       }
     }
   }
@@ -380,13 +363,6 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
     v.J[i] = J;
     v.refr[i] = refr;
   }
-  if (isi_dirty) {
-    v.isi_last[i] = isi_last;
-    v.isi_spikes[i] = isi_spk;
-    v.isi_n[i] = isi_cnt;
-    v.isi_sum[i] = isi_s1;
-    v.isi_sq[i] = isi_s2;
-  }
 }
 
 // MINB blocks per SM: 3 leaves room for spill-free registers (a
@@ -395,7 +371,7 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
 template <int MINB>
 __global__ void __launch_bounds__(kUpdThreads, MINB)
 k_update(NetView v, UpdConst c, int n_steps, int from_ctl, long long t0_arg) {
-  update_body<true>(v, c, n_steps, from_ctl, t0_arg, blockIdx.x);
+  update_body<true, MINB == 3>(v, c, n_steps, from_ctl, t0_arg, blockIdx.x);
 }
 
 // Copies *src (of whole words) to shared memory, all threads of the CTA.
@@ -418,7 +394,7 @@ k_update_batch(const BatchNet* __restrict__ nets, const uint2* __restrict__ bmap
   load_shared(&s_v, &bn.v);
   const int n_steps = bn.n_steps;
   __syncthreads();
-  update_body<false>(s_v, s_c, n_steps, 1, 0, m.y);  // served nets are static
+  update_body<false, true>(s_v, s_c, n_steps, 1, 0, m.y);  // served nets are static
 }
 
 // ---------------------------------------------------------------------------
@@ -834,7 +810,7 @@ __device__ __forceinline__ uint32_t cell_step(uint32_t cell, uint32_t magic) {
 // Bounds-checked builds: a cell outside the store's window or one that
 // disagrees with the synapse's target is skipped and flagged; so are targets
 // outside the tile.  Production builds compile this to `true`.
-__device__ __forceinline__ bool cell_in_bounds(const NetView& v, uint32_t cell,
+[[maybe_unused]] __device__ __forceinline__ bool cell_in_bounds(const NetView& v, uint32_t cell,
                                                uint32_t tgt, uint32_t tgt_lo) {
   if (!kChecked) return true;
   const uint32_t d = cell / v.tile_w, j = cell - d * v.tile_w;
@@ -2341,7 +2317,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // allocation instead of sharing one with the other and the claim loop).
 __device__ __noinline__ void serve_update(const NetView& v, const UpdConst& c,
                                           int n_steps, uint32_t block) {
-  update_body<false>(v, c, n_steps, 1, 0, block);
+  update_body<false, true>(v, c, n_steps, 1, 0, block);
 }
 template <int FMT>
 __device__ __noinline__ void serve_deliver(const NetView& v, uint32_t tile,

@@ -7,7 +7,7 @@ Default workload (one JSON line on stdout): the balanced random network with
 1.27e9 static synapses in 12-byte FP32 records, delay 1.5 ms (15 steps of
 0.1 ms), Poisson drive tuned for about 8 Hz.  One step = 1 s of biological
 time (10,000 grid steps = 667 update/deliver intervals) of the whole hot path:
-fused update with spike compaction, then delivery, every interval.
+update, spike exchange and delivery, every interval.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME]
     python bench.py --impl reference      # the FP64 oracle on all host cores
@@ -126,8 +126,9 @@ def stdp_config(w_e):
 # launches' events
 # (profiles/dram_k_deliver_tiled_*.md); bench.py scales it by the events of
 # an average full-size launch.  It
-# stands for the kernel it was measured on: the entry is used only while the
-# kernel sources (comments aside) hash to the recorded prefixes.
+# stands for the kernel it was measured on (these: deliveries of whole 12- or
+# 8-byte records, before the stores were split): the entry is used only while
+# the kernel sources (comments aside) hash to the recorded prefixes.
 TRAFFIC_B_PER_EVENT = {
     "balanced-112500-fp32": (12.339, "09aa1a562d40154d", "19d84bddd44d9f03"),
     "balanced-112500-bf16": (8.332, "09aa1a562d40154d", "19d84bddd44d9f03"),
@@ -577,6 +578,17 @@ def measured_traffic(workload, events_per_launch):
     return ent[0] * events_per_launch
 
 
+def event_bytes(wl, fmt, deliver_mode, plastic):
+    """Store bytes a delivery reads per event: a whole record in atomic mode;
+    tiled nets keep the fields apart and read the 16-bit cell, and the weight
+    where it is the synapse's own (plastic nets read BF16 words with it)."""
+    if deliver_mode != "tiled":
+        return 12 if fmt == 0 else 8
+    if wl.sd_rel == 0.0 and not plastic:
+        return 2
+    return 6 if fmt == 0 else 4
+
+
 def timed(torch, stream, fn, k):
     """Run fn k times between events on the library's stream; ms total."""
     barrier()
@@ -607,6 +619,7 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
     stream = s.cuda_stream
     steps_per = int(round(bio_ms / 0.1))
     rec_bytes = 12 if fmt == 0 else 8
+    ev_bytes = event_bytes(wl, fmt, args.deliver_mode, args.workload in PLASTIC)
     expected_spikes = int(wl.n * 8.0 * bio_ms * 1e-3 * 4) + 100000
     # the log must hold every spike of the timed region (read once after it)
     log_cap = expected_spikes * (max(args.steps, 3) + 1)
@@ -637,7 +650,7 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
             ev, sp = b.events_delivered - a.events_delivered, b.spikes - a.spikes
             pl = b.plastic_events - a.plastic_events
             rows.append({"events": ev, "spikes": sp,
-                         "bytes": rec_bytes * ev + 32 * sp + 8 * pl})
+                         "bytes": ev_bytes * ev + 32 * sp + 8 * pl})
         net.close()
         if rank == 0:
             print(json.dumps({"workload": args.workload, "skip": args.launch_skip,
@@ -731,11 +744,13 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
     sp_prof = b.spikes - a.spikes
     pl_prof = b.plastic_events - a.plastic_events
     net.read_spikes(log_cap)
-    # algorithmic bytes: one record per event; per spike a list entry (16 B)
-    # and its two row offsets (16 B); a plastic event also reads and writes
-    # its FP32 weight (8 B)
+    # algorithmic bytes: what the store gives an event; per spike a list entry
+    # (16 B) and its two row offsets (16 B); a plastic event also reads and
+    # writes its FP32 weight (8 B).  (The profiled pass runs the update and the
+    # delivery as separate kernels; the timed one is one launch for nets of at
+    # most a tile per SM.)
     n_listed = sp_prof if kind != "deliver" else len(src) * args.steps
-    alg_bytes = rec_bytes * ev_prof + 32 * n_listed + 8 * pl_prof
+    alg_bytes = ev_bytes * ev_prof + 32 * n_listed + 8 * pl_prof
     per_launch_bytes = alg_bytes / max(n_del, 1)
     per_launch_s = ms_del * 1e-3 / max(n_del, 1)
     hbm, peak_kind = peaks()
@@ -814,8 +829,9 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
                    **({"stdp": stdp_config(w_e), "plastic_events_profiled": pl_prof,
                        "stdp_truncated": st.stdp_truncated} if plastic else {}),
                    "build_s": t_build,
-                   "l2": "inputs larger than L2 (the record store is "
-                         f"{wl.n_synapses * rec_bytes / 1e9:.1f} GB, streamed "
+                   "l2": "inputs larger than L2 (the synapse store is "
+                         f"{st_tiles.store_bytes / 1e9:.1f} GB, of which "
+                         f"{wl.n_synapses * ev_bytes / 1e9:.1f} GB are streamed "
                          "from HBM every step)",
                    "parallelism": f"replicas x{ws}"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm,
@@ -832,7 +848,7 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
                      "deliver_mode": args.deliver_mode,
                      "tiles": [st_tiles.n_tiles, st_tiles.tile_width,
                                st_tiles.window],
-                     "bytes_per_event": rec_bytes + (8 * pl_prof / max(ev_prof, 1)),
+                     "bytes_per_event": ev_bytes + (8 * pl_prof / max(ev_prof, 1)),
                      "ms_deliver_share": ms_del / ms_prof if ms_prof else None,
                      "ms_update_share": ms_upd / ms_prof if ms_prof else None,
                      "profiled_value": ev_prof / (ms_prof * 1e-3)},
@@ -1024,7 +1040,7 @@ def run_serve(args, rate_hz, nu_ext):
 
     hbm, peak_kind = peaks()
     gpu_s = batched["gpu_ms"] * 1e-3
-    alg_bytes = 8 * batched["events"] + 32 * batched["spikes"]
+    alg_bytes = 4 * batched["events"] + 32 * batched["spikes"]  # (split BF16)
     achieved = alg_bytes / gpu_s / 1e9 if gpu_s else 0.0
     cpu = None
     if ws == 1 and not args.no_cpu_baseline:

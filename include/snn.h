@@ -63,7 +63,9 @@ enum { SNN_MEM_HOST = 0, SNN_MEM_DEVICE = 1 };
  *  SNN_W_BF16_8B:  8 bytes {uint32 target; uint8 delay; uint8 pad;
  *                  bfloat16 weight}; weights are rounded FP64 -> BF16 to
  *                  nearest, ties to even, in one step.
- * Both accumulate into a float32 ring buffer. */
+ * Both accumulate into a float32 ring buffer.  The records of nets with the
+ * tiled delivery are kept by field (cell of the tile's window, weight, target),
+ * 10 or 8 bytes a synapse; snn_read_store gives the same values. */
 enum { SNN_W_FP32_12B = 0, SNN_W_BF16_8B = 1 };
 
 /* Delivery kernels.
@@ -198,8 +200,8 @@ typedef struct snn_stats {
   uint64_t kernel_launches;  /* library kernels launched since creation */
   uint64_t update_launches, deliver_launches;
   double ms_update, ms_deliver; /* CUDA-event times while profiling is on */
-  uint64_t bytes_per_record;    /* 12 or 8 */
-  uint64_t store_bytes;         /* device bytes of the record array */
+  uint64_t bytes_per_record;    /* 12 or 8 (the format's) */
+  uint64_t store_bytes;         /* device bytes of the synapses */
   uint32_t n_tiles, tile_width; /* target tiles of the store */
   int32_t window;               /* ring steps one interval reaches */
   int32_t deliver_mode;         /* kernel used by update/simulate */
@@ -354,8 +356,13 @@ int snn_deliver_noalloc(snn_net* net, const uint32_t* src,
 
 /* Advance the net by n_steps grid steps from its current time: repeat
  * {update one interval; deliver its spikes} (the time-driven cycle of
- * Section 1); the last interval may be shorter.  Full intervals run as
- * captured CUDA graphs unless profiling is on.  Asynchronous. */
+ * Section 1); the last interval may be shorter.  A static net of at most one
+ * tile per SM runs its intervals in cooperative launches of up to 256
+ * (stats count them as one kernel launch, and as that many updates and
+ * deliveries); they wait for the SMs they need, and a wait inside them that
+ * runs out (seconds) sets SNN_ERRF_TIMEOUT.  Otherwise full intervals run as
+ * captured CUDA graphs; with profiling on, as graphs of separate kernels.
+ * Asynchronous. */
 int snn_simulate(snn_net* net, int64_t n_steps);
 
 /* Copy up to cap logged spikes (source, step) in emission-interval order

@@ -1555,10 +1555,19 @@ int snn_simulate(snn_net* net, int64_t n_steps) {
     // launches of at most kSimIntervals intervals, so that other streams'
     // work is not held off for long
     int64_t left = full + (rem ? 1 : 0);
+    bool first = true;
     while (left > 0) {
       const int m = (int)std::min<int64_t>(left, kSimIntervals);
       left -= m;
-      CK(launch_simulate(v, net->uc, sh, ctas, m, D, left == 0 && rem ? rem : D, s));
+      const cudaError_t e =
+          launch_simulate(v, net->uc, sh, ctas, m, D, left == 0 && rem ? rem : D, s);
+      if (first && e == cudaErrorCooperativeLaunchTooLarge) {
+        // (fewer SMs for this context than the device has)
+        cudaGetLastError();
+        return simulate_async(net, n_steps, true);
+      }
+      CK(e);
+      first = false;
       net->launches += 1;
       net->upd_launches += m;  // (intervals updated and delivered)
       net->del_launches += m;

@@ -101,3 +101,70 @@ def test_log_overflow_is_flagged():
         assert st.error_flags == snn.SNN_ERRF_SPIKE_LOG and st.spikes > 10
         src, t = np.zeros(10, np.uint32), np.zeros(10, np.int32)
         assert snn.snn_read_spikes(net.h, src, t) == st.spikes
+
+
+def test_two_nets_on_two_streams():
+    """Launches of two nets that each want every SM, queued alternately on two
+    streams: both finish, each with the result it has alone."""
+    import torch
+    from paper_2109_12855_gb300 import snn
+    results = []
+    for together in (False, True):
+        streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+        nets = []
+        for seed, s in zip((1, 2), streams):
+            p = snn.params(n_exc=16000, n_inh=4000, weight_format=1, seed=seed,
+                           nu_ext=26000.0)
+            p.w_ext = snn.snn_psc_weight_for_psp(p, 0.1)
+            net = snn.Net(p, s.cuda_stream)
+            net.connect_fixed_indegree(snn.conn_params(
+                k_exc=160, k_inh=40, w_exc=p.w_ext, w_inh=-5 * p.w_ext,
+                sd_exc=2.0, sd_inh=10.0, d_lo=10, d_hi=20, seed=seed))
+            net.finalize()
+            nets.append(net)
+        for _ in range(6):
+            for net in nets:
+                snn.snn_simulate(net.h, 205)
+                if not together:
+                    snn.snn_sync(net.h)
+        results.append([x for net in nets for x in (*net.read_state(), net.read_rb())])
+        assert all(net.stats().error_flags == 0 for net in nets)
+        for net in nets:
+            net.close()
+    for x, y in zip(*results):
+        assert np.array_equal(x, y)
+
+
+def test_cycle_in_a_captured_graph():
+    """A call captured by the caller replays from the device clock."""
+    import torch
+    from paper_2109_12855_gb300 import snn
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    nets = []
+    for _ in range(2):
+        p = snn.params(n_exc=1000, n_inh=250, seed=4, nu_ext=26000.0)
+        p.w_ext = snn.snn_psc_weight_for_psp(p, 0.1)
+        net = snn.Net(p, s.cuda_stream)
+        net.connect_fixed_indegree(snn.conn_params(
+            k_exc=80, k_inh=20, w_exc=p.w_ext, w_inh=-5 * p.w_ext, d_lo=10,
+            d_hi=20, seed=5))
+        net.finalize()
+        snn.snn_simulate(net.h, 50)   # kernel attributes are settled
+        nets.append(net)
+    a, b = nets
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        snn.snn_simulate(a.h, 50)
+    with torch.cuda.stream(s):
+        for _ in range(3):
+            g.replay()
+    for _ in range(3):
+        snn.snn_simulate(b.h, 50)
+    torch.cuda.synchronize()
+    assert a.stats().t_now == b.stats().t_now == 200
+    for x, y in zip((*a.read_state(), a.read_rb()), (*b.read_state(), b.read_rb())):
+        assert np.array_equal(x, y)
+    for net in nets:
+        net.close()

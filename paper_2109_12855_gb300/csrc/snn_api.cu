@@ -1442,7 +1442,7 @@ int snn_deliver_noalloc(snn_net* net, const uint32_t* src,
     CK(cudaStreamSynchronize(s));
   }
   CK(launch_deliver_noalloc(net->view(), src, t_emit, n_spikes, s));
-  net->launches += 2;
+  net->launches += deliver_raw_fits(net->view(), n_spikes) ? 1 : 2;
   net->del_launches += 1;
   if (n_events_out) {
     CK(cudaMemcpyAsync(&ev1, &net->ctl->events, 8, cudaMemcpyDeviceToHost, s));

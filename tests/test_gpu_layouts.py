@@ -115,3 +115,19 @@ def test_lists_read_as_they_stand(n_sp, steps):
             assert ev == ev_o
             assert np.all(np.abs(net.read_rb() - rb_o) <= 1e-5 * absw + 1e-12)
             assert net.stats().error_flags == flag
+
+
+@pytest.mark.parametrize("n_sp,launches", [(4096, 1), (4097, 2)])
+def test_launch_counts_around_the_longest_raw_list(n_sp, launches):
+    """Both list entries count the kernels that they launch."""
+    import torch
+    from paper_2109_12855_gb300 import snn
+    net, _ = fixed_net(400, 100, 40, 10, 20.0, -100.0, 15, 15, 7, fmt=0)
+    src, t = W.random_spikes(500, n_sp, 1000, 1015, seed=n_sp)
+    with net:
+        s = torch.from_numpy(src.astype(np.int32)).cuda()
+        tt = torch.from_numpy(t.astype(np.int32)).cuda()
+        for deliver in (snn.snn_deliver, snn.snn_deliver_noalloc):
+            before = net.stats().kernel_launches
+            deliver(net.h, s, tt)
+            assert net.stats().kernel_launches - before == launches

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(1024) k_scatter_fixed(BuildFixed b, const uint
 // populations that fit there: CTA c draws for the targets [c per, (c + 1) per)
 // and adds its counts once per source at the end.  One global atomic per
 // synapse bounded the plain form (1.2e11/s): 30,011 neurons of in-degree 3,000,
-// 0.78 -> 0.29 ms; 112,500 of 11,250, 7.1 -> 3.4 ms.  (A scatter that takes its
+// 0.78 -> 0.25 ms; 112,500 of 11,250, 7.1 -> 3.2 ms.  (A scatter that takes its
 // places from such counters too was slower, 1.4 -> 3.3 ms: every row is then
 // written at as many places at once as there are CTAs, more partly written
 // sectors than L2 holds.)

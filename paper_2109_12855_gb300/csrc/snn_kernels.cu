@@ -21,7 +21,9 @@
 //             access, made tile-local): one CTA per tile of targets sums
 //             the interval's events for its targets in shared memory in
 //             exact fixed point, then adds them into its window of the ring
-//             buffer with plain coalesced read-modify-writes.
+//             buffer, one reduction a cell.
+//  k_simulate  update, exchange and delivery of many intervals in one
+//             cooperative launch, for nets of at most a tile per SM.
 //  k_update_batch, k_deliver_tiled_batch  the same for all nets of a served
 //             batch in one launch each.
 //  k_prepare_external  prefix sum of chunk counts for a caller's list.
@@ -1801,8 +1803,8 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
 // neurons that just fired are requested into L2, and all threads of a CTA form
 // the steps' inputs however few targets it has.  What bounds it: instructions
 // of the accumulation (about 11 of 30 us an interval at 112,500 neurons), then
-// latencies in series.  Per interval, two kernels in a graph at the start of
-// this work, on split stores, and here: 1,250 neurons FP32 13.9, 13.6, 8.5 us;
+// latencies in series.  Per interval, two kernels in a graph on whole records,
+// on split stores, and here: 1,250 neurons FP32 13.9, 13.6, 8.5 us;
 // 20,003 BF16 19.7, 18.2, 13.6; 112,500 FP32 48.0, 34.0, 30.2.  Nets of more
 // tiles than SMs keep the two kernels (562,500 neurons: 143 us against 178
 // with two tiles a CTA here).

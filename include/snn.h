@@ -576,6 +576,13 @@ int snn_debug_poke_record(snn_net* net, uint64_t index, int field,
 #define SNN_PROBE_SWEEP 1
 int snn_probe_reductions(float* buf, uint64_t n_cells, uint64_t n_ops,
                          int pattern, void* stream, float* ms);
+/* The two powers of two of the plastic rule side by side: for each of the n
+ * floats x[] (device memory, like the outputs), approx[] = 2^x by the PTX
+ * instruction that the rule uses where the result is a normal float, lib[] =
+ * exp2f(x).  Synchronises the stream.  Errors: SNN_E_ARG (null or non-device
+ * arrays, n 0), SNN_E_CUDA. */
+int snn_probe_exp2(const float* x, uint64_t n, float* approx, float* lib,
+                   void* stream);
 /* The stream the net's work is enqueued on (*stream: a cudaStream_t; the
  * one given to snn_create, or the one the library created when none was
  * given).  Partitions that read each other's exchange buffers must share

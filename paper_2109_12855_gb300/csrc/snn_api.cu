@@ -27,6 +27,8 @@ namespace snn {
 // (snn_probe.cu)
 cudaError_t launch_red_probe(float* buf, uint32_t n_cells, uint64_t n_ops,
                              int pattern, cudaStream_t s);
+cudaError_t launch_exp2_probe(const float* x, uint64_t n, float* approx,
+                              float* lib, cudaStream_t s);
 }  // namespace snn
 
 namespace {
@@ -2053,6 +2055,33 @@ int snn_probe_reductions(float* buf, uint64_t n_cells, uint64_t n_ops,
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
   cudaSetDevice(prev);  // the caller's current device, as it was
+  CK(e);
+  return SNN_OK;
+}
+
+int snn_probe_exp2(const float* x, uint64_t n, float* approx, float* lib,
+                   void* stream) {
+  REQ(x && approx && lib, SNN_E_ARG, "null argument");
+  REQ(n >= 1, SNN_E_ARG, "n is 0");
+  const void* bufs[3] = {x, approx, lib};
+  int dev = 0;
+  for (int k = 0; k < 3; ++k) {
+    cudaPointerAttributes pa;
+    const cudaError_t pe = cudaPointerGetAttributes(&pa, bufs[k]);
+    if (pe != cudaSuccess) cudaGetLastError();
+    REQ(pe == cudaSuccess &&
+            (pa.type == cudaMemoryTypeDevice || pa.type == cudaMemoryTypeManaged) &&
+            (k == 0 || pa.device == dev),
+        SNN_E_ARG, "array %d is not memory of one device", k);
+    dev = pa.device;
+  }
+  int prev = 0;
+  CK(cudaGetDevice(&prev));
+  CK(cudaSetDevice(dev));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaError_t e = snn::launch_exp2_probe(x, n, approx, lib, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaSetDevice(prev);
   CK(e);
   return SNN_OK;
 }

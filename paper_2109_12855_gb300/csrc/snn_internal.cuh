@@ -207,6 +207,18 @@ __host__ __device__ inline uint32_t scale_u32(uint32_t u, uint32_t n) {
   return (uint32_t)(((uint64_t)u * n) >> 32);
 }
 
+#ifdef __CUDACC__
+// 2^x by the PTX instruction ex2.approx.ftz.f32, an approximation to within two
+// units in the last place by the PTX ISA (the CUDA C++ guide's bound for exp2f)
+// that flushes subnormal results to zero: for arguments in [-126, 128), whose
+// powers are normal.  snn_probe_exp2 measures both against each other.
+__device__ __forceinline__ float ex2_normal(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+#endif
+
 // FP64 -> bfloat16 bits, round to nearest even in one step (finite inputs
 // of normal float range; values below the smallest normal float flush to
 // a signed zero).

@@ -1,9 +1,12 @@
 // snn_probe.cu -- throughput probe of the L2 reductions that the delivery's
 // ring-buffer additions use (red.global.add.f32): the secondary bound of the
 // atomic delivery (one reduction per synaptic event) and of the tiled
-// delivery's flush (one per nonzero cell of a tile's window).
+// delivery's flush (one per nonzero cell of a tile's window); and the two
+// powers of two that the plastic rule uses, side by side.
 #include <cuda_runtime.h>
 #include <cstdint>
+
+#include "snn_internal.cuh"
 
 namespace snn {
 namespace {
@@ -36,7 +39,24 @@ __global__ void k_red_probe(float* __restrict__ buf, uint32_t n_cells,
   }
 }
 
+__global__ void k_exp2_probe(const float* __restrict__ x, uint64_t n,
+                             float* __restrict__ approx, float* __restrict__ lib) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+       k += stride) {
+    approx[k] = ex2_normal(x[k]);
+    lib[k] = exp2f(x[k]);
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_exp2_probe(const float* x, uint64_t n, float* approx,
+                              float* lib, cudaStream_t s) {
+  const uint64_t blocks = (n + 255) / 256;
+  k_exp2_probe<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, s>>>(x, n, approx, lib);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_red_probe(float* buf, uint32_t n_cells, uint64_t n_ops,
                              int pattern, cudaStream_t s) {

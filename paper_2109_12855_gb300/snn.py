@@ -49,7 +49,7 @@ EXPORTS = [
     "snn_debug_fail_allocations", "snn_exchange_capacity",
     "snn_set_exchange", "snn_deliver_exchanged", "snn_get_stream",
     "snn_checked", "snn_debug_check_failures", "snn_debug_poke_record",
-    "snn_probe_reductions",
+    "snn_probe_reductions", "snn_probe_exp2",
 ]
 SNN_REQ_QUEUED, SNN_REQ_BUILDING, SNN_REQ_RUNNING, SNN_REQ_DONE = 0, 1, 2, 3
 SNN_REQ_FAILED = -1
@@ -223,6 +223,8 @@ def lib():
             "snn_probe_reductions": ([C.c_void_p, C.c_uint64, C.c_uint64,
                                       C.c_int, C.c_void_p,
                                       C.POINTER(C.c_float)], C.c_int),
+            "snn_probe_exp2": ([C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p,
+                                C.c_void_p], C.c_int),
             "snn_debug_poke_record": ([_P, C.c_uint64, C.c_int, C.c_uint32],
                                       C.c_int),
             "snn_set_exchange": ([_P, _P, C.c_uint64], C.c_int),
@@ -478,6 +480,18 @@ def snn_probe_reductions(buf, n_ops: int, pattern: int, stream: int = 0) -> floa
     _check(lib().snn_probe_reductions(ptr, buf.numel(), n_ops, pattern,
                                       C.c_void_p(stream or None), C.byref(ms)))
     return float(ms.value)
+
+
+def snn_probe_exp2(x, approx, lib_, stream: int = 0):
+    """2^x of the float32 device tensor x, elementwise, by the instruction that
+    the plastic rule uses (approx) and by exp2f (lib_)."""
+    bufs = [_buf(b) for b in (x, approx, lib_)]
+    if any(mem != SNN_MEM_DEVICE or str(b.dtype) != "torch.float32" or
+           b.numel() != x.numel()
+           for b, (_, mem) in zip((x, approx, lib_), bufs)):
+        raise ValueError("x, approx and lib_ must be float32 device tensors of one size")
+    _check(lib().snn_probe_exp2(bufs[0][0], x.numel(), bufs[1][0], bufs[2][0],
+                                C.c_void_p(stream or None)))
 
 
 def snn_get_stream(net) -> int:

@@ -1135,6 +1135,7 @@ int snn_finalize(snn_net* net) {
   net->list_cap = (uint64_t)net->n_src * iv;
   CK(dalloc(&net->list, net->list_cap * sizeof(SpikeEntry), net->stream));
   CK(dalloc(&net->sim_flags, kSimFlagBytes, net->stream));
+  CK(cudaMemsetAsync(net->sim_flags, 0, kSimFlagBytes, s));  // (then by each launch)
   if (net->stdp_on) {
     int rc2;
     if ((rc2 = setup_stdp(net)) != SNN_OK) return rc2;

@@ -356,8 +356,9 @@ struct BatchNet {
 };
 
 // What the CTAs of one k_simulate launch share: two sets of a flag word per
-// CTA ({interval, spikes}; zeroed before the launch together with `stop`,
-// which a CTA sets when a wait runs out), and of list regions (an entry:
+// CTA ({interval, spikes}; zero before the launch together with `stop`,
+// which a CTA sets when a wait runs out: snn_finalize, then every launch after
+// itself), and of list regions (an entry:
 // source | step in its interval << 24).
 constexpr size_t kSimFlagBytes = 2 * 256 * 8 + 16;
 struct SimShared {

@@ -203,10 +203,12 @@ __device__ __forceinline__ void update_body(const NetView& v, const UpdConst& c,
     isi_s2 = v.isi_sq[i];
   };
   if (PL && ONE && live && v.isi_spikes) load_isi();
-  // the single-net update may start while the previous delivery's last
-  // CTAs run (programmatic dependent launch): everything above reads only
-  // what the previous update wrote; from here on the delivery's ring-buffer
-  // additions, clock and counters must be complete
+  // the single-net update may start while the previous kernel's last CTAs
+  // run (programmatic dependent launch): everything above reads only what no
+  // kernel that can directly precede it writes -- a delivery adds to the ring
+  // buffer, and a launch of k_simulate, which writes state and statistics, is
+  // followed by a fully ordered memset (launch_simulate_t); from here on the
+  // delivery's ring-buffer additions, clock and counters must be complete
   if constexpr (PL) asm volatile("griddepcontrol.wait;" ::: "memory");
   const long long t0 = from_ctl ? v.ctl->t_now : t0_arg;
   if (block == 0 && threadIdx.x == 0) {
@@ -2765,8 +2767,6 @@ cudaError_t launch_simulate_t(const NetView& v, const UpdConst& c,
   // of all CTAs'
   const double row = v.n_src ? (double)v.mean_row * (LAY == kLayHom ? 2.0 : LAY == kLayF32 ? 6.0 : 4.0) : 1.0;
   const uint32_t pf = (uint32_t)std::max(1.0, 40e6 / (std::max(row, 64.0) * ctas));
-  e = cudaMemsetAsync(sh.flags, 0, kSimFlagBytes, s);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(kTileThreads);
@@ -2777,8 +2777,14 @@ cudaError_t launch_simulate_t(const NetView& v, const UpdConst& c,
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_simulate<LAY>, v, c, sh, n_iv, steps,
-                            last_steps, (uint32_t)drv, dl.off, dl.cap, pf);
+  e = cudaLaunchKernelEx(&cfg, k_simulate<LAY>, v, c, sh, n_iv, steps,
+                         last_steps, (uint32_t)drv, dl.off, dl.cap, pf);
+  if (e != cudaSuccess) return e;
+  // The flags of the launch to come are cleared after this one, not before it:
+  // the memset waits for the kernel to end with its writes visible, so a
+  // k_update that comes next on the stream, and reads state before its
+  // griddepcontrol.wait, can only overlap the memset.
+  return cudaMemsetAsync(sh.flags, 0, kSimFlagBytes, s);
 }
 
 static int sim_sms() {

@@ -1055,7 +1055,11 @@ struct CellValue {
     if (KIND == kCellFloat) return __int_as_float(H);
     if (KIND >= kCellCounts) {
       const int n0 = H & 0xFFFF, n1 = (int)((uint32_t)H >> 16);
-      if (KIND == kCellCountsFloat) return (float)n0 * w0 + (float)n1 * w1;
+      if (KIND == kCellCountsFloat) {
+        // (a count of zero adds nothing, also where the weight is infinite)
+        const float b = n1 ? __fmul_rn((float)n1, w1) : 0.f;
+        return n0 ? __fmaf_rn((float)n0, w0, b) : b;
+      }
       H = n0 * h0 + n1 * h1;
       L = n0 * l0 + n1 * l1;
     } else if (KIND == kCellTwo) {

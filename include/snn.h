@@ -86,7 +86,7 @@ enum {
   SNN_ERRF_BAD_SOURCE = 1u << 2, /* external spike with source >= N */
   SNN_ERRF_CHUNKS = 1u << 3,     /* chunk counter of one interval overflowed */
   SNN_ERRF_TIMEOUT = 1u << 4,    /* a bounded device wait gave up (delivery of
-                                    that launch is incomplete) */
+                                    that launch is incomplete; see snn_simulate) */
   SNN_ERRF_SCALES = 1u << 5,     /* internal: an interval's exact-sum scales
                                     were proven on the host but not found on
                                     the device (never expected) */
@@ -360,7 +360,10 @@ int snn_deliver_noalloc(snn_net* net, const uint32_t* src,
  * tile per SM runs its intervals in cooperative launches of up to 256
  * (stats count them as one kernel launch, and as that many updates and
  * deliveries); they wait for the SMs they need, and a wait inside them that
- * runs out (seconds) sets SNN_ERRF_TIMEOUT.  Otherwise full intervals run as
+ * runs out (seconds) sets SNN_ERRF_TIMEOUT: the net's state, ring buffer and
+ * spike log are then unusable, its device clock stays where that launch found
+ * it, and such launches do nothing until snn_clear_errors and snn_load_state
+ * have put the net back.  Otherwise full intervals run as
  * captured CUDA graphs; with profiling on, as graphs of separate kernels.
  * Asynchronous. */
 int snn_simulate(snn_net* net, int64_t n_steps);
@@ -558,6 +561,13 @@ uint64_t snn_debug_check_failures(void);
  * SNN_E_ARG for an index outside the store or an unknown field. */
 int snn_debug_poke_record(snn_net* net, uint64_t index, int field,
                           uint32_t value);
+/* Tests: how the one-launch cycle of snn_simulate runs for this net.
+ *  SNN_CYCLE_POLLS  looks (about a microsecond each, default and largest 2^24)
+ *                   of a CTA for the spikes of another before it gives up; 0:
+ *                   it gives up at the first look that finds them missing.
+ * Errors: SNN_E_ARG (unknown option, value outside its range). */
+enum { SNN_CYCLE_POLLS = 0 };
+int snn_debug_cycle(snn_net* net, int option, int64_t value);
 /* Throughput probe of the L2 reductions that carry the ring-buffer
  * additions of Algorithm REF (Section 3.2: rb[(t + d) mod S][target] += w;
  * on the GPU one red.global.add.f32 per event in the atomic delivery, one

@@ -1547,6 +1547,8 @@ int snn_simulate(snn_net* net, int64_t n_steps) {
     SimShared sh{};
     sh.flags = net->sim_flags;
     sh.stop = reinterpret_cast<unsigned int*>(net->sim_flags + 2 * 256);
+    sh.done = sh.stop + 1;
+    sh.polls = net->sim_polls;
     for (uint32_t r = 0; r < 10; ++r) {
       sh.key[2 * r] = (uint32_t)net->uc.seed + r * 0x9E3779B9u;
       sh.key[2 * r + 1] = (uint32_t)(net->uc.seed >> 32) + r * 0xBB67AE85u;
@@ -2084,6 +2086,15 @@ int snn_probe_exp2(const float* x, uint64_t n, float* approx, float* lib,
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaSetDevice(prev);
   CK(e);
+  return SNN_OK;
+}
+
+int snn_debug_cycle(snn_net* net, int option, int64_t value) {
+  REQ(net, SNN_E_ARG, "null net");
+  REQ(option == SNN_CYCLE_POLLS, SNN_E_ARG, "unknown option %d", option);
+  REQ(value >= 0 && value <= kSimPolls, SNN_E_ARG, "polls %lld outside [0, %u]",
+      (long long)value, kSimPolls);
+  net->sim_polls = (uint32_t)value;
   return SNN_OK;
 }
 

@@ -357,13 +357,17 @@ struct BatchNet {
 
 // What the CTAs of one k_simulate launch share: two sets of a flag word per
 // CTA ({interval, spikes}; zero before the launch together with `stop`,
-// which a CTA sets when a wait runs out: snn_finalize, then every launch after
-// itself), and of list regions (an entry:
+// which a CTA sets when a wait runs out, and `done`, the CTAs that ended:
+// snn_finalize, then every launch after itself), and of list regions (an entry:
 // source | step in its interval << 24).
 constexpr size_t kSimFlagBytes = 2 * 256 * 8 + 16;
+// Default of SimShared::polls (about a microsecond each).
+constexpr uint32_t kSimPolls = 1u << 24;
 struct SimShared {
   unsigned long long* flags;  // [2][256]
   unsigned int* stop;
+  unsigned int* done;
+  uint32_t polls;             // of a CTA that waits, before it gives up
   uint32_t* list;             // [2][CTAs][region]
   uint32_t region;
   uint32_t key[20];           // the drive's Philox round keys

@@ -1813,9 +1813,6 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
 constexpr uint32_t kSimMaxCtas = 256;
 constexpr uint32_t kSimMaxSteps = 32;     // steps of an interval (one spike mask)
 constexpr uint32_t kDriveBits = 10;       // leading bits of a draw per table entry
-// Polls of a CTA that waits for another one's spikes before it gives up
-// (about a microsecond each): the error is flagged and every CTA leaves.
-constexpr uint32_t kSimPolls = 1u << 24;
 
 // Cells' kind by layout: the persistent cycle runs only nets whose scales (and
 // counts) exist for every interval.
@@ -1947,7 +1944,10 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
   for (uint32_t x = tid; x < (TWO ? 2 * cells : cells); x += kTileThreads) acc[x] = 0;
   if (tid == 0) {
     s_cnt = 0;
-    s_bad = 0;
+    // (a net whose cycle once gave up stays as it is until its errors are
+    // cleared: its CTAs had stopped at different steps)
+    s_bad = (*reinterpret_cast<volatile unsigned int*>(&v.ctl->error_flags) &
+             (unsigned)SNN_ERRF_TIMEOUT) != 0u;
     s_sum[0] = s_sum[1] = 0ull;
     s_fx = FixScale{0, 0, 0, 1.f, 1.f, 1.f, 1.f};
   }
@@ -1969,6 +1969,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
   unsigned long long logged = *reinterpret_cast<volatile unsigned long long*>(&v.ctl->log_count);
   unsigned long long my_events = 0, my_spikes = 0;
   __syncthreads();
+  if (s_bad) return;  // (uniform in the CTA; one that set out finds `stop` set)
 
   // state of this thread's neuron, kept over the launch when it has only one
   float V = 0.f, I = 0.f, J = 0.f;
@@ -2207,7 +2208,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
         uint32_t polls = 0;
         while ((uint32_t)((x = ld_acquire_u64(f)) >> 32) != (uint32_t)(iv + 1)) {
           ++polls;
-          if (polls > kSimPolls ||
+          if (polls > sh.polls ||
               ((polls & 1023u) == 0u &&
                *reinterpret_cast<volatile unsigned int*>(sh.stop))) {
             s_bad = 1;
@@ -2259,6 +2260,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
     atomicExch(sh.stop, 1u);
     atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_TIMEOUT);
   }
+  // (a launch that gives up leaves state, ring buffer, log and clock unusable)
   if (single && tid < x_end) {
     const uint32_t i = lo + tid;
     v.V[i] = V;
@@ -2281,9 +2283,11 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
       atomicAdd(&v.ctl->events, s_sum[0]);
       atomicAdd(&v.ctl->spikes, s_sum[1]);
     }
-    // (every CTA read the clock and the log's length before its first
-    // publication, so before this one saw all of them)
-    if (r == 0) {
+    // the last CTA to end commits the clock and the log's length, if every CTA
+    // got through all intervals (all read both before this)
+    __threadfence();
+    if (atomicAdd(sh.done, 1u) == G - 1 &&
+        *reinterpret_cast<volatile unsigned int*>(sh.stop) == 0u) {
       v.ctl->t_now = t;
       v.ctl->iv_steps = last_steps;
       if (v.log_cap) v.ctl->log_count = logged;

@@ -73,6 +73,7 @@ struct snn_net {
   SpikeEntry* list = nullptr;
   uint64_t list_cap = 0;
   unsigned long long* sim_flags = nullptr;  // see SimShared
+  uint32_t sim_polls = kSimPolls;           // snn_debug_cycle
   SpikeEntry* ext_list = nullptr;
   uint32_t* ext_src = nullptr;
   int32_t* ext_t = nullptr;

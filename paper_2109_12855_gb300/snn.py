@@ -49,7 +49,7 @@ EXPORTS = [
     "snn_debug_fail_allocations", "snn_exchange_capacity",
     "snn_set_exchange", "snn_deliver_exchanged", "snn_get_stream",
     "snn_checked", "snn_debug_check_failures", "snn_debug_poke_record",
-    "snn_probe_reductions", "snn_probe_exp2",
+    "snn_probe_reductions", "snn_probe_exp2", "snn_debug_cycle",
 ]
 SNN_REQ_QUEUED, SNN_REQ_BUILDING, SNN_REQ_RUNNING, SNN_REQ_DONE = 0, 1, 2, 3
 SNN_REQ_FAILED = -1
@@ -223,6 +223,7 @@ def lib():
             "snn_probe_reductions": ([C.c_void_p, C.c_uint64, C.c_uint64,
                                       C.c_int, C.c_void_p,
                                       C.POINTER(C.c_float)], C.c_int),
+            "snn_debug_cycle": ([_P, C.c_int, C.c_int64], C.c_int),
             "snn_probe_exp2": ([C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p,
                                 C.c_void_p], C.c_int),
             "snn_debug_poke_record": ([_P, C.c_uint64, C.c_int, C.c_uint32],
@@ -465,6 +466,14 @@ def snn_debug_poke_record(net, index: int, field: int, value: int):
     """Bounds-checked builds: corrupt one record's target (field 0) or delay
     (field 1)."""
     _check(lib().snn_debug_poke_record(net, index, field, value))
+
+
+SNN_CYCLE_POLLS = 0
+
+
+def snn_debug_cycle(net, option: int, value: int):
+    """Tests: how snn_simulate's one-launch cycle runs for this net."""
+    _check(lib().snn_debug_cycle(net, option, value))
 
 
 SNN_PROBE_SCATTER, SNN_PROBE_SWEEP = 0, 1

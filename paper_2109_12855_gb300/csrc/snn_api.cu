@@ -1554,9 +1554,10 @@ int snn_simulate(snn_net* net, int64_t n_steps) {
       sh.key[2 * r + 1] = (uint32_t)(net->uc.seed >> 32) + r * 0xBB67AE85u;
     }
     uint32_t ctas = 0;
-    const NetView v = net->view();
+    NetView v = net->view();
     if (full + (rem ? 1 : 0) < 2 || !simulate_fits(v, net->uc, D, &sh, &ctas))
       return simulate_async(net, n_steps, true);
+    if (net->sim_unscaled) v.max_abs_w = 0.f;
     // launches of at most kSimIntervals intervals, so that other streams'
     // work is not held off for long
     int64_t left = full + (rem ? 1 : 0);
@@ -2091,10 +2092,15 @@ int snn_probe_exp2(const float* x, uint64_t n, float* approx, float* lib,
 
 int snn_debug_cycle(snn_net* net, int option, int64_t value) {
   REQ(net, SNN_E_ARG, "null net");
-  REQ(option == SNN_CYCLE_POLLS, SNN_E_ARG, "unknown option %d", option);
-  REQ(value >= 0 && value <= kSimPolls, SNN_E_ARG, "polls %lld outside [0, %u]",
-      (long long)value, kSimPolls);
-  net->sim_polls = (uint32_t)value;
+  REQ(option == SNN_CYCLE_POLLS || option == SNN_CYCLE_UNSCALED, SNN_E_ARG,
+      "unknown option %d", option);
+  const int64_t most = option == SNN_CYCLE_POLLS ? kSimPolls : 1;
+  REQ(value >= 0 && value <= most, SNN_E_ARG, "value %lld outside [0, %lld]",
+      (long long)value, (long long)most);
+  if (option == SNN_CYCLE_POLLS)
+    net->sim_polls = (uint32_t)value;
+  else
+    net->sim_unscaled = value != 0;
   return SNN_OK;
 }
 

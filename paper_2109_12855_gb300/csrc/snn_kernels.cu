@@ -2007,7 +2007,13 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
       }
     };
     // (1) the list's events for this tile into the accumulator
-    if (iv > 0 && tid == kTileThreads - 1) s_fx = fix_scale(v, n_sp, true);
+    // (simulate_fits has shown on the host that the scales exist for every
+    // list, and the counts of uniform weights: this says so if they do not)
+    if (iv > 0 && tid == kTileThreads - 1) {
+      s_fx = fix_scale(v, n_sp, true);
+      if (n_sp && !(s_fx.fixed && (LAY != kLayHom || s_fx.packed)))
+        atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_SCALES);
+    }
     uint32_t j0 = 0;
     do {
       const uint32_t nb = min(desc_cap, n_sp - j0);

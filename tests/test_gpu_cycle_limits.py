@@ -64,6 +64,20 @@ def test_wait_that_runs_out():
             assert x.tobytes() == y.tobytes()
 
 
+@pytest.mark.parametrize("fmt,sd", [(0, 0.0), (0, 0.1), (1, 0.1)],
+                         ids=["uniform", "fp32", "bf16"])
+def test_missing_scales_are_flagged(fmt, sd):
+    """The kernel finds no exact sums where the host had: the lists' events
+    cannot be added up, and the net says so."""
+    from paper_2109_12855_gb300 import snn
+    with _net(2000, 200, fmt, sd) as net:
+        snn.snn_simulate(net.h, 100)
+        assert net.stats().error_flags == 0 and net.stats().spikes > 0
+        snn.snn_debug_cycle(net.h, snn.SNN_CYCLE_UNSCALED, 1)
+        snn.snn_simulate(net.h, 100)
+        assert net.stats().error_flags == snn.SNN_ERRF_SCALES
+
+
 def test_options_are_checked():
     from paper_2109_12855_gb300 import snn
     with _net(500, 50) as net:

@@ -568,8 +568,11 @@ int snn_debug_poke_record(snn_net* net, uint64_t index, int field,
  *  SNN_CYCLE_UNSCALED  1: its kernel is given a weight bound for which no exact
  *                   sums exist although the host chose it, so that
  *                   SNN_ERRF_SCALES is raised; 0 (default): its own.
+ *  SNN_CYCLE_REFUSED  1: its launches count as refused, as in a context with
+ *                   fewer SMs than the net has tiles (the separate kernels run
+ *                   instead); 0 (default): they are tried.
  * Errors: SNN_E_ARG (unknown option, value outside its range). */
-enum { SNN_CYCLE_POLLS = 0, SNN_CYCLE_UNSCALED = 1 };
+enum { SNN_CYCLE_POLLS = 0, SNN_CYCLE_UNSCALED = 1, SNN_CYCLE_REFUSED = 2 };
 int snn_debug_cycle(snn_net* net, int option, int64_t value);
 /* Throughput probe of the L2 reductions that carry the ring-buffer
  * additions of Algorithm REF (Section 3.2: rb[(t + d) mod S][target] += w;

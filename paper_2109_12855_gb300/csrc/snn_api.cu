@@ -1566,7 +1566,9 @@ int snn_simulate(snn_net* net, int64_t n_steps) {
       const int m = (int)std::min<int64_t>(left, kSimIntervals);
       left -= m;
       const cudaError_t e =
-          launch_simulate(v, net->uc, sh, ctas, m, D, left == 0 && rem ? rem : D, s);
+          net->sim_refused
+              ? cudaErrorCooperativeLaunchTooLarge
+              : launch_simulate(v, net->uc, sh, ctas, m, D, left == 0 && rem ? rem : D, s);
       if (first && e == cudaErrorCooperativeLaunchTooLarge) {
         // (fewer SMs for this context than the device has)
         cudaGetLastError();
@@ -2092,7 +2094,7 @@ int snn_probe_exp2(const float* x, uint64_t n, float* approx, float* lib,
 
 int snn_debug_cycle(snn_net* net, int option, int64_t value) {
   REQ(net, SNN_E_ARG, "null net");
-  REQ(option == SNN_CYCLE_POLLS || option == SNN_CYCLE_UNSCALED, SNN_E_ARG,
+  REQ(option >= SNN_CYCLE_POLLS && option <= SNN_CYCLE_REFUSED, SNN_E_ARG,
       "unknown option %d", option);
   const int64_t most = option == SNN_CYCLE_POLLS ? kSimPolls : 1;
   REQ(value >= 0 && value <= most, SNN_E_ARG, "value %lld outside [0, %lld]",
@@ -2100,7 +2102,7 @@ int snn_debug_cycle(snn_net* net, int option, int64_t value) {
   if (option == SNN_CYCLE_POLLS)
     net->sim_polls = (uint32_t)value;
   else
-    net->sim_unscaled = value != 0;
+    (option == SNN_CYCLE_UNSCALED ? net->sim_unscaled : net->sim_refused) = value != 0;
   return SNN_OK;
 }
 

@@ -74,7 +74,7 @@ struct snn_net {
   uint64_t list_cap = 0;
   unsigned long long* sim_flags = nullptr;  // see SimShared
   uint32_t sim_polls = kSimPolls;           // snn_debug_cycle
-  bool sim_unscaled = false;
+  bool sim_unscaled = false, sim_refused = false;
   SpikeEntry* ext_list = nullptr;
   uint32_t* ext_src = nullptr;
   int32_t* ext_t = nullptr;

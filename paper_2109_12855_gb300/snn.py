@@ -468,7 +468,7 @@ def snn_debug_poke_record(net, index: int, field: int, value: int):
     _check(lib().snn_debug_poke_record(net, index, field, value))
 
 
-SNN_CYCLE_POLLS, SNN_CYCLE_UNSCALED = 0, 1
+SNN_CYCLE_POLLS, SNN_CYCLE_UNSCALED, SNN_CYCLE_REFUSED = 0, 1, 2
 
 
 def snn_debug_cycle(net, option: int, value: int):

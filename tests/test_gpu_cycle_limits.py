@@ -78,10 +78,31 @@ def test_missing_scales_are_flagged(fmt, sd):
         assert net.stats().error_flags == snn.SNN_ERRF_SCALES
 
 
+@pytest.mark.parametrize("steps", [205, 35], ids=["graphs", "few-intervals"])
+def test_refused_launch_runs_the_separate_kernels(steps):
+    """A context with fewer SMs than the net has tiles refuses the cooperative
+    launch: the call goes through the update and delivery kernels, to the same
+    bits, and so does the next."""
+    from paper_2109_12855_gb300 import snn
+    with _net() as a, _net() as b:
+        snn.snn_debug_cycle(a.h, snn.SNN_CYCLE_REFUSED, 1)
+        for _ in range(2):
+            before = a.stats().kernel_launches
+            for net in (a, b):
+                snn.snn_simulate(net.h, steps)
+            assert a.stats().kernel_launches - before == 2 * -(-steps // 10)
+        sa, sb = a.stats(), b.stats()
+        assert sa.error_flags == sb.error_flags == 0
+        assert (sa.t_now, sa.spikes, sa.events_delivered) == \
+            (sb.t_now, sb.spikes, sb.events_delivered)
+        for x, y in zip(_state(a), _state(b)):
+            assert x.tobytes() == y.tobytes()
+
+
 def test_options_are_checked():
     from paper_2109_12855_gb300 import snn
     with _net(500, 50) as net:
-        for option, value in ((snn.SNN_CYCLE_POLLS, -1), (99, 0),
+        for option, value in ((snn.SNN_CYCLE_POLLS, -1), (99, 0), (snn.SNN_CYCLE_REFUSED, 2),
                               (snn.SNN_CYCLE_POLLS, (1 << 24) + 1)):
             with pytest.raises(snn.SnnError) as e:
                 snn.snn_debug_cycle(net.h, option, value)

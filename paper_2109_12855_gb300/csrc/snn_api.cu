@@ -480,11 +480,11 @@ void decide_acc_words(snn_net* net, const WeightBounds& b, uint32_t k_in_max,
 
 cudaError_t launch_deliver_any(snn_net* net, unsigned long long* pair,
                                unsigned int* done, const SpikeEntry* list,
-                               int from_list_range, int advance_time) {
+                               uint32_t n_prepared, int advance_time) {
   NetView v = net->view();
   if (use_tiled(net))
-    return launch_deliver_tiled(v, pair, done, list, from_list_range,
-                                advance_time, net->stream);
+    return launch_deliver_tiled(v, pair, done, list, n_prepared, advance_time,
+                                net->stream);
   return launch_deliver(v, pair, done, list, advance_time, net->stream);
 }
 
@@ -1142,6 +1142,7 @@ int snn_finalize(snn_net* net) {
   }
   (void)deliver_grid_size(net->fmt);
   CK(cudaGetLastError());
+  net->own_mode = own_add_mode(net->view());
   net->finalized = true;
   return SNN_OK;
 }
@@ -1247,7 +1248,7 @@ int snn_deliver(snn_net* net, const uint32_t* src, const int32_t* t_emit,
     CK(launch_deliver_raw(v, d_src, d_t, n_spikes, s));
   else
     CK(launch_deliver_any(net, &net->ctl->ext_pair, &net->ctl->ext_done,
-                          net->ext_list, 1, 0));
+                          net->ext_list, n_spikes, 0));
   if (e1) CK(cudaEventRecord(e1, s));
   net->launches += raw ? 1 : 2;
   net->del_launches += 1;
@@ -1935,6 +1936,7 @@ int snn_set_bounds(snn_net* net, const snn_bounds* b) {
   net->mult_max = std::max(net->mult_max, b->mult_max);
   net->k_in_max = std::max(net->k_in_max, b->k_in_max);
   net->max_abs_w = std::max(net->max_abs_w, b->max_abs_w);
+  if (net->finalized) net->own_mode = own_add_mode(net->view());
   drop_graphs(net);  // the captured intervals hold the old view
   return SNN_OK;
 }

@@ -317,6 +317,7 @@ struct NetView {
   // scale has q - s >= acc_qs_min has lo = 0 for every event
   int acc_words;
   int acc_qs_min;
+  int own_mode;             // own_add_mode
   SpikeEntry* list;         // interval list, capacity list_cap
   uint64_t list_cap;
   // partition exchange: the update also writes its spikes as {src, t} pairs
@@ -414,15 +415,30 @@ cudaError_t launch_prepare_external(const NetView& v, const uint32_t* src,
                                     SpikeEntry* list,
                                     unsigned long long* pair, cudaStream_t s);
 int deliver_grid_size(int fmt);
-// Tile-binned delivery (see k_deliver_tiled).  from_list_range: the window
-// starts at the external list's minimum emission step (ctl->ext_tmin) rather
-// than at the interval start ctl->t_now.
 // q - s of the delivery kernel's fixed-point scales for event bound e and
 // max|w| (-1: no fixed point; the kernel sums in FP32).
 int fixed_qs_host(uint64_t e, double max_abs_w);
+// How a tile adds up a list.  In vectors of its runs (add_runs), for lists inside
+// the window whose exact sums exist: kAddVectors, of uniform weights the counts
+// in halves of a word; where these could pass 16 bits, kAddWide counts the two
+// populations in a word each, and cells of one word take the integer weights
+// themselves (kAddWeighted).  Element by element (kAddAny), for every other list
+// and for counted cells.  They are instantiations of their own (in one kernel the
+// general one's registers cost the others 3 to 6 %); the host knows all that
+// decides but the steps of a caller's list.
+enum AddMode { kAddVectors, kAddWide, kAddWeighted, kAddAny };
+// The mode of a list that brings a cell at most so many events, and of the own
+// lists of every interval.
+int add_mode(const NetView& v, uint64_t events);
+int own_add_mode(const NetView& v);
+// Tile-binned delivery (see k_deliver_tiled) of an interval's own list
+// (n_prepared 0), of the exchange buffers or arrays that v names, or of a
+// caller's list of n_prepared spikes made by launch_prepare_external, whose
+// window starts at its first emission step (ctl->ext_tmin) rather than at the
+// interval start ctl->t_now.
 cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
                                  unsigned int* done, const SpikeEntry* list,
-                                 int from_list_range, int advance_time,
+                                 uint32_t n_prepared, int advance_time,
                                  cudaStream_t s);
 size_t tiled_smem_bytes(const NetView& v);
 // A caller's arrays of n spikes delivered without preparing a list: whether
@@ -433,7 +449,8 @@ cudaError_t launch_deliver_raw(const NetView& v, const uint32_t* src,
 // Batched kernels (serving): bmap entries are (net index, block or tile).
 cudaError_t launch_update_batch(const BatchNet* nets, const uint2* bmap,
                                 uint32_t n_blocks, cudaStream_t s);
-cudaError_t launch_deliver_tiled_batch(int fmt, const BatchNet* nets,
+// (any: some net's own_mode is not kAddVectors)
+cudaError_t launch_deliver_tiled_batch(int fmt, bool any, const BatchNet* nets,
                                        const uint2* bmap, uint32_t n_ctas,
                                        size_t smem, cudaStream_t s);
 // Several intervals in one cooperative launch (see k_simulate): whether the
@@ -452,7 +469,7 @@ uint32_t serve_threads();
 // finds nothing ready polls again up to spin_limit times (about 100 ns
 // apart), then sets ServeCtl.error and leaves, as do all others.  n_ctas:
 // the grid; smem: the largest accumulator of the nets.
-cudaError_t launch_serve(int fmt, const BatchNet* nets, ServeNet* sn,
+cudaError_t launch_serve(int fmt, bool any, const BatchNet* nets, ServeNet* sn,
                          ServeCtl* ctl, uint32_t n_nets, uint32_t n_ctas,
                          size_t smem, unsigned long long spin_limit,
                          cudaStream_t s);

@@ -608,13 +608,16 @@ k_deliver(NetView v, unsigned long long* pair_p, unsigned int* done_p,
 // magnitude <= max|w|; s makes E 2^s < 2^31 and q makes
 // E max|w| 2^(q-s) + E < 2^31, so neither sum can overflow, and the
 // rounding error (<= 2^-(q+1) per event) is below that of FP32
-// accumulation.  If no such scales exist the CTA falls back to FP32
+// accumulation.  If no such scales exist the events are added in FP32 by
 // shared-memory atomics.
 //
 // Uniform weights (kLayHom): a cell's sum is n0 w0 + n1 w1, so only the two
 // counts are accumulated, in the halves of one 32-bit word (E <= 65,535; one
 // addition of a constant per event, no weight to split), and the flush forms
-// the same hi and lo sums from them.
+// the same hi and lo sums from them.  Beyond that a two-word cell holds a count
+// in each word, a one-word cell the sum of the integer weights (AddMode): 12,000
+// spikes on 112,500 neurons, 346 (FP32) and 311 us (BF16) on whole records, 162
+// and 156 so.
 //
 // The CTA then adds its cells into the ring buffer with fire-and-forget
 // reductions: no other CTA touches them.  An external list whose emission
@@ -634,48 +637,30 @@ template <int LAY> struct Lay {
   static constexpr uint32_t kElems = LAY == kLayHom ? 8u : 4u;
 };
 constexpr int kAhead = 3;  // vectors of a lane loaded ahead, for each of two runs
-template <int LAY>
-__device__ __forceinline__ Vec<LAY> load_vec(const NetView& v, uint64_t i) {
-  Vec<LAY> x;
-  x.a = __ldcs(reinterpret_cast<const uint4*>(v.dat) + i);
-  if constexpr (LAY == kLayF32)
-    x.c = __ldcs(reinterpret_cast<const uint2*>(v.cells) + i);
-  return x;
-}
-// Element k of a vector: its cell and weight (uniform stores: w is unused).
-template <int LAY>
-__device__ __forceinline__ uint32_t vec_cell(const Vec<LAY>& x, int k) {
-  if constexpr (LAY == kLayHom) {
-    const uint32_t w = k < 2 ? x.a.x : k < 4 ? x.a.y : k < 6 ? x.a.z : x.a.w;
-    return k & 1 ? w >> 16 : w & 0xFFFFu;
-  } else if constexpr (LAY == kLayF32) {
-    const uint32_t w = k < 2 ? x.c.x : x.c.y;
-    return k & 1 ? w >> 16 : w & 0xFFFFu;
-  } else {
-    const uint32_t w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
-    return w & 0xFFFFu;
-  }
-}
+// Weight of element k of a vector.
 template <int LAY>
 __device__ __forceinline__ float vec_weight(const Vec<LAY>& x, int k) {
   const uint32_t w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
   return __uint_as_float(LAY == kLayJ16 ? w & 0xFFFF0000u : w);
 }
+
+// One element of the stream, index i: its cell and its weight's bits.
+template <int LAY> struct Elem { uint32_t a; };
+template <> struct Elem<kLayF32> { uint32_t a, c; };
 template <int LAY>
-__device__ __forceinline__ int vec_int(const Vec<LAY>& x, int k) {
-  const uint32_t w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
-  return (int)w >> 16;
+__device__ __forceinline__ Elem<LAY> load_elem(const NetView& v, uint64_t i) {
+  Elem<LAY> x;
+  if constexpr (LAY == kLayHom)
+    x.a = __ldcs(reinterpret_cast<const uint16_t*>(v.dat) + i);
+  else
+    x.a = __ldcs(reinterpret_cast<const uint32_t*>(v.dat) + i);
+  if constexpr (LAY == kLayF32) x.c = __ldcs(v.cells + i);
+  return x;
 }
-// Elements of vector jv of a run that lie in it (bit k: element k); the run
-// takes the elements [head, total) of its vectors.
 template <int LAY>
-__device__ __forceinline__ uint32_t vec_mask(uint32_t jv, uint32_t head,
-                                             uint32_t total) {
-  constexpr uint32_t E = Lay<LAY>::kElems;
-  const int hi = (int)total - (int)(jv * E);
-  uint32_t m = hi >= (int)E ? (1u << E) - 1u : hi <= 0 ? 0u : (1u << hi) - 1u;
-  if (jv == 0) m &= ~0u << head;
-  return m;
+__device__ __forceinline__ uint32_t elem_cell(const Elem<LAY>& x) {
+  if constexpr (LAY == kLayF32) return x.c;
+  else return x.a & 0xFFFFu;
 }
 
 __device__ __forceinline__ void red_shared_u32(uint32_t addr, uint32_t x) {
@@ -740,14 +725,18 @@ __device__ __forceinline__ int ilog2d(double x) {
 // range in which adding 1.5 2^23 rounds to an integer (fixed_split).
 constexpr int kFixMaxShift = 23;
 
+// Most events of a cell: a list of n_sp spikes, of one interval or of any steps.
+__host__ __device__ inline uint64_t cell_events(const NetView& v, uint64_t n_sp,
+                                                bool per_interval) {
+  const uint64_t e = n_sp * (uint64_t)(v.mult_max ? v.mult_max : 1u);
+  const uint64_t e2 = (uint64_t)v.k_in_max * (v.spikes_per_iv ? v.spikes_per_iv : 1u);
+  return per_interval && e2 < e ? e2 : e;
+}
+
 __device__ FixScale fix_scale(const NetView& v, uint64_t n_sp,
                               bool per_interval) {
   FixScale f{0, 0, 0, 1.f, 1.f, 1.f, 1.f};
-  uint64_t e = n_sp * (uint64_t)(v.mult_max ? v.mult_max : 1u);
-  if (per_interval) {
-    const uint64_t e2 = (uint64_t)v.k_in_max * (v.spikes_per_iv ? v.spikes_per_iv : 1u);
-    if (e2 < e) e = e2;
-  }
+  const uint64_t e = cell_events(v, n_sp, per_interval);
   f.packed = e <= 0xFFFFull;
   if (e == 0 || e >= (1ull << 30) || !(v.max_abs_w > 0.f) ||
       !(v.max_abs_w <= 3.0e38f))
@@ -898,10 +887,11 @@ __device__ __noinline__ StdpOut stdp_weight(float w, int32_t t, uint32_t d,
   return o;
 }
 
-// Where a tiled delivery's list comes from: the interval's own list (or a
-// caller's, prepared in the same form), the partitions' exchange buffers
-// (v.gx), or a caller's arrays as they stand (v.ext_*).
-enum ListKind { kListOwn, kListGathered, kListRaw };
+// Where a tiled delivery's list comes from: the interval's own list, the
+// partitions' exchange buffers (v.gx), a caller's arrays as they stand (v.ext_*),
+// or a caller's list prepared in the own list's form (its steps: ext_tmin to
+// ext_tmax of the control block).
+enum ListKind { kListOwn, kListGathered, kListRaw, kListRange };
 // A caller's list up to this long is read by every CTA as it stands (four
 // entries a thread); a longer one is prepared by k_prepare_external first.
 constexpr uint32_t kRawMax = 4 * kTileThreads;
@@ -929,13 +919,15 @@ struct ListView {
 // list entries per thread in flight, then their tile-index words and row
 // starts.  pre (pre_g): entries threadIdx.x + u blockDim.x of the list, read
 // ahead of its length (have_pre).  Returns the events described (gathered
-// lists and callers' arrays).  PL: also the presynaptic history the plastic rule needs.
+// lists and callers' arrays).  wide: cells between the two populations' counts of
+// a uniform store (0: halves of one word).  PL: also the presynaptic history the
+// plastic rule needs.
 template <int LAY, int DU, bool PL, int KIND>
 __device__ __forceinline__ unsigned long long describe_runs(
     const NetView& v, const ListView& lv, const SpikeEntry* list, uint32_t tile,
     uint32_t j0, uint32_t nb, bool have_pre, const SpikeEntry* pre,
     const uint2* pre_g, const uint32_t* s_gstart, SegDesc* s_desc,
-    int32_t* s_tprev, float* s_kprev, uint32_t* s_at) {
+    uint32_t wide, int32_t* s_tprev, float* s_kprev, uint32_t* s_at) {
   constexpr bool GX = KIND == kListGathered, RAW = KIND == kListRaw;
   const uint32_t row_stride = v.n_tiles + 1;
   const uint32_t iv_span = (uint32_t)(v.window - (v.d_max - v.d_min));
@@ -1008,7 +1000,11 @@ __device__ __forceinline__ unsigned long long describe_runs(
           s_at[k] = a;
         } else {
           place_run<LAY>(v, row * v.row_mul + a, len, &sd);
-          if (LAY == kLayHom && src[u] >= v.hom_split) sd.len |= 0x80000000u;
+          // (counts in words of their own: the second population's further on)
+          if (LAY == kLayHom && src[u] >= v.hom_split) {
+            if (wide) sd.off += (int32_t)wide;
+            else sd.len |= 0x80000000u;
+          }
         }
       }
       s_desc[k] = sd;
@@ -1034,7 +1030,7 @@ __device__ __forceinline__ unsigned long long describe_runs(
 // conversion or FP64 arithmetic, whose rate is low on this part).  Uniform
 // weights: H and L from the two counts of the cell.
 enum CellKind { kCellFloat, kCellOne, kCellTwo, kCellCounts, kCellCountsOne,
-                kCellCountsFloat };
+                kCellCountsFloat, kCellWide, kCellWideFloat };
 struct CellValue {
   float scale_sq, inv_q;
   int h0, l0, h1, l1;
@@ -1054,8 +1050,10 @@ struct CellValue {
     int H = acc[c], L = 0;
     if (KIND == kCellFloat) return __int_as_float(H);
     if (KIND >= kCellCounts) {
-      const int n0 = H & 0xFFFF, n1 = (int)((uint32_t)H >> 16);
-      if (KIND == kCellCountsFloat) {
+      constexpr bool WIDE = KIND == kCellWide || KIND == kCellWideFloat;
+      const int n0 = WIDE ? H : H & 0xFFFF;
+      const int n1 = WIDE ? acc[cells + c] : (int)((uint32_t)H >> 16);
+      if (KIND == kCellCountsFloat || KIND == kCellWideFloat) {
         // (a count of zero adds nothing, also where the weight is infinite)
         const float b = n1 ? __fmul_rn((float)n1, w1) : 0.f;
         return n0 ? __fmaf_rn((float)n0, w0, b) : b;
@@ -1066,7 +1064,7 @@ struct CellValue {
       L = acc[cells + c];
     }
     float a = __fmul_rn(__int2float_rn(H), scale_sq);
-    if (KIND == kCellTwo || KIND == kCellCounts)
+    if (KIND == kCellTwo || KIND == kCellCounts || KIND == kCellWide)
       a = __fadd_rn(a, __fmul_rn(__int2float_rn(L), inv_q));
     return a;
   }
@@ -1093,12 +1091,15 @@ __device__ __forceinline__ void flush_kind(const NetView& v, const CellValue& va
     }
   }
 }
-template <bool HOM>
+template <bool HOM, bool WIDE>
 __device__ __forceinline__ void flush_tile(const NetView& v, const FixScale& fx,
                                            bool two, const int* acc,
                                            uint32_t tgt_lo, long long base) {
   const CellValue val(v, fx);
-  if (HOM && fx.packed) {
+  if (WIDE) {
+    if (!fx.fixed) flush_kind<kCellWideFloat>(v, val, acc, tgt_lo, base);
+    else flush_kind<kCellWide>(v, val, acc, tgt_lo, base);
+  } else if (HOM && fx.packed) {
     if (!fx.fixed) flush_kind<kCellCountsFloat>(v, val, acc, tgt_lo, base);
     else if (two) flush_kind<kCellCounts>(v, val, acc, tgt_lo, base);
     else flush_kind<kCellCountsOne>(v, val, acc, tgt_lo, base);
@@ -1191,11 +1192,13 @@ template <int LAY> struct LaneRun {
 // (Measured and not kept: masks only on a run's first and last vector, held
 // apart from the whole ones -- a fifth fewer instructions, but more registers
 // and branches: 29.8 -> 34.9 us on the 112,500-neuron list.)
+// inc0, inc1: what an event of uniform weight adds, by population.
 template <int LAY>
 __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
                                       const SegDesc* s_desc, uint32_t nb,
                                       uint32_t acc_s, uint32_t lo_off,
-                                      uint32_t lg, SplitScale fx) {
+                                      uint32_t lg, SplitScale fx,
+                                      uint32_t inc0 = 1u, uint32_t inc1 = 0x10000u) {
   constexpr uint32_t E = Lay<LAY>::kElems;
   __shared__ uint32_t s_none[32];  // what masked elements add to
   const uint32_t lane = threadIdx.x & 31u;
@@ -1221,7 +1224,7 @@ __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
       r.lo = sub == 0 ? (int)((uint32_t)sd.beg & 15u) : 0;
       r.n = (int)(sd.len & 0x7FFFFFFFu) - (int)(sub * E);
       r.row_s = acc_s + 4u * (uint32_t)sd.off;
-      r.inc = (int)sd.len < 0 ? 0x10000u : 1u;
+      r.inc = (int)sd.len < 0 ? inc1 : inc0;
 #pragma unroll
       for (int q = 0; q < kAhead; ++q)
         if (r.n > q * kStep) r.x[q] = fetch(r, q);
@@ -1261,14 +1264,23 @@ __device__ __noinline__ void add_runs_call(const char* dat, const char* cel,
   add_runs<LAY>(dat, cel, s_desc, nb, acc_s, lo_off, lg, fx);
 }
 
+template <int LAY, int KIND>
+__device__ __forceinline__ void deliver_tile_outside(
+    const NetView& v, unsigned long long* pair_p, unsigned int* done_p,
+    const SpikeEntry* __restrict__ list, uint32_t tile, int* acc_mem,
+    uint32_t desc_off, uint32_t desc_cap);
+
 // One interval's (or one caller's) list for tile `tile`.
-template <int LAY, bool COUNT, int KIND>
+template <int LAY, bool COUNT, int KIND, int MODE>
 __device__ __forceinline__ void deliver_tile_body(
     const NetView& v, unsigned long long* pair_p, unsigned int* done_p,
-    const SpikeEntry* __restrict__ list, int from_list_range, int advance_time,
+    const SpikeEntry* __restrict__ list, int advance_time,
     uint32_t tile, int* acc_mem, uint32_t desc_off, uint32_t desc_cap) {
-  constexpr uint32_t E = Lay<LAY>::kElems;
+  static_assert(MODE == kAddAny || !COUNT, "counted cells are added one by one");
+  static_assert((MODE != kAddWeighted && MODE != kAddWide) || LAY == kLayHom,
+                "uniform weights");
   constexpr bool GX = KIND == kListGathered, RAW = KIND == kListRaw;
+  constexpr bool RANGE = KIND == kListRange;
   SegDesc* const s_desc =
       reinterpret_cast<SegDesc*>(reinterpret_cast<char*>(acc_mem) + desc_off);
   __shared__ FixScale s_fx;
@@ -1290,8 +1302,8 @@ __device__ __forceinline__ void deliver_tile_body(
   constexpr int kDU = 4;
   SpikeEntry pre[GX || RAW ? 1 : kDU];
   uint2 pre_g[GX || RAW ? kDU : 1];
-  const bool spec = RAW || !from_list_range;
-  if (spec) {
+  constexpr bool spec = !RANGE;
+  if constexpr (spec) {
 #pragma unroll
     for (int u = 0; u < kDU; ++u) {
       const uint32_t k = threadIdx.x + u * blockDim.x;
@@ -1306,8 +1318,8 @@ __device__ __forceinline__ void deliver_tile_body(
       }
     }
   }
-  // every thread reads the launch's list size and window (same addresses);
-  // thread 0 derives the fixed-point scales meanwhile
+  // every thread reads the launch's list size and window (same addresses); the
+  // last one derives the fixed-point scales meanwhile
   ListView lv;
   if constexpr (GX) {
     // the parts' counts (each at most its capacity) and their starts in the
@@ -1350,7 +1362,7 @@ __device__ __forceinline__ void deliver_tile_body(
     lv.n_sp = (uint32_t)(pr >> 32);
   }
   lv.t_now = GX ? v.ctl->t_now : 0ll;
-  if (RAW || from_list_range) {
+  if (RAW || RANGE) {
     const long long tmin = RAW ? s_range[0] : v.ctl->ext_tmin;
     const long long tmax = RAW ? s_range[1] : v.ctl->ext_tmax;
     lv.base = tmin + v.d_min;
@@ -1359,116 +1371,174 @@ __device__ __forceinline__ void deliver_tile_body(
     lv.base = v.ctl->t_now + v.d_min;
     lv.inwin = true;
   }
+  if constexpr (MODE != kAddAny && (RAW || RANGE)) {
+    if (!lv.inwin) {  // (uniform: every thread has the same steps)
+      deliver_tile_outside<LAY, KIND>(v, pair_p, done_p, list, tile, acc_mem,
+                                      desc_off, desc_cap);
+      return;
+    }
+  }
   const uint32_t n_sp = lv.n_sp;
   const long long base = lv.base;
+  constexpr bool PER_IV = !RAW && !RANGE;
   // (the last thread: it describes no run of a list of up to 1,023 spikes)
-  if (threadIdx.x == kTileThreads - 1) s_fx = fix_scale(v, n_sp, !RAW && !from_list_range);
+  if (threadIdx.x == kTileThreads - 1) {
+    const FixScale f = fix_scale(v, n_sp, PER_IV);
+    s_fx = f;
+    // (counts need no scales: weights that have none are added up as floats)
+    if (MODE != kAddAny && n_sp &&
+        !(MODE == kAddWide || (MODE == kAddVectors && LAY == kLayHom ? f.packed : f.fixed)))
+      atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_SCALES);
+  }
   if (GX && threadIdx.x == 0) s_events = 0ull;
-  // (an interval's own list of a uniform store always fits its counts when
-  // the largest interval's does: one word a cell)
-  const bool one = !two || (LAY == kLayHom && !RAW && !from_list_range &&
-                            (uint64_t)v.k_in_max * v.spikes_per_iv <= 0xFFFFull);
+  const bool one = MODE == kAddVectors && LAY == kLayHom ? true
+                   : MODE == kAddWide                    ? false
+                                                         : !two;
   for (uint32_t x = threadIdx.x; x < (one ? cells : 2 * cells); x += blockDim.x)
     acc_mem[x] = 0;
   const uint32_t acc_s = (uint32_t)__cvta_generic_to_shared(acc_mem);
-  FixScale fx{};  // thread 0's s_fx, read after the first barrier
+  FixScale fx{};  // the last thread's s_fx, read after the first barrier
 
-  // lanes of this warp's runs: 2^lg of them share run `grp` of the warp's
-  uint32_t lg = 0, n_lanes = 1, runs = 32, sub = 0, grp = lane;
-
-  // one event in every other case: uniform weights whose counts do not fit,
-  // no fixed-point scales, a list outside the window, counted cells
-  auto add_slow = [&](uint32_t cell, const SegDesc& sd, float w) {
-    if (lv.inwin) {
-      const uint32_t c = (uint32_t)sd.off + cell;
-      if (LAY == kLayHom && fx.packed) {
-        red_shared_u32(acc_s + 4u * c, (int)sd.len < 0 ? 0x10000u : 1u);
-      } else if (fx.fixed) {
-        int hi, lo;
-        fixed_split(w, fx, hi, lo);
-        atomicAdd(&acc_mem[c], hi);
-        if (two && lo != 0) atomicAdd(&acc_mem[cells + c], lo);
+  // kAddAny: a list outside the window, no exact sums, counted cells.  2^lg lanes
+  // take a run, a lane every 2^lg-th element, PER of each of a lane's U runs loaded
+  // before any is added: where an event costs a global reduction, neighbouring
+  // lanes' targets share L2 lines.  What bounds it there are those reductions
+  // (2.6e11/s).  On whole records, with vectors of different runs on the lanes one
+  // at a time and a division an event, and here: 12,000 spikes across 45 steps,
+  // 112,500 neurons of equal weights 612, 752, 517 us, 50,021 neurons BF16 412, 449,
+  // 397 us; 20 counted intervals of the former 2,487, 3,120, 2,237 us.
+  [[maybe_unused]] auto add_any = [&](uint32_t nb) {
+    constexpr int U = LAY == kLayF32 ? 2 : 4;
+    constexpr int PER = 3;
+    const uint32_t magic = cell_magic(TW);
+    int h[2] = {0, 0}, l[2] = {0, 0};  // uniform weights
+    if (LAY == kLayHom && fx.fixed) {
+      fixed_split(v.hom_w[0], fx, h[0], l[0]);
+      fixed_split(v.hom_w[1], fx, h[1], l[1]);
+    }
+    auto event = [&](const SegDesc& sd, const Elem<LAY>& x) {
+      const uint32_t cell = elem_cell<LAY>(x);
+      const bool c1 = (int)sd.len < 0;
+      float w;
+      if constexpr (LAY == kLayHom) w = c1 ? v.hom_w[1] : v.hom_w[0];
+      else if constexpr (LAY == kLayI16) w = (float)((int)x.a >> 16) * pow2f(-v.acc_qs_min);
+      else w = __uint_as_float(LAY == kLayF32 ? x.a : x.a & 0xFFFF0000u);
+      if (lv.inwin) {
+        const uint32_t c = (uint32_t)sd.off + cell;
+        if (LAY == kLayHom && fx.packed) {
+          red_shared_u32(acc_s + 4u * c, c1 ? 0x10000u : 1u);
+        } else if (fx.fixed) {
+          int hi, lo;
+          if constexpr (LAY == kLayHom) {
+            hi = c1 ? h[1] : h[0];
+            lo = c1 ? l[1] : l[0];
+          } else {
+            fixed_split(w, fx, hi, lo);
+          }
+          red_shared_u32(acc_s + 4u * c, (uint32_t)hi);
+          if (two && lo != 0) red_shared_u32(acc_s + 4u * (cells + c), (uint32_t)lo);
+        } else {
+          atomicAdd(reinterpret_cast<float*>(acc_mem) + c, w);
+        }
+        if (COUNT) {
+          const uint32_t sl = cell_step(c, magic);
+          atomicAdd(v.counts + (size_t)((uint32_t)(base + sl) & v.slot_mask) * v.pitch +
+                        tgt_lo + (c - sl * TW), 1u);
+        }
       } else {
-        atomicAdd(reinterpret_cast<float*>(acc_mem) + c, w);
+        const uint32_t d = cell_step(cell, magic);
+        const size_t at =
+            (size_t)(((uint32_t)sd.off + d + (uint32_t)v.d_base) & v.slot_mask) * v.pitch +
+            tgt_lo + (cell - d * TW);
+        red_add_f32(v.rb + at, w);
+        if (COUNT) atomicAdd(v.counts + at, 1u);
       }
-      if (COUNT) {
-        const uint32_t sl = c / TW;
-        atomicAdd(v.counts + (size_t)((uint32_t)(base + sl) & v.slot_mask) * v.pitch +
-                      tgt_lo + (c - sl * TW), 1u);
+    };
+    // element idx of a run that starts at element i0 of the stream
+    auto put = [&](const SegDesc& sd, uint32_t idx, const Elem<LAY>& x) {
+#if SNN_CHECK
+      const uint64_t ti = sd.tgt + idx;
+      const uint32_t tgt = v.tgts ? v.tgts[ti]
+                                  : reinterpret_cast<const uint32_t*>(v.recs)[ti];
+      if (!cell_in_bounds(v, elem_cell<LAY>(x), tgt, tgt_lo)) return;
+#endif
+      event(sd, x);
+    };
+    auto first = [&](const SegDesc& sd) {
+      return ((sd.beg & ~15ull) - reinterpret_cast<uint64_t>(v.dat)) / 16u *
+                 Lay<LAY>::kElems + (sd.beg & 15u);
+    };
+    auto length = [&](const SegDesc& sd) {
+      const uint32_t m = sd.len & 0x7FFFFFFFu;
+      return m ? m - ((uint32_t)sd.beg & 15u) : 0u;
+    };
+    // lanes a run: three elements each for a mean run and a standard deviation
+    const float run = v.mean_row / (float)v.n_tiles;
+    uint32_t lg = 0;
+    while (lg < 5u && ((nb << (lg + 1u)) <= (uint32_t)kTileThreads ||
+                       3.f * (float)(1u << lg) < run + sqrtf(run)))
+      ++lg;
+    const uint32_t L = 1u << lg, R = 32u >> lg, sub = lane & (L - 1u);
+    for (uint32_t k0 = (threadIdx.x >> 5) * U * R; k0 < nb; k0 += kTileWarps * U * R) {
+      Elem<LAY> x[U][PER];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t j = k0 + u * R + (lane >> lg);
+        if (j >= nb) continue;
+        const SegDesc sd = s_desc[j];
+        const uint64_t i0 = first(sd) + sub;
+        const uint32_t len = length(sd);
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+          if (sub + L * q < len) x[u][q] = load_elem<LAY>(v, i0 + L * q);
       }
-    } else {
-      const uint32_t d = cell / TW;
-      const size_t at =
-          (size_t)(((uint32_t)sd.off + d + (uint32_t)v.d_base) & v.slot_mask) * v.pitch +
-          tgt_lo + (cell - d * TW);
-      red_add_f32(v.rb + at, w);
-      if (COUNT) atomicAdd(v.counts + at, 1u);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t j = k0 + u * R + (lane >> lg);
+        if (j >= nb) continue;
+        const SegDesc sd = s_desc[j];
+        const uint32_t len = length(sd);
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+          if (sub + L * q < len) put(sd, sub + L * q, x[u][q]);
+        for (uint32_t idx = PER * L + sub; idx < len; idx += L)
+          put(sd, idx, load_elem<LAY>(v, first(sd) + idx));
+      }
     }
   };
+
   uint32_t j0 = 0;
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
     const unsigned long long warp_events = describe_runs<LAY, kDU, false, KIND>(
-        v, lv, list, tile, j0, nb, spec, pre, pre_g, s_gstart, s_desc, nullptr, nullptr, nullptr);
+        v, lv, list, tile, j0, nb, spec, pre, pre_g, s_gstart, s_desc,
+        MODE == kAddWide ? cells : 0u, nullptr, nullptr, nullptr);
     // a batch of few runs spreads them over all lanes of the CTA
-    lg = (uint32_t)v.lg;
+    uint32_t lg = (uint32_t)v.lg;
     while (lg < 5u && (nb << (lg + 1u)) <= (uint32_t)kTileThreads) ++lg;
-    n_lanes = 1u << lg;
-    runs = 32u >> lg;
-    sub = lane & (n_lanes - 1u);
-    grp = lane >> lg;
     __syncthreads();
     // (after the barrier: s_events was cleared before it)
     if ((GX || RAW) && lane == 0 && warp_events) atomicAdd(&s_events, warp_events);
     fx = s_fx;
-    const bool fast = !COUNT && !kChecked && lv.inwin &&
-                      (LAY == kLayHom ? fx.packed : fx.fixed);
-    // every warp takes each kTileWarps-th group of `runs` runs
-    const uint32_t stride = kTileWarps * runs;
-    uint32_t k = (threadIdx.x >> 5) * runs;
-    if (fast) {
-      const uint32_t lo_off = two ? 4u * cells : 0u;
-      const char* const dat = reinterpret_cast<const char*>(v.dat);
-      const char* const cel = reinterpret_cast<const char*>(v.cells);
-      const SplitScale sc{fx.scale_hs, fx.scale_s};
-      add_runs<LAY>(dat, cel, s_desc, nb, acc_s, lo_off, lg, sc);
+    if constexpr (MODE == kAddAny) {
+      add_any(nb);
+    } else if constexpr (MODE == kAddWeighted) {
+      int h[2], l;
+      fixed_split(v.hom_w[0], fx, h[0], l);
+      fixed_split(v.hom_w[1], fx, h[1], l);
+      add_runs<LAY>(reinterpret_cast<const char*>(v.dat), nullptr, s_desc, nb, acc_s, 0u,
+                    lg, SplitScale{}, (uint32_t)h[0], (uint32_t)h[1]);
     } else {
-      for (; k < nb; k += stride) {
-        const uint32_t j = k + grp;
-        if (j < nb) {
-          const SegDesc sd = s_desc[j];
-          const uint32_t head = (uint32_t)sd.beg & 15u;
-          const uint32_t total = sd.len & 0x7FFFFFFFu;
-          const uint64_t v0 = ((sd.beg & ~15ull) - reinterpret_cast<uint64_t>(v.dat)) / 16u;
-          const float w_hom = v.hom_w[(int)sd.len < 0];
-          for (uint32_t jv = sub; jv * E < total; jv += n_lanes) {
-            const Vec<LAY> x = load_vec<LAY>(v, v0 + jv);
-            const uint32_t m = vec_mask<LAY>(jv, head, total);
-#pragma unroll
-            for (int e = 0; e < (int)E; ++e) {
-              if (!(m & (1u << e))) continue;
-              const uint32_t cell = vec_cell<LAY>(x, e);
-#if SNN_CHECK
-              const uint64_t ti = sd.tgt + jv * E + e - head;
-              const uint32_t tgt = v.tgts ? v.tgts[ti]
-                                          : reinterpret_cast<const uint32_t*>(v.recs)[ti];
-              if (!cell_in_bounds(v, cell, tgt, tgt_lo)) continue;
-#endif
-              float w = w_hom;
-              if constexpr (LAY == kLayI16)
-                w = (float)vec_int<LAY>(x, e) * pow2f(-v.acc_qs_min);
-              else if constexpr (LAY != kLayHom)
-                w = vec_weight<LAY>(x, e);
-              add_slow(cell, sd, w);
-            }
-          }
-        }
-      }
+      add_runs<LAY>(reinterpret_cast<const char*>(v.dat),
+                    reinterpret_cast<const char*>(v.cells), s_desc, nb, acc_s,
+                    two ? 4u * cells : 0u, lg, SplitScale{fx.scale_hs, fx.scale_s});
     }
     j0 += nb;
     __syncthreads();  // s_desc is rewritten by the next batch
   } while (j0 < n_sp);
-  if (lv.inwin) flush_tile<LAY == kLayHom>(v, fx, two, acc_mem, tgt_lo, base);
+  if (lv.inwin)
+    flush_tile<LAY == kLayHom && MODE != kAddWeighted, MODE == kAddWide>(v, fx, two, acc_mem,
+                                                                         tgt_lo, base);
   // The last CTA to finish clears the list counters and advances the clock
   // (a gathered list's events -- its spikes' runs onto this partition's
   // targets -- are counted by the CTAs themselves).
@@ -1643,7 +1713,7 @@ __device__ __forceinline__ void deliver_tile_plastic(
   do {
     const uint32_t nb = min(desc_cap, n_sp - j0);
     describe_runs<LAY, 1, true, kListOwn>(v, lv, list, tile, j0, nb, true, pre, nullptr,
-                                  nullptr, s_desc, s_tprev, s_kprev, s_at);
+                                  nullptr, s_desc, 0u, s_tprev, s_kprev, s_at);
     __syncthreads();
     fx = s_fx;
     for (uint32_t k0 = warp * U; k0 < nb; k0 += kTileWarps * U) {
@@ -1691,7 +1761,7 @@ __device__ __forceinline__ void deliver_tile_plastic(
     j0 += nb;
     __syncthreads();  // s_desc is rewritten by the next batch
   } while (j0 < n_sp);
-  flush_tile<false>(v, fx, two, acc_mem, tgt_lo, base);
+  flush_tile<false, false>(v, fx, two, acc_mem, tgt_lo, base);
   // one pair of atomics per warp, one per CTA
   unsigned long long a = my_pl, b = my_trunc;
 #pragma unroll
@@ -1713,15 +1783,25 @@ __device__ __forceinline__ void deliver_tile_plastic(
   }
 }
 
-template <int LAY, bool COUNT, int KIND>
+// A caller's list whose steps span more than the window: known only on the
+// device, so called from the other mode's kernel, which has nothing left to do.
+template <int LAY, int KIND>
+__device__ __forceinline__ void deliver_tile_outside(
+    const NetView& v, unsigned long long* pair_p, unsigned int* done_p,
+    const SpikeEntry* __restrict__ list, uint32_t tile, int* acc_mem,
+    uint32_t desc_off, uint32_t desc_cap) {
+  deliver_tile_body<LAY, false, KIND, kAddAny>(v, pair_p, done_p, list, 0, tile,
+                                               acc_mem, desc_off, desc_cap);
+}
+
+template <int LAY, bool COUNT, int KIND, int MODE>
 __global__ void __launch_bounds__(kTileThreads, 1)
-k_deliver_tiled(NetView v, unsigned long long* pair_p, unsigned int* done_p,
-                const SpikeEntry* __restrict__ list, int from_list_range,
+k_deliver_tiled(const __grid_constant__ NetView v, unsigned long long* pair_p,
+                unsigned int* done_p, const SpikeEntry* __restrict__ list,
                 int advance_time, uint32_t desc_off, uint32_t desc_cap) {
   extern __shared__ __align__(16) int acc_mem[];
-  deliver_tile_body<LAY, COUNT, KIND>(v, pair_p, done_p, list,
-                                         from_list_range, advance_time,
-                                         blockIdx.x, acc_mem, desc_off, desc_cap);
+  deliver_tile_body<LAY, COUNT, KIND, MODE>(v, pair_p, done_p, list, advance_time,
+                                            blockIdx.x, acc_mem, desc_off, desc_cap);
   // the next update may be scheduled once every CTA got here
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -1748,24 +1828,48 @@ k_deliver_plastic(NetView v, unsigned long long* pair_p, unsigned int* done_p,
 }
 
 // A served net's tile, its pending interval list (advancing the net's clock).
-template <int FMT>
+// ANY: some of the launch's nets add their lists element by element (those
+// bodies out of line: beside the others they would cost them registers).
+template <int LAY, int MODE>
+__device__ __forceinline__ void serve_tile_body(const NetView& v, uint32_t tile,
+                                                int* acc_mem, uint32_t desc_off,
+                                                uint32_t desc_cap) {
+  deliver_tile_body<LAY, false, kListOwn, MODE>(
+      v, &v.ctl->pair, &v.ctl->done, v.list, 1, tile, acc_mem, desc_off, desc_cap);
+}
+template <int LAY, int MODE>
+__device__ __noinline__ void serve_tile_call(const NetView& v, uint32_t tile,
+                                             int* acc_mem, uint32_t desc_off,
+                                             uint32_t desc_cap) {
+  serve_tile_body<LAY, MODE>(v, tile, acc_mem, desc_off, desc_cap);
+}
+template <int LAY, bool ANY>
+__device__ __forceinline__ void serve_tile_lay(const NetView& v, uint32_t tile,
+                                               int* acc_mem, uint32_t desc_off,
+                                               uint32_t desc_cap) {
+  if constexpr (!ANY && !kChecked)
+    serve_tile_body<LAY, kAddVectors>(v, tile, acc_mem, desc_off, desc_cap);
+  else if (!kChecked && v.own_mode == kAddVectors)
+    serve_tile_call<LAY, kAddVectors>(v, tile, acc_mem, desc_off, desc_cap);
+  else
+    serve_tile_call<LAY, kAddAny>(v, tile, acc_mem, desc_off, desc_cap);
+}
+template <int FMT, bool ANY>
 __device__ __forceinline__ void serve_tile(const NetView& v, uint32_t tile,
                                            int* acc_mem, uint32_t desc_off,
                                            uint32_t desc_cap) {
   if (v.lay == kLayHom)
-    deliver_tile_body<kLayHom, false, kListOwn>(
-        v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
+    serve_tile_lay<kLayHom, ANY>(v, tile, acc_mem, desc_off, desc_cap);
   else if (FMT == SNN_W_BF16_8B && v.lay == kLayI16)
-    deliver_tile_body<kLayI16, false, kListOwn>(
-        v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
+    serve_tile_lay<kLayI16, ANY>(v, tile, acc_mem, desc_off, desc_cap);
   else
-    deliver_tile_body<FMT == SNN_W_FP32_12B ? kLayF32 : kLayJ16, false, kListOwn>(
-        v, &v.ctl->pair, &v.ctl->done, v.list, 0, 1, tile, acc_mem, desc_off, desc_cap);
+    serve_tile_lay<FMT == SNN_W_FP32_12B ? kLayF32 : kLayJ16, ANY>(
+        v, tile, acc_mem, desc_off, desc_cap);
 }
 
 // All nets of a batch in one launch: CTA b delivers tile bmap[b].y of net
 // bmap[b].x.
-template <int FMT>
+template <int FMT, bool ANY>
 __global__ void __launch_bounds__(kTileThreads, 1)
 k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
                       const uint2* __restrict__ bmap, uint32_t desc_off,
@@ -1777,7 +1881,7 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
   const uint2 m = bmap[blockIdx.x];
   load_shared(&s_v, &nets[m.x].v);
   __syncthreads();
-  serve_tile<FMT>(s_v, m.y, acc_mem, desc_off, desc_cap);
+  serve_tile<FMT, ANY>(s_v, m.y, acc_mem, desc_off, desc_cap);
 }
 
 // ---------------------------------------------------------------------------
@@ -2332,14 +2436,14 @@ __device__ __noinline__ void serve_update(const NetView& v, const UpdConst& c,
                                           int n_steps, uint32_t block) {
   update_body<false, true>(v, c, n_steps, 1, 0, block);
 }
-template <int FMT>
+template <int FMT, bool ANY>
 __device__ __noinline__ void serve_deliver(const NetView& v, uint32_t tile,
                                            int* acc_mem, uint32_t desc_off,
                                            uint32_t desc_cap) {
-  serve_tile<FMT>(v, tile, acc_mem, desc_off, desc_cap);
+  serve_tile<FMT, ANY>(v, tile, acc_mem, desc_off, desc_cap);
 }
 
-template <int FMT>
+template <int FMT, bool ANY>
 __global__ void __launch_bounds__(kTileThreads, 1)
 k_serve(const BatchNet* __restrict__ nets, ServeNet* sn, ServeCtl* ctl,
         uint32_t n_nets, uint32_t desc_off, uint32_t desc_cap,
@@ -2412,7 +2516,7 @@ k_serve(const BatchNet* __restrict__ nets, ServeNet* sn, ServeCtl* ctl,
       __syncthreads();
       serve_update(v, s_c, nets[j].n_steps, w);
     } else {
-      serve_deliver<FMT>(v, w - q.ub, acc_mem, desc_off, desc_cap);
+      serve_deliver<FMT, ANY>(v, w - q.ub, acc_mem, desc_off, desc_cap);
     }
     __threadfence();
     __syncthreads();
@@ -2538,6 +2642,18 @@ int fixed_qs_host(uint64_t e, double max_abs_w) {
   qs = std::min(qs, 21 - wexp);
   if (qs < 0) return -1;
   return std::min(qs, 100);
+}
+
+int add_mode(const NetView& v, uint64_t events) {
+  if (v.lay == kLayHom && (events <= 0xFFFFull || v.acc_words == 2))
+    return events <= 0xFFFFull ? kAddVectors : kAddWide;
+  const int qs = v.lay == kLayRecords ? -1 : fixed_qs_host(events, v.max_abs_w);
+  if (qs < 0 || (v.acc_words == 1 && qs < v.acc_qs_min)) return kAddAny;
+  return v.lay == kLayHom ? kAddWeighted : kAddVectors;
+}
+// (the largest bound decides: scales only grow as it shrinks)
+int own_add_mode(const NetView& v) {
+  return add_mode(v, cell_events(v, ~0u, true));
 }
 
 int deliver_grid_size(int fmt) {
@@ -2680,21 +2796,39 @@ cudaError_t desc_layout(size_t used, size_t dyn_max, bool plastic,
   return cudaSuccess;
 }
 
-template <int LAY, bool COUNT, int KIND>
+template <int LAY, bool COUNT, int KIND, int MODE>
 cudaError_t launch_tiled_t(const NetView& v, unsigned long long* pair,
                            unsigned int* done, const SpikeEntry* list,
-                           int from_list_range, int advance_time,
-                           cudaStream_t s) {
+                           int advance_time, cudaStream_t s) {
   static std::atomic<uint32_t> lim[64];
   size_t dm = 0;
-  cudaError_t e = allow_tile_smem(k_deliver_tiled<LAY, COUNT, KIND>, lim, &dm);
+  cudaError_t e = allow_tile_smem(k_deliver_tiled<LAY, COUNT, KIND, MODE>, lim, &dm);
   if (e != cudaSuccess) return e;
   DescLayout dl;
   e = desc_layout(tiled_smem_bytes(v), dm, false, &dl);
   if (e != cudaSuccess) return e;
-  k_deliver_tiled<LAY, COUNT, KIND><<<v.n_tiles, kTileThreads, dl.smem, s>>>(
-      v, pair, done, list, from_list_range, advance_time, dl.off, dl.cap);
+  k_deliver_tiled<LAY, COUNT, KIND, MODE><<<v.n_tiles, kTileThreads, dl.smem, s>>>(
+      v, pair, done, list, advance_time, dl.off, dl.cap);
   return cudaGetLastError();
+}
+template <int LAY, int KIND>
+cudaError_t launch_tiled_k(const NetView& v, unsigned long long* pair,
+                           unsigned int* done, const SpikeEntry* list, int mode,
+                           int advance_time, cudaStream_t s) {
+  if (v.counts)
+    return launch_tiled_t<LAY, true, KIND, kAddAny>(v, pair, done, list, advance_time, s);
+  if (mode == kAddVectors)
+    return launch_tiled_t<LAY, false, KIND, kAddVectors>(v, pair, done, list,
+                                                         advance_time, s);
+  if constexpr (LAY == kLayHom) {
+    if (mode == kAddWide)
+      return launch_tiled_t<LAY, false, KIND, kAddWide>(v, pair, done, list,
+                                                        advance_time, s);
+    if (mode == kAddWeighted)
+      return launch_tiled_t<LAY, false, KIND, kAddWeighted>(v, pair, done, list,
+                                                            advance_time, s);
+  }
+  return launch_tiled_t<LAY, false, KIND, kAddAny>(v, pair, done, list, advance_time, s);
 }
 
 template <int LAY, bool COUNT>
@@ -2718,25 +2852,28 @@ cudaError_t launch_plastic_t(const NetView& v, unsigned long long* pair,
 
 cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
                                  unsigned int* done, const SpikeEntry* list,
-                                 int from_list_range, int advance_time,
+                                 uint32_t n_prepared, int advance_time,
                                  cudaStream_t s) {
-  if ((v.gx || v.ext_src) && from_list_range) return cudaErrorInvalidValue;
+  if ((v.gx || v.ext_src) && n_prepared) return cudaErrorInvalidValue;
   if (v.plastic) {
-    if (v.gx || v.ext_src || from_list_range) return cudaErrorNotSupported;
+    if (v.gx || v.ext_src || n_prepared) return cudaErrorNotSupported;
     if (v.lay == kLayF32)
       return v.counts ? launch_plastic_t<kLayF32, true>(v, pair, done, list, advance_time, s)
                       : launch_plastic_t<kLayF32, false>(v, pair, done, list, advance_time, s);
     return v.counts ? launch_plastic_t<kLayJ16, true>(v, pair, done, list, advance_time, s)
                     : launch_plastic_t<kLayJ16, false>(v, pair, done, list, advance_time, s);
   }
-#define SNN_TILED_K(L, C)                                                     \
-  (v.gx ? launch_tiled_t<L, C, kListGathered>(v, pair, done, list, 0,         \
-                                              advance_time, s)                \
-   : v.ext_src ? launch_tiled_t<L, C, kListRaw>(v, pair, done, list, 0, 0, s) \
-               : launch_tiled_t<L, C, kListOwn>(v, pair, done, list,          \
-                                                from_list_range,              \
-                                                advance_time, s))
-#define SNN_TILED(L) (v.counts ? SNN_TILED_K(L, true) : SNN_TILED_K(L, false))
+  const uint32_t n_caller = v.ext_src ? v.ext_n : n_prepared;
+  const int mode = kChecked ? (int)kAddAny
+                   : n_caller ? add_mode(v, cell_events(v, n_caller, false))
+                              : v.own_mode;
+#define SNN_TILED(L)                                                            \
+  (v.gx ? launch_tiled_k<L, kListGathered>(v, pair, done, list, mode,           \
+                                           advance_time, s)                     \
+   : v.ext_src ? launch_tiled_k<L, kListRaw>(v, pair, done, list, mode, 0, s) \
+   : n_prepared ? launch_tiled_k<L, kListRange>(v, pair, done, list, mode, 0, s) \
+                : launch_tiled_k<L, kListOwn>(v, pair, done, list, mode,        \
+                                              advance_time, s))
   switch (v.lay) {
     case kLayHom: return SNN_TILED(kLayHom);
     case kLayF32: return SNN_TILED(kLayF32);
@@ -2744,7 +2881,6 @@ cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
     default: return SNN_TILED(kLayJ16);
   }
 #undef SNN_TILED
-#undef SNN_TILED_K
 }
 
 bool deliver_raw_fits(const NetView& v, uint32_t n) {
@@ -2757,7 +2893,7 @@ cudaError_t launch_deliver_raw(const NetView& v, const uint32_t* src,
   x.ext_src = src;
   x.ext_t = t;
   x.ext_n = n;
-  return launch_deliver_tiled(x, nullptr, nullptr, nullptr, 0, 0, s);
+  return launch_deliver_tiled(x, nullptr, nullptr, nullptr, 0u, 0, s);
 }
 
 // Whether the intervals of a net can run in k_simulate: a split store whose
@@ -2886,54 +3022,63 @@ cudaError_t launch_update_batch(const BatchNet* nets, const uint2* bmap,
   return cudaGetLastError();
 }
 
-cudaError_t launch_deliver_tiled_batch(int fmt, const BatchNet* nets,
-                                       const uint2* bmap, uint32_t n_ctas,
-                                       size_t smem, cudaStream_t s) {
-  if (n_ctas == 0) return cudaSuccess;
-  static std::atomic<uint32_t> lim[2][64];
-  const int k = fmt == SNN_W_FP32_12B ? 0 : 1;
+template <int FMT, bool ANY>
+static cudaError_t launch_batch_t(const BatchNet* nets, const uint2* bmap,
+                                  uint32_t n_ctas, size_t smem, cudaStream_t s) {
+  static std::atomic<uint32_t> lim[64];
   size_t dm = 0;
-  cudaError_t e = k == 0
-      ? allow_tile_smem(k_deliver_tiled_batch<SNN_W_FP32_12B>, lim[0], &dm)
-      : allow_tile_smem(k_deliver_tiled_batch<SNN_W_BF16_8B>, lim[1], &dm);
+  cudaError_t e = allow_tile_smem(k_deliver_tiled_batch<FMT, ANY>, lim, &dm);
   if (e != cudaSuccess) return e;
   DescLayout dl;  // after the largest accumulator of the batch
   e = desc_layout(smem, dm, false, &dl);
   if (e != cudaSuccess) return e;
-  if (k == 0)
-    k_deliver_tiled_batch<SNN_W_FP32_12B><<<n_ctas, kTileThreads, dl.smem, s>>>(
-        nets, bmap, dl.off, dl.cap);
-  else
-    k_deliver_tiled_batch<SNN_W_BF16_8B><<<n_ctas, kTileThreads, dl.smem, s>>>(
-        nets, bmap, dl.off, dl.cap);
+  k_deliver_tiled_batch<FMT, ANY><<<n_ctas, kTileThreads, dl.smem, s>>>(nets, bmap, dl.off,
+                                                                       dl.cap);
   return cudaGetLastError();
+}
+
+cudaError_t launch_deliver_tiled_batch(int fmt, bool any, const BatchNet* nets,
+                                       const uint2* bmap, uint32_t n_ctas,
+                                       size_t smem, cudaStream_t s) {
+  if (n_ctas == 0) return cudaSuccess;
+  if (fmt == SNN_W_FP32_12B)
+    return any ? launch_batch_t<SNN_W_FP32_12B, true>(nets, bmap, n_ctas, smem, s)
+               : launch_batch_t<SNN_W_FP32_12B, false>(nets, bmap, n_ctas, smem, s);
+  return any ? launch_batch_t<SNN_W_BF16_8B, true>(nets, bmap, n_ctas, smem, s)
+             : launch_batch_t<SNN_W_BF16_8B, false>(nets, bmap, n_ctas, smem, s);
 }
 
 uint32_t update_threads() { return kUpdThreads; }
 
 uint32_t serve_threads() { return kTileThreads; }
 
-cudaError_t launch_serve(int fmt, const BatchNet* nets, ServeNet* sn,
-                         ServeCtl* ctl, uint32_t n_nets, uint32_t n_ctas,
-                         size_t smem, unsigned long long spin_limit,
-                         cudaStream_t s) {
-  if (n_nets == 0 || n_ctas == 0) return cudaSuccess;
-  static std::atomic<uint32_t> lim[2][64];
-  const int k = fmt == SNN_W_FP32_12B ? 0 : 1;
+template <int FMT, bool ANY>
+static cudaError_t launch_serve_t(const BatchNet* nets, ServeNet* sn, ServeCtl* ctl,
+                                  uint32_t n_nets, uint32_t n_ctas, size_t smem,
+                                  unsigned long long spin_limit, cudaStream_t s) {
+  static std::atomic<uint32_t> lim[64];
   size_t dm = 0;
-  cudaError_t e = k == 0 ? allow_tile_smem(k_serve<SNN_W_FP32_12B>, lim[0], &dm)
-                         : allow_tile_smem(k_serve<SNN_W_BF16_8B>, lim[1], &dm);
+  cudaError_t e = allow_tile_smem(k_serve<FMT, ANY>, lim, &dm);
   if (e != cudaSuccess) return e;
   DescLayout dl;  // after the largest accumulator of the nets
   e = desc_layout(smem, dm, false, &dl);
   if (e != cudaSuccess) return e;
-  if (k == 0)
-    k_serve<SNN_W_FP32_12B><<<n_ctas, kTileThreads, dl.smem, s>>>(
-        nets, sn, ctl, n_nets, dl.off, dl.cap, spin_limit);
-  else
-    k_serve<SNN_W_BF16_8B><<<n_ctas, kTileThreads, dl.smem, s>>>(
-        nets, sn, ctl, n_nets, dl.off, dl.cap, spin_limit);
+  k_serve<FMT, ANY><<<n_ctas, kTileThreads, dl.smem, s>>>(nets, sn, ctl, n_nets, dl.off,
+                                                          dl.cap, spin_limit);
   return cudaGetLastError();
+}
+
+cudaError_t launch_serve(int fmt, bool any, const BatchNet* nets, ServeNet* sn,
+                         ServeCtl* ctl, uint32_t n_nets, uint32_t n_ctas,
+                         size_t smem, unsigned long long spin_limit,
+                         cudaStream_t s) {
+  if (n_nets == 0 || n_ctas == 0) return cudaSuccess;
+#define SNN_SERVE(F, ANY) \
+  launch_serve_t<F, ANY>(nets, sn, ctl, n_nets, n_ctas, smem, spin_limit, s)
+  if (fmt == SNN_W_FP32_12B)
+    return any ? SNN_SERVE(SNN_W_FP32_12B, true) : SNN_SERVE(SNN_W_FP32_12B, false);
+  return any ? SNN_SERVE(SNN_W_BF16_8B, true) : SNN_SERVE(SNN_W_BF16_8B, false);
+#undef SNN_SERVE
 }
 
 cudaError_t launch_prepare_external(const NetView& v, const uint32_t* src,
@@ -3006,7 +3151,7 @@ cudaError_t launch_deliver_noalloc(const NetView& v, const uint32_t* src,
   e = launch_prepare_external(v, src, t, n, sc->list, &sc->pair, s);
   if (e != cudaSuccess) return e;
   return v.lay != kLayRecords
-             ? launch_deliver_tiled(v, &sc->pair, &sc->done, sc->list, 1, 0, s)
+             ? launch_deliver_tiled(v, &sc->pair, &sc->done, sc->list, n, 0, s)
              : launch_deliver(v, &sc->pair, &sc->done, sc->list, 0, s);
 }
 }  // namespace snn

@@ -68,6 +68,7 @@ struct snn_net {
   int lo_bits = 0;
   int window = 0;
   uint32_t mult_max = 0, k_in_max = 0, spikes_per_iv = 1;
+  int own_mode = kAddAny;  // own_add_mode, from snn_finalize on
   int acc_words = 2, acc_qs_min = 0;  // accumulator cells (see NetView)
   float max_abs_w = 0.f;
   SpikeEntry* list = nullptr;
@@ -192,6 +193,7 @@ struct snn_net {
     v.isi_n = isi_n;
     v.isi_sum = isi_sum;
     v.isi_sq = isi_sq;
+    v.own_mode = own_mode;
     return v;
   }
 };

@@ -138,6 +138,7 @@ struct LaneTables {
   size_t cap_nets = 0, cap_umap = 0, cap_dmap = 0;
   uint32_t n_ublocks = 0, n_dctas = 0;
   size_t dsmem = 0;
+  bool any = false;  // (see launch_deliver_tiled_batch)
   // host copies, kept until the next rewrite (the copies to the device are
   // asynchronous)
   std::vector<BatchNet> h_nets;
@@ -433,6 +434,8 @@ int rebuild_tables(Lane* ln, bool* busy) {
   t.n_ublocks = (uint32_t)t.h_umap.size();
   t.n_dctas = (uint32_t)t.h_dmap.size();
   t.dsmem = smem;
+  t.any = false;
+  for (const BatchNet& b : t.h_nets) t.any = t.any || b.v.own_mode != kAddVectors;
   for (cudaGraphExec_t& g : t.graph)
     if (g) {
       cudaGraphExecDestroy(g);
@@ -447,8 +450,8 @@ int launch_intervals(Lane* ln, int fmt, int m) {
   const LaneTables& t = ln->tab[ln->cur];
   for (int i = 0; i < m; ++i) {
     SCK(launch_update_batch(t.d_nets, t.d_umap, t.n_ublocks, ln->stream));
-    SCK(launch_deliver_tiled_batch(fmt, t.d_nets, t.d_dmap, t.n_dctas, t.dsmem,
-                                   ln->stream));
+    SCK(launch_deliver_tiled_batch(fmt, t.any, t.d_nets, t.d_dmap, t.n_dctas,
+                                   t.dsmem, ln->stream));
   }
   return SNN_OK;
 }
@@ -966,7 +969,7 @@ int lane_step_persistent(snn_server* sv, Lane* ln, bool* launched) {
   // builds run at a higher priority and need no reserve)
   const int ctas =
       std::max(1, sv->sms - (sv->building_large.load() ? kBuildReserveSms : 0));
-  SCK(launch_serve(sv->fmt, tb.d_nets, ln->d_sn, ln->d_ctl, (uint32_t)n,
+  SCK(launch_serve(sv->fmt, tb.any, tb.d_nets, ln->d_sn, ln->d_ctl, (uint32_t)n,
                    (uint32_t)ctas, tb.dsmem, sv->spin_limit, ln->stream));
   SCK(cudaMemcpyAsync(ln->h_sn_back[slot], ln->d_sn, n * sizeof(ServeNet),
                       cudaMemcpyDeviceToHost, ln->stream));

@@ -546,9 +546,11 @@ int snn_clear_errors(snn_net* net);
 /* Wait for all work of the net. */
 int snn_sync(snn_net* net);
 /* 1 for a bounds-checked build of the library (compiled with SNN_CHECK:
- * every record's target and delay, every tile index entry and the order of
- * every chunk offset is checked before use, failures raise SNN_ERRF_CHECK
- * and skip the access), 0 for the production build. */
+ * every record's target and delay, every vector of a run and the cell it adds
+ * to, every tile index entry, the one-launch cycle's list entries and the order
+ * of every chunk offset is checked before use, failures raise SNN_ERRF_CHECK
+ * and skip the access; it launches the same kernels as the production build),
+ * 0 for the production build. */
 int snn_checked(void);
 /* Bounds-checked builds: the number of nets whose SNN_ERRF_CHECK flag was
  * seen set by snn_get_stats or snn_destroy since the library was loaded

@@ -142,9 +142,11 @@ constexpr int32_t kNoSpike = INT32_MIN;
 constexpr int kMaxStdpHistory = 32;
 constexpr uint32_t kMaxGatherParts = 64;  // exchange buffers of one delivery
 // SNN_CHECK builds (-DSNN_CHECK=1) compile bounds checks into the kernels:
-// a record whose target or delay lies outside the store's ranges, a tile
-// index entry outside its row, or a spike list whose chunk offsets are not
-// non-decreasing is skipped and raises SNN_ERRF_CHECK instead of being used.
+// a record whose target or delay lies outside the store's ranges, a vector
+// outside the store or a cell outside the accumulator, a tile index entry outside
+// its row, an entry of the one-launch cycle's list outside its interval, or a
+// spike list whose chunk offsets are not non-decreasing is skipped and raises
+// SNN_ERRF_CHECK instead of being used.
 #ifndef SNN_CHECK
 #define SNN_CHECK 0
 #endif
@@ -293,6 +295,9 @@ struct NetView {
   const uint16_t* cells;
   const uint32_t* tgts;     // kLayF32 and FP32 kLayHom: the targets
   uint32_t row_mul;
+#if SNN_CHECK
+  uint64_t n_pad;           // records the store has room for
+#endif
   int d_base;
   int lg;                   // log2 of the lanes that share a run
   float mean_row;           // synapses per source

@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "snn_internal.cuh"
 
@@ -1184,7 +1185,44 @@ template <int LAY> struct LaneRun {
   const char* p;   // the lane's first vector
   int n, lo;
   uint32_t row_s, inc;
+#if SNN_CHECK
+  uint64_t tgt;    // index of the target of the lane's element 0
+  int32_t off;
+#endif
 };
+
+// Bounds-checked builds: what the vectors and elements of a tile's runs are
+// checked against; the vector at p must lie in the store, an element's cell in
+// its window, on its target and in the accumulator.
+#if SNN_CHECK
+struct RunCheck {
+  const NetView* v;
+  uint32_t tgt_lo;
+  uint32_t acc_len;  // cells of the accumulator
+};
+__device__ __forceinline__ bool flag_check(const NetView& v, bool ok) {
+  if (!ok) atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_CHECK);
+  return ok;
+}
+__device__ __forceinline__ bool vec_in_store(const NetView& v, const char* p) {
+  const uint64_t b = reinterpret_cast<uint64_t>(p) - reinterpret_cast<uint64_t>(v.dat);
+  const uint64_t bytes =
+      v.fmt != SNN_W_FP32_12B ? 8 * v.n_pad : (v.lay == kLayHom ? 2 : 4) * v.n_pad;
+  return flag_check(v, b % 16 == 0 && b < bytes && b + 16 <= bytes);
+}
+template <int LAY>
+__device__ __forceinline__ uint32_t vec_cell(const Vec<LAY>& x, int k) {
+  uint32_t w;
+  if constexpr (LAY == kLayF32) w = k < 2 ? x.c.x : x.c.y;
+  else if constexpr (LAY == kLayHom)
+    w = k < 2 ? x.a.x : k < 4 ? x.a.y : k < 6 ? x.a.z : x.a.w;
+  else w = k == 0 ? x.a.x : k == 1 ? x.a.y : k == 2 ? x.a.z : x.a.w;
+  return (LAY == kLayF32 || LAY == kLayHom) && (k & 1) ? w >> 16 : w & 0xFFFFu;
+}
+#define SNN_CHECKED(...) , __VA_ARGS__
+#else
+#define SNN_CHECKED(...)
+#endif
 
 // Phase (B) for a batch of nb described runs, 2^lg lanes a run: every warp
 // takes each kTileWarps-th group of 32 / 2^lg runs, and loads a lane's first
@@ -1197,7 +1235,8 @@ template <int LAY>
 __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
                                       const SegDesc* s_desc, uint32_t nb,
                                       uint32_t acc_s, uint32_t lo_off,
-                                      uint32_t lg, SplitScale fx,
+                                      uint32_t lg,
+                                      SplitScale fx SNN_CHECKED(RunCheck chk),
                                       uint32_t inc0 = 1u, uint32_t inc1 = 0x10000u) {
   constexpr uint32_t E = Lay<LAY>::kElems;
   __shared__ uint32_t s_none[32];  // what masked elements add to
@@ -1225,21 +1264,50 @@ __device__ __forceinline__ void add_runs(const char* dat, const char* cel,
       r.n = (int)(sd.len & 0x7FFFFFFFu) - (int)(sub * E);
       r.row_s = acc_s + 4u * (uint32_t)sd.off;
       r.inc = (int)sd.len < 0 ? inc1 : inc0;
+#if SNN_CHECK
+      r.tgt = sd.tgt + sub * E - (sd.beg & 15u);
+      r.off = sd.off;
+      for (int q = 0; r.n > q * kStep; ++q)
+        if (!vec_in_store(*chk.v, r.p + (size_t)q * (L * 16u))) r.n = q * kStep;
+#endif
 #pragma unroll
       for (int q = 0; q < kAhead; ++q)
         if (r.n > q * kStep) r.x[q] = fetch(r, q);
     }
   };
+  // elements [lo, r.n - q kStep) of the lane's vector q; CLIP: lo may not be 0
+  auto put = [&](auto clip, const LaneRun<LAY>& r, const Vec<LAY>& x, int q, int lo) {
+    constexpr bool CLIP = decltype(clip)::value;
+    const int n = r.n - q * kStep;
+#if SNN_CHECK
+    uint32_t good = 0, all = 0;
+    for (int k = lo; k < min(n, (int)E); ++k) {
+      const uint32_t cell = vec_cell<LAY>(x, k);
+      const uint64_t ti = r.tgt + (uint64_t)(q * kStep + k);
+      const uint32_t tgt = chk.v->tgts ? chk.v->tgts[ti]
+                                       : reinterpret_cast<const uint32_t*>(chk.v->recs)[ti];
+      all |= 1u << k;
+      if (cell_in_bounds(*chk.v, cell, tgt, chk.tgt_lo) &&
+          flag_check(*chk.v, (uint32_t)r.off + cell < chk.acc_len))
+        good |= 1u << k;
+    }
+    if (good != all) {  // the others one by one
+      for (int k = 0; k < (int)E; ++k)
+        if (good >> k & 1u)
+          add_vec<LAY, true>(x, r.row_s, r.inc, k + 1, k, lo_off, none, fx);
+      return;
+    }
+#endif
+    add_vec<LAY, CLIP>(x, r.row_s, r.inc, n, lo, lo_off, none, fx);
+  };
   auto add = [&](LaneRun<LAY>& r) {
-    if (r.n > 0) add_vec<LAY, true>(r.x[0], r.row_s, r.inc, r.n, r.lo, lo_off, none, fx);
+    if (r.n > 0) put(std::true_type{}, r, r.x[0], 0, r.lo);
 #pragma unroll
     for (int q = 1; q < kAhead; ++q)
-      if (r.n > q * kStep)
-        add_vec<LAY, false>(r.x[q], r.row_s, r.inc, r.n - q * kStep, 0, lo_off,
-                            none, fx);
+      if (r.n > q * kStep) put(std::false_type{}, r, r.x[q], q, 0);
     for (int q = kAhead; r.n > q * kStep; ++q) {
       const Vec<LAY> x = fetch(r, q);
-      add_vec<LAY, false>(x, r.row_s, r.inc, r.n - q * kStep, 0, lo_off, none, fx);
+      put(std::false_type{}, r, x, q, 0);
     }
   };
   uint32_t k = (threadIdx.x >> 5) * R;
@@ -1260,8 +1328,9 @@ template <int LAY>
 __device__ __noinline__ void add_runs_call(const char* dat, const char* cel,
                                            const SegDesc* s_desc, uint32_t nb,
                                            uint32_t acc_s, uint32_t lo_off,
-                                           uint32_t lg, SplitScale fx) {
-  add_runs<LAY>(dat, cel, s_desc, nb, acc_s, lo_off, lg, fx);
+                                           uint32_t lg,
+                                           SplitScale fx SNN_CHECKED(RunCheck chk)) {
+  add_runs<LAY>(dat, cel, s_desc, nb, acc_s, lo_off, lg, fx SNN_CHECKED(chk));
 }
 
 template <int LAY, int KIND>
@@ -1520,6 +1589,9 @@ __device__ __forceinline__ void deliver_tile_body(
     // (after the barrier: s_events was cleared before it)
     if ((GX || RAW) && lane == 0 && warp_events) atomicAdd(&s_events, warp_events);
     fx = s_fx;
+#if SNN_CHECK
+    const RunCheck chk{&v, tgt_lo, MODE == kAddWide ? 2 * cells : cells};
+#endif
     if constexpr (MODE == kAddAny) {
       add_any(nb);
     } else if constexpr (MODE == kAddWeighted) {
@@ -1527,11 +1599,12 @@ __device__ __forceinline__ void deliver_tile_body(
       fixed_split(v.hom_w[0], fx, h[0], l);
       fixed_split(v.hom_w[1], fx, h[1], l);
       add_runs<LAY>(reinterpret_cast<const char*>(v.dat), nullptr, s_desc, nb, acc_s, 0u,
-                    lg, SplitScale{}, (uint32_t)h[0], (uint32_t)h[1]);
+                    lg, SplitScale{} SNN_CHECKED(chk), (uint32_t)h[0], (uint32_t)h[1]);
     } else {
       add_runs<LAY>(reinterpret_cast<const char*>(v.dat),
                     reinterpret_cast<const char*>(v.cells), s_desc, nb, acc_s,
-                    two ? 4u * cells : 0u, lg, SplitScale{fx.scale_hs, fx.scale_s});
+                    two ? 4u * cells : 0u, lg,
+                    SplitScale{fx.scale_hs, fx.scale_s} SNN_CHECKED(chk));
     }
     j0 += nb;
     __syncthreads();  // s_desc is rewritten by the next batch
@@ -1847,9 +1920,9 @@ template <int LAY, bool ANY>
 __device__ __forceinline__ void serve_tile_lay(const NetView& v, uint32_t tile,
                                                int* acc_mem, uint32_t desc_off,
                                                uint32_t desc_cap) {
-  if constexpr (!ANY && !kChecked)
+  if constexpr (!ANY)
     serve_tile_body<LAY, kAddVectors>(v, tile, acc_mem, desc_off, desc_cap);
-  else if (!kChecked && v.own_mode == kAddVectors)
+  else if (v.own_mode == kAddVectors)
     serve_tile_call<LAY, kAddVectors>(v, tile, acc_mem, desc_off, desc_cap);
   else
     serve_tile_call<LAY, kAddAny>(v, tile, acc_mem, desc_off, desc_cap);
@@ -2135,12 +2208,24 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
             const uint32_t mid = (at + hi) >> 1;
             if (s_start[mid] <= g) at = mid; else hi = mid;
           }
+#if SNN_CHECK
+          if (!flag_check(v, at < G && g - s_start[at] < sh.region)) {
+            e[u] = 0xFFFFFFFFu;
+            continue;
+          }
+#endif
           e[u] = ld_list(list + (size_t)at * sh.region + (g - s_start[at]));
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           if (k0 + u * kTileThreads >= nb) continue;
           const uint32_t src = e[u] & 0xFFFFFFu;
+#if SNN_CHECK
+          if (!flag_check(v, src < v.n_src && (int)(e[u] >> 24) < v.d_min)) {
+            e[u] = 0u;
+            continue;  // (an empty run)
+          }
+#endif
           const uint32_t* to = v.tile_off + (uint64_t)src * (v.n_tiles + 1) + r;
           ra[u] = ld_list(to);
           rb[u] = ld_list(to + 1);
@@ -2152,6 +2237,13 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
           const uint32_t k = k0 + u * kTileThreads;
           if (k >= nb) continue;
           SegDesc sd;
+#if SNN_CHECK
+          const uint64_t row_end = v.row_ptr[(e[u] & 0xFFFFFFu) + 1];
+          if (!flag_check(v, ra[u] <= rb[u] && (rb[u] == 0 || row[u] + rb[u] <= row_end)))
+            rb[u] = ra[u];
+          sd.tgt = v.fmt == SNN_W_FP32_12B ? row[u] + ra[u]
+                                           : 2 * row[u] + (row_end - row[u]) + ra[u];
+#endif
           place_run<LAY>(v, row[u] * v.row_mul + ra[u], rb[u] - ra[u], &sd);
           // (base = t_list + d_min)
           sd.off = ((int32_t)(e[u] >> 24) - v.d_min + v.d_base) * (int32_t)TW;
@@ -2166,7 +2258,8 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
         add_runs_call<LAY>(reinterpret_cast<const char*>(v.dat),
                            reinterpret_cast<const char*>(v.cells), s_desc, nb,
                            acc_s, TWO ? 4u * cells : 0u, lg,
-                           SplitScale{s_fx.scale_hs, s_fx.scale_s});
+                           SplitScale{s_fx.scale_hs, s_fx.scale_s}
+                               SNN_CHECKED(RunCheck{&v, lo, cells}));
       j0 += nb;
       if (j0 < n_sp) __syncthreads();  // s_desc is rewritten by the next batch
     } while (j0 < n_sp);
@@ -2864,9 +2957,7 @@ cudaError_t launch_deliver_tiled(const NetView& v, unsigned long long* pair,
                     : launch_plastic_t<kLayJ16, false>(v, pair, done, list, advance_time, s);
   }
   const uint32_t n_caller = v.ext_src ? v.ext_n : n_prepared;
-  const int mode = kChecked ? (int)kAddAny
-                   : n_caller ? add_mode(v, cell_events(v, n_caller, false))
-                              : v.own_mode;
+  const int mode = n_caller ? add_mode(v, cell_events(v, n_caller, false)) : v.own_mode;
 #define SNN_TILED(L)                                                            \
   (v.gx ? launch_tiled_k<L, kListGathered>(v, pair, done, list, mode,           \
                                            advance_time, s)                     \
@@ -2957,7 +3048,7 @@ bool simulate_fits(const NetView& v, const UpdConst& c, int interval,
                    SimShared* sh, uint32_t* ctas) {
   // (a reset at or above the threshold fires at every step, refractory or not)
   if (!(c.v_reset < c.v_th)) return false;
-  if (kChecked || v.lay == kLayRecords || v.plastic || v.counts || v.xbuf ||
+  if (v.lay == kLayRecords || v.plastic || v.counts || v.xbuf ||
       interval < 1 || interval > (int)kSimMaxSteps || v.n_tiles == 0)
     return false;
   const uint64_t e = (uint64_t)v.k_in_max * std::max(v.spikes_per_iv, 1u);

@@ -120,6 +120,9 @@ struct snn_net {
     v->cells = nullptr;
     v->tgts = nullptr;
     v->row_mul = 1;
+#if SNN_CHECK
+    v->n_pad = n_pad;
+#endif
     v->lg = 0;
     v->mean_row = n_src ? (float)((double)n_syn / n_src) : 0.f;
     if (lay == kLayRecords) return;

@@ -797,6 +797,7 @@ __device__ __forceinline__ void fixed_split(float w, const Scale& fx,
 __device__ __forceinline__ uint32_t cell_magic(uint32_t tw) {
   return tw > 1u ? (uint32_t)(0x100000000ull / tw) + 1u : 0u;
 }
+// (The quotient of any multiple of TW, which exceeds it by no more.)
 __device__ __forceinline__ uint32_t cell_step(uint32_t cell, uint32_t magic) {
   return magic ? __umulhi(cell, magic) : cell;  // (one target a tile)
 }
@@ -1815,7 +1816,10 @@ __device__ __forceinline__ void deliver_tile_plastic(
         if (j >= nb) break;  // (uniform across the warp)
         const SegDesc sd = s_desc[j];
         const bool pl = tile_plastic && s_kprev[j] >= 0.f;
-        const int32_t t = (int32_t)(base - v.d_base) + sd.off / (int32_t)TW;
+        // (the run's step after base - d_base, from a multiple of TW)
+        const int32_t t =
+            (int32_t)(base - v.d_base) - 256 +
+            (int32_t)cell_step((uint32_t)(sd.off + 256 * (int32_t)TW), magic);
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
           const uint32_t idx = lane + 32u * q;

@@ -103,13 +103,22 @@ struct snn_net {
   double* isi_sum = nullptr;
   double* isi_sq = nullptr;
 
-  // Lanes per run (2^lg), for runs of up to the mean length plus three
-  // standard deviations of a Poisson count, in 16-byte vectors (8 cells, or 4
-  // joined words or weights): three vectors of a lane are loaded ahead, later
-  // ones one at a time, and every group of 32 / lanes runs costs a fixed
-  // number of instructions.  Measured (deliveries of 1,314 to 2,389 spikes):
-  // 74 cells 29.8 us on 8 lanes, 31.7 on 4, 33.5 on 16; 37 words 48.4 us on 4,
-  // 56.8 on 8, 73.9 on 16; 13 words 16.7 us on 4, 18.4 on 2, 18.2 on 8.
+  // Lanes per run (2^lg) from the mean run of a tile (in synapses) and the number
+  // of rows.  A lane has three 16-byte vectors loaded ahead (8 cells, or 4 joined
+  // words or weights) and every group of 32 / lanes runs costs a fixed number of
+  // instructions; runs past what is ahead want more lanes, and so do rows that lie
+  // far apart, of which a warp's request then touches fewer: the first lines sit
+  // at run x sqrt(rows).  Measured where two numbers of lanes take the same time
+  // (deliveries of 1,400 and 3,000 spikes; 20,003, 60,000 and 112,500 neurons):
+  //             1 | 2      2 | 4 lanes                4 | 8       8 | 16  16 | 32
+  //   cells     9-10       26, 17, 12                 92          310     500
+  //   words     3.5        16, 5.5, 5                 47          110     235
+  //   FP32      3          11, 4.5, 4.5               22, 11.5, 9.5  90   320
+  // (500: extrapolated.)  Either side, 3,000 spikes, 60,000 neurons, us: cells 74
+  // on 4 lanes 38.3, on 8 40.8, 120 52.4, 50.5; words 37 28.5, 32.4, 60 41.1, 36.8;
+  // FP32 9 33.9, 38.0, 20 50.1, 40.4, 37 73.1, 48.8.  Words between 5.5 and 16 are a
+  // compromise: 13 on 20,003 neurons take 19.2 us on 2 lanes and 21.2 on 4, but the
+  // shorter lists of their one-launch cycle 1,428 and 1,378 us for 100 intervals.
   void set_layout(NetView* v) const {
     v->lay = lay;
     v->d_base = d_base;
@@ -136,10 +145,16 @@ struct snn_net {
     }
     const double run =
         n_src && n_tiles ? (double)n_syn / ((double)n_src * n_tiles) : 0.0;
-    const double vecs = (run + 3.0 * sqrt(run)) / (lay == kLayHom ? 8.0 : 4.0) + 0.5;
-    const double most = lay == kLayHom ? 3.0 : 3.6;
-    v->lg = vecs > 3.0 ? 2 : vecs > 1.5 ? 1 : 0;
-    while (v->lg < 5 && most * (1 << v->lg) < vecs) ++v->lg;
+    const int k = lay == kLayHom ? 0 : lay == kLayF32 ? 2 : 1;
+    static const double first[3] = {9.5, 3.5, 3.0}, far_apart[3] = {4000, 1750, 1350};
+    static const double more[3][3] = {{92, 310, 500}, {47, 110, 235}, {0, 90, 320}};
+    const double spread = run * sqrt((double)n_src);
+    if (run < first[k]) return;
+    v->lg = 1;
+    if (spread < far_apart[k]) return;
+    v->lg = 2;
+    if (k == 2 ? spread < 3000.0 : run < more[k][0]) return;
+    v->lg = run < more[k][1] ? 3 : run < more[k][2] ? 4 : 5;
   }
 
   NetView view() const {

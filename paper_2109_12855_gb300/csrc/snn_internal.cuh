@@ -210,6 +210,17 @@ __host__ __device__ inline uint32_t scale_u32(uint32_t u, uint32_t n) {
 }
 
 #ifdef __CUDACC__
+// Delay steps above d_base of a cell (cell / TW) by a multiplication: with
+// m = floor(2^32 / TW) + 1, cell m / 2^32 exceeds cell / TW by less than
+// cell / 2^32 < 1 / TW (cells are below 2^16), so the floor is the same.
+__device__ __forceinline__ uint32_t cell_magic(uint32_t tw) {
+  return tw > 1u ? (uint32_t)(0x100000000ull / tw) + 1u : 0u;
+}
+// (The quotient of any multiple of TW, which exceeds it by no more.)
+__device__ __forceinline__ uint32_t cell_step(uint32_t cell, uint32_t magic) {
+  return magic ? __umulhi(cell, magic) : cell;  // (one target a tile)
+}
+
 // 2^x by the PTX instruction ex2.approx.ftz.f32, an approximation to within two
 // units in the last place by the PTX ISA (the CUDA C++ guide's bound for exp2f)
 // that flushes subnormal results to zero: for arguments in [-126, 128), whose

@@ -791,17 +791,6 @@ __device__ __forceinline__ void fixed_split(float w, const Scale& fx,
   lo = __float_as_int(__fmaf_rn(fr, fx.scale_s, kFixM)) - __float_as_int(kFixM);
 }
 
-// Delay steps above d_base of a cell (cell / TW) by a multiplication: with
-// m = floor(2^32 / TW) + 1, cell m / 2^32 exceeds cell / TW by less than
-// cell / 2^32 < 1 / TW (cells are below 2^16), so the floor is the same.
-__device__ __forceinline__ uint32_t cell_magic(uint32_t tw) {
-  return tw > 1u ? (uint32_t)(0x100000000ull / tw) + 1u : 0u;
-}
-// (The quotient of any multiple of TW, which exceeds it by no more.)
-__device__ __forceinline__ uint32_t cell_step(uint32_t cell, uint32_t magic) {
-  return magic ? __umulhi(cell, magic) : cell;  // (one target a tile)
-}
-
 // Bounds-checked builds: a cell outside the store's window or one that
 // disagrees with the synapse's target is skipped and flagged; so are targets
 // outside the tile.  Production builds compile this to `true`.

@@ -4,8 +4,8 @@ roofline fraction of spike delivery on one GB300.
 
 Default workload (one JSON line on stdout): the balanced random network with
 112,500 neurons (90,000 E + 22,500 I), in-degree 11,250 (9,000 E + 2,250 I),
-1.27e9 static synapses in 12-byte FP32 records, delay 1.5 ms (15 steps of
-0.1 ms), Poisson drive tuned for about 8 Hz.  One step = 1 s of biological
+1.27e9 static synapses with FP32 weights (10 bytes each as stored), delay 1.5 ms
+(15 steps of 0.1 ms), Poisson drive tuned for about 8 Hz.  One step = 1 s of biological
 time (10,000 grid steps = 667 update/deliver intervals) of the whole hot path:
 update, spike exchange and delivery, every interval.
 
@@ -705,7 +705,7 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
         per_s.clear()
         snn.snn_clear_spike_stats(h)
 
-    # ---- timed region: production path (graphs) --------------------------
+    # ---- timed region: production path --------------------------
     gpu_index = int(os.environ.get("CUDA_VISIBLE_DEVICES", str(local)).split(",")[0]) \
         if os.environ.get("CUDA_VISIBLE_DEVICES", "").split(",")[0].isdigit() else local
     clocks = Clocks(gpu_index)
@@ -717,6 +717,8 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
     events = b.events_delivered - a.events_delivered
     spikes = b.spikes - a.spikes
     launches = b.kernel_launches - a.kernel_launches
+    # (many intervals a launch: snn_simulate's one-launch cycle)
+    cycle = 0 < launches < b.update_launches - a.update_launches
     net.read_spikes(log_cap)
     ms_max, events_all, spikes_all = reduce_over_ranks(ms, events, spikes)
     value = events_all / (ms_max * 1e-3)
@@ -746,9 +748,7 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
     net.read_spikes(log_cap)
     # algorithmic bytes: what the store gives an event; per spike a list entry
     # (16 B) and its two row offsets (16 B); a plastic event also reads and
-    # writes its FP32 weight (8 B).  (The profiled pass runs the update and the
-    # delivery as separate kernels; the timed one is one launch for nets of at
-    # most a tile per SM.)
+    # writes its FP32 weight (8 B)
     n_listed = sp_prof if kind != "deliver" else len(src) * args.steps
     alg_bytes = ev_bytes * ev_prof + 32 * n_listed + 8 * pl_prof
     per_launch_bytes = alg_bytes / max(n_del, 1)
@@ -810,6 +810,34 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
             cpu = cpu_baseline_all_cores(args, wl, nu_ext)
             cpu["single_core"] = one
             cpu["host"] = host_info()
+    separate = {"kernel": "k_deliver_tiled" if args.deliver_mode == "tiled"
+                          else "k_deliver",
+                "achieved": achieved, "frac": achieved / hbm,
+                "frac_of_nominal": achieved / HBM_NOMINAL_GBS,
+                "algorithmic_bytes_per_launch": per_launch_bytes,
+                "launches": n_del, "avg_launch_us": 1e3 * ms_del / max(n_del, 1),
+                "traffic": measured_traffic(args.workload, ev_prof / max(n_del, 1)),
+                "ms_deliver_share": ms_del / ms_prof if ms_prof else None,
+                "ms_update_share": ms_upd / ms_prof if ms_prof else None,
+                "profiled_value": ev_prof / (ms_prof * 1e-3)}
+    if cycle:
+        # the timed kernel: update, exchange and delivery of up to 256 intervals
+        # a launch, on the timed region's clock; the profiled pass runs the update
+        # and the delivery as kernels of their own ("separate_kernels")
+        cycle_bytes = ev_bytes * events + 32 * spikes
+        got = cycle_bytes / (ms * 1e-3) / 1e9
+        roofline = {"kernel": "k_simulate", "achieved": got, "frac": got / hbm,
+                    "frac_of_nominal": got / HBM_NOMINAL_GBS,
+                    "algorithmic_bytes_per_launch": cycle_bytes / launches,
+                    "launches": launches, "avg_launch_us": 1e3 * ms / launches,
+                    "traffic": None, "separate_kernels": separate}
+    else:
+        roofline = dict(separate)
+    roofline.update(bound="hbm", peak=hbm, unit="GB/s", peak_source=peak_kind,
+                    traffic_unit="bytes per launch (ncu dram read+write)",
+                    deliver_mode=args.deliver_mode,
+                    tiles=[st_tiles.n_tiles, st_tiles.tile_width, st_tiles.window],
+                    bytes_per_event=ev_bytes + (8 * pl_prof / max(ev_prof, 1)))
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws,
         "steps": args.steps, "warmup": args.warmup,
@@ -820,8 +848,10 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
         "real_time_factor": (ms_max / args.steps) / bio_ms,
         "config": {"workload": args.workload, "neurons": wl.n,
                    "in_degree": wl.k, "synapses": wl.n_synapses,
-                   "record_bytes": rec_bytes, "interval_steps": D,
-                   "bio_ms_per_step": bio_ms, "nu_ext_hz": nu_ext,
+                   "record_bytes": rec_bytes,
+                   "store_bytes_per_synapse": round(
+                       st_tiles.store_bytes / max(wl.n_synapses, 1), 2),
+                   "interval_steps": D, "bio_ms_per_step": bio_ms, "nu_ext_hz": nu_ext,
                    "mean_rate_hz": spikes_all / ws / wl.n / (
                        args.steps * bio_ms * 1e-3),
                    "events_timed": events_all, "spikes_timed": int(spikes_all),
@@ -834,24 +864,7 @@ def run_ours(args, wl, fmt, bio_ms, kind, nu_ext):
                          f"{wl.n_synapses * ev_bytes / 1e9:.1f} GB are streamed "
                          "from HBM every step)",
                    "parallelism": f"replicas x{ws}"},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm,
-                     "unit": "GB/s", "frac": achieved / hbm,
-                     "peak_source": peak_kind,
-                     "frac_of_nominal": achieved / HBM_NOMINAL_GBS,
-                     "traffic": measured_traffic(args.workload,
-                                                 ev_prof / max(n_del, 1)),
-                     "traffic_unit": "bytes per launch (ncu dram read+write)",
-                     "algorithmic_bytes_per_launch": per_launch_bytes,
-                     "kernel": "k_deliver_tiled" if args.deliver_mode == "tiled"
-                               else "k_deliver",
-                     "launches": n_del, "avg_launch_us": 1e3 * ms_del / max(n_del, 1),
-                     "deliver_mode": args.deliver_mode,
-                     "tiles": [st_tiles.n_tiles, st_tiles.tile_width,
-                               st_tiles.window],
-                     "bytes_per_event": ev_bytes + (8 * pl_prof / max(ev_prof, 1)),
-                     "ms_deliver_share": ms_del / ms_prof if ms_prof else None,
-                     "ms_update_share": ms_upd / ms_prof if ms_prof else None,
-                     "profiled_value": ev_prof / (ms_prof * 1e-3)},
+        "roofline": roofline,
         "cpu_baseline": cpu,
         "e2e": e2e,
         "gpu_launches": launches,

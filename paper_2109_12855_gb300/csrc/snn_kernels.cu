@@ -2078,7 +2078,9 @@ __device__ __forceinline__ uint64_t ld_row(const uint64_t* p) {
   return x;
 }
 
-template <int LAY>
+// LIMITED: the limit of a wait is the launch's (tests); a parameter compared in the
+// poll loop costs 2 % at 20,003 neurons.
+template <int LAY, bool LIMITED>
 __global__ void __launch_bounds__(kTileThreads, 1)
 k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c,
            SimShared sh, int n_iv, int n_steps, int last_steps,
@@ -2114,10 +2116,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
   for (uint32_t x = tid; x < (TWO ? 2 * cells : cells); x += kTileThreads) acc[x] = 0;
   if (tid == 0) {
     s_cnt = 0;
-    // (a net whose cycle once gave up stays as it is until its errors are
-    // cleared: its CTAs had stopped at different steps)
-    s_bad = (*reinterpret_cast<volatile unsigned int*>(&v.ctl->error_flags) &
-             (unsigned)SNN_ERRF_TIMEOUT) != 0u;
+    s_bad = 0;
     s_sum[0] = s_sum[1] = 0ull;
     s_fx = FixScale{0, 0, 0, 1.f, 1.f, 1.f, 1.f};
   }
@@ -2138,8 +2137,13 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
   int t = (int)*reinterpret_cast<volatile long long*>(&v.ctl->t_now);
   unsigned long long logged = *reinterpret_cast<volatile unsigned long long*>(&v.ctl->log_count);
   unsigned long long my_events = 0, my_spikes = 0;
-  __syncthreads();
-  if (s_bad) return;  // (uniform in the CTA; one that set out finds `stop` set)
+  // (a net whose cycle once gave up stays as it is until its errors are cleared:
+  // its CTAs had stopped at different steps; a CTA that set out beside one that
+  // finds this finds `stop` set)
+  if (__syncthreads_or(tid == 0 &&
+                       (*reinterpret_cast<volatile unsigned int*>(&v.ctl->error_flags) &
+                        (unsigned)SNN_ERRF_TIMEOUT)))
+    return;
 
   // state of this thread's neuron, kept over the launch when it has only one
   float V = 0.f, I = 0.f, J = 0.f;
@@ -2404,7 +2408,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
         uint32_t polls = 0;
         while ((uint32_t)((x = ld_acquire_u64(f)) >> 32) != (uint32_t)(iv + 1)) {
           ++polls;
-          if (polls > sh.polls ||
+          if (polls > (LIMITED ? sh.polls : kSimPolls) ||
               ((polls & 1023u) == 0u &&
                *reinterpret_cast<volatile unsigned int*>(sh.stop))) {
             s_bad = 1;
@@ -2980,17 +2984,13 @@ cudaError_t launch_deliver_raw(const NetView& v, const uint32_t* src,
   return launch_deliver_tiled(x, nullptr, nullptr, nullptr, 0u, 0, s);
 }
 
-// Whether the intervals of a net can run in k_simulate: a split store whose
-// scales (and counts) exist for every interval, nothing that only the
-// separate kernels do (plasticity, counted cells, exchange buffers, bounds
-// checks), and lists that fit the interval list's memory.
-template <int LAY>
+template <int LAY, bool LIMITED>
 cudaError_t launch_simulate_t(const NetView& v, const UpdConst& c,
                               const SimShared& sh, uint32_t ctas, int n_iv,
                               int steps, int last_steps, cudaStream_t s) {
   static std::atomic<uint32_t> lim[64];
   size_t dm = 0;
-  cudaError_t e = allow_tile_smem(k_simulate<LAY>, lim, &dm);
+  cudaError_t e = allow_tile_smem(k_simulate<LAY, LIMITED>, lim, &dm);
   if (e != cudaSuccess) return e;
   DescLayout dl;  // after the accumulator and the drive (5 or 9 blocks)
   const size_t drv = ((size_t)v.tile_w * v.window * (SimCell<LAY>::kTwo ? 8u : 4u) + 15u) & ~(size_t)15u;
@@ -3011,7 +3011,7 @@ cudaError_t launch_simulate_t(const NetView& v, const UpdConst& c,
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, k_simulate<LAY>, v, c, sh, n_iv, steps,
+  e = cudaLaunchKernelEx(&cfg, k_simulate<LAY, LIMITED>, v, c, sh, n_iv, steps,
                          last_steps, (uint32_t)drv, dl.off, dl.cap, pf);
   if (e != cudaSuccess) return e;
   // The flags of the launch to come are cleared after this one, not before it:
@@ -3037,6 +3037,10 @@ static int sim_sms() {
   return m;
 }
 
+// Whether the intervals of a net can run in k_simulate: a split store whose
+// scales (and counts) exist for every interval, nothing that only the
+// separate kernels do (plasticity, counted cells, exchange
+// buffers), and lists that fit the interval list's memory.
 bool simulate_fits(const NetView& v, const UpdConst& c, int interval,
                    SimShared* sh, uint32_t* ctas) {
   // (a reset at or above the threshold fires at every step, refractory or not)
@@ -3075,12 +3079,17 @@ bool simulate_fits(const NetView& v, const UpdConst& c, int interval,
 cudaError_t launch_simulate(const NetView& v, const UpdConst& c,
                             const SimShared& sh, uint32_t ctas, int n_iv,
                             int steps, int last_steps, cudaStream_t s) {
+#define SNN_SIMULATE(L)                                                              \
+  (sh.polls == kSimPolls                                                             \
+       ? launch_simulate_t<L, false>(v, c, sh, ctas, n_iv, steps, last_steps, s)     \
+       : launch_simulate_t<L, true>(v, c, sh, ctas, n_iv, steps, last_steps, s))
   switch (v.lay) {
-    case kLayHom: return launch_simulate_t<kLayHom>(v, c, sh, ctas, n_iv, steps, last_steps, s);
-    case kLayF32: return launch_simulate_t<kLayF32>(v, c, sh, ctas, n_iv, steps, last_steps, s);
-    case kLayI16: return launch_simulate_t<kLayI16>(v, c, sh, ctas, n_iv, steps, last_steps, s);
-    default: return launch_simulate_t<kLayJ16>(v, c, sh, ctas, n_iv, steps, last_steps, s);
+    case kLayHom: return SNN_SIMULATE(kLayHom);
+    case kLayF32: return SNN_SIMULATE(kLayF32);
+    case kLayI16: return SNN_SIMULATE(kLayI16);
+    default: return SNN_SIMULATE(kLayJ16);
   }
+#undef SNN_SIMULATE
 }
 
 cudaError_t launch_fill_i32(int32_t* p, int32_t value, uint64_t n,

@@ -61,7 +61,6 @@ int fail(int code, const char* fmt, ...) {
   } while (0)
 
 constexpr int kGraphIntervals = 8;
-constexpr int kSimIntervals = 256;  // intervals of one k_simulate launch at most
 constexpr size_t kTileSmemBudget = 200 * 1024;  // accumulator bytes per CTA
 
 // ---------------------------------------------------------------------------
@@ -1556,15 +1555,16 @@ int snn_simulate(snn_net* net, int64_t n_steps) {
     }
     uint32_t ctas = 0;
     NetView v = net->view();
-    if (full + (rem ? 1 : 0) < 2 || !simulate_fits(v, net->uc, D, &sh, &ctas))
+    if (full + (rem ? 1 : 0) < 2 || net->cycle_max == 0 ||
+        !simulate_fits(v, net->uc, D, &sh, &ctas))
       return simulate_async(net, n_steps, true);
     if (net->sim_unscaled) v.max_abs_w = 0.f;
-    // launches of at most kSimIntervals intervals, so that other streams'
-    // work is not held off for long
+    // launches of a bounded number of intervals, so that other streams' work is
+    // not held off for long
     int64_t left = full + (rem ? 1 : 0);
     bool first = true;
     while (left > 0) {
-      const int m = (int)std::min<int64_t>(left, kSimIntervals);
+      const int m = (int)std::min<int64_t>(left, net->cycle_max);
       left -= m;
       const cudaError_t e =
           net->sim_refused
@@ -2091,6 +2091,14 @@ int snn_probe_exp2(const float* x, uint64_t n, float* approx, float* lib,
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaSetDevice(prev);
   CK(e);
+  return SNN_OK;
+}
+
+int snn_set_cycle(snn_net* net, int max_intervals) {
+  REQ(net, SNN_E_ARG, "null net");
+  REQ(max_intervals >= 0 && max_intervals <= kCycleMax, SNN_E_ARG,
+      "max_intervals %d outside [0, %d]", max_intervals, kCycleMax);
+  net->cycle_max = max_intervals;
   return SNN_OK;
 }
 

@@ -378,6 +378,8 @@ struct BatchNet {
 // snn_finalize, then every launch after itself), and of list regions (an entry:
 // source | step in its interval << 24).
 constexpr size_t kSimFlagBytes = 2 * 256 * 8 + 16;
+// Intervals of one launch at most (snn_set_cycle).
+constexpr int kCycleMax = 256;
 // Default of SimShared::polls (about a microsecond each).
 constexpr uint32_t kSimPolls = 1u << 24;
 struct SimShared {

@@ -74,6 +74,7 @@ struct snn_net {
   SpikeEntry* list = nullptr;
   uint64_t list_cap = 0;
   unsigned long long* sim_flags = nullptr;  // see SimShared
+  int cycle_max = kCycleMax;                // snn_set_cycle
   uint32_t sim_polls = kSimPolls;           // snn_debug_cycle
   bool sim_unscaled = false, sim_refused = false;
   SpikeEntry* ext_list = nullptr;

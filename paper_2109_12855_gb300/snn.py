@@ -49,7 +49,7 @@ EXPORTS = [
     "snn_debug_fail_allocations", "snn_exchange_capacity",
     "snn_set_exchange", "snn_deliver_exchanged", "snn_get_stream",
     "snn_checked", "snn_debug_check_failures", "snn_debug_poke_record",
-    "snn_probe_reductions", "snn_probe_exp2", "snn_debug_cycle",
+    "snn_probe_reductions", "snn_probe_exp2", "snn_debug_cycle", "snn_set_cycle",
 ]
 SNN_REQ_QUEUED, SNN_REQ_BUILDING, SNN_REQ_RUNNING, SNN_REQ_DONE = 0, 1, 2, 3
 SNN_REQ_FAILED = -1
@@ -223,6 +223,7 @@ def lib():
             "snn_probe_reductions": ([C.c_void_p, C.c_uint64, C.c_uint64,
                                       C.c_int, C.c_void_p,
                                       C.POINTER(C.c_float)], C.c_int),
+            "snn_set_cycle": ([_P, C.c_int], C.c_int),
             "snn_debug_cycle": ([_P, C.c_int, C.c_int64], C.c_int),
             "snn_probe_exp2": ([C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p,
                                 C.c_void_p], C.c_int),
@@ -344,6 +345,12 @@ def snn_deliver_noalloc(net, src, t_emit, want_events: bool = True):
 
 def snn_simulate(net, n_steps: int):
     _check(lib().snn_simulate(net, n_steps))
+
+
+def snn_set_cycle(net, max_intervals: int):
+    """Intervals that one launch of snn_simulate's cycle runs at most (0: the
+    separate kernels)."""
+    _check(lib().snn_set_cycle(net, max_intervals))
 
 
 def snn_read_spikes(net, src, t):

@@ -99,6 +99,24 @@ def test_refused_launch_runs_the_separate_kernels(steps):
             assert x.tobytes() == y.tobytes()
 
 
+@pytest.mark.parametrize("most,launches", [(0, 2 * 41), (1, 41), (7, 6), (256, 1)])
+def test_intervals_of_a_launch(most, launches):
+    from paper_2109_12855_gb300 import snn
+    with _net() as a, _net() as b:
+        snn.snn_set_cycle(a.h, most)
+        before = a.stats().kernel_launches
+        for net in (a, b):
+            snn.snn_simulate(net.h, 405)
+        assert a.stats().kernel_launches - before == launches
+        for x, y in zip(_state(a), _state(b)):
+            assert x.tobytes() == y.tobytes()
+        assert a.stats().t_now == b.stats().t_now == 405
+        for bad in (-1, 257):
+            with pytest.raises(snn.SnnError) as e:
+                snn.snn_set_cycle(a.h, bad)
+            assert e.value.code == snn.SNN_E_ARG
+
+
 def test_options_are_checked():
     from paper_2109_12855_gb300 import snn
     with _net(500, 50) as net:

@@ -542,10 +542,10 @@ int snn_load_state(snn_net* net, const void* host_buf, uint64_t size);
 int snn_set_time(snn_net* net, int64_t t);
 /* Profiling on: every update and deliver launch is bracketed by CUDA events
  * on the net's stream; times accumulate into snn_stats.ms_update /
- * ms_deliver.  snn_simulate keeps its CUDA graphs of whole intervals, with
- * the events captured as graph nodes, so the kernels are timed in the launch
- * context of the production path (the host waits after each graph to read
- * the times); other calls record the events around plain launches. */
+ * ms_deliver.  snn_simulate then runs the update and delivery kernels in CUDA
+ * graphs of whole intervals (not the one-launch cycle), with the events captured
+ * as graph nodes (the host waits after each graph to read the times); other calls
+ * record the events around plain launches. */
 int snn_set_profiling(snn_net* net, int on);
 /* Counters (synchronises). */
 int snn_get_stats(snn_net* net, snn_stats* out);
@@ -735,7 +735,7 @@ int snn_server_set_option(snn_server* sv, int32_t option, double value);
 /* Queue a request; *id identifies it.  Thread-safe.  SNN_E_ARG for invalid
  * parameters or a footprint above the whole budget.  A request with
  * params.tile_width == 0 gets delivery tiles in proportion to its synapses
- * (about one per 4.2e6, at most one per SM), since all served nets share
+ * (about one per 5.2e5, at most 120; persistent: per 4.2e6), since all served nets share
  * each delivery launch. */
 int snn_server_submit(snn_server* sv, const snn_request* req, uint64_t* id);
 /* Admit built nets, advance every lane by one step (its autotuned number

@@ -532,8 +532,9 @@ int build_store(snn_net* net, uint32_t* d_deg, Scatter scatter,
     balance_plastic_tiles(net->n, net->p.n_exc, &net->tile_w, &net->lo_bits,
                           &net->n_tiles, &net->pl_tiles, &net->tile_grp);
   CK(dalloc(&net->tile_off, (uint64_t)n * (net->n_tiles + 1) * sizeof(uint32_t), net->stream));
-  // layout of the store: split by field for the tiled delivery (its cells fit
-  // 16 bits whenever the tile fits, but for windows of one step and the like)
+  // layout of the store: split by field for the tiled delivery (its cells fit 16
+  // bits whenever the tile fits: 200 KB hold at most 51,200 one-word cells, and the
+  // delay range has at most as many steps as the window; the test is a guard)
   net->d_base = d_lo;
   net->n_pad = padded;
   net->lay = kLayRecords;

@@ -96,9 +96,9 @@ __global__ void k_fill_i32(int32_t* p, int32_t value, uint64_t n) {
 // 4-step blocks that the drive is drawn in: a block's ring-buffer loads, draws
 // and table look-ups are independent and issued together, then its steps run in
 // order.  What bounds it: issue, where several waves of blocks hide the
-// latencies (562,500 neurons: 1,517 warp instructions for 10 steps, 63 % of the
-// issue slots; groups of eight steps, with the words of two or three blocks
-// selected by alignment, took 1,756), else the latency of a thread's chain.
+// latencies (562,500 neurons, 10 steps: 1,240 warp instructions a warp without
+// spikes, 1,440 with an interval's spikes, 66 % of the issue slots), else the latency of a
+// thread's chain.
 // Spikes are kept as a per-thread bit mask of step indices and compacted once
 // per warp for up to 32 steps: a warp scan of the per-thread counts, then one
 // set of global atomics per warp with spikes reserves its list entries and
@@ -588,16 +588,18 @@ k_deliver(NetView v, unsigned long long* pair_p, unsigned int* done_p,
 // start + min delay).  Rows are sorted by target tile, so the synapses of
 // spike j for tile tau are one contiguous run, located by the row's tile
 // index.  (A) the CTA describes a batch of runs in shared memory; (B) its 32
-// warps take 32 / 2^lg runs at a time, 2^lg lanes a run; a lane reads aligned 16-byte vectors of its run (the store's split
-// layouts, snn_internal.cuh: 8 cells, 4 {cell, weight} words, or 4 weights
-// with their 4 cells), the next runs' vectors being loaded before the current
-// ones are added, and masks the elements outside the run.
+// warps take 32 / 2^lg runs at a time, 2^lg lanes a run; a lane reads aligned
+// 16-byte vectors of its run (the store's split layouts, snn_internal.cuh: 8
+// cells, 4 {cell, weight} words, or 4 weights with their 4 cells), the next runs'
+// vectors being loaded before the current ones are added, and masks the elements
+// outside the run.
 //
-// What bounds it: with 12- or 8-byte records one event cost 1.35 (FP32) or
-// about 1.2 (BF16) warp instructions and the launch was half issue, half
-// load latency (39.6 us FP32 and 31.6 us BF16 at 1.27e9 synapses, 1,350
-// spikes; 118 us at 6.3e9).  The split layouts move 2, 4 or 6 bytes an event,
-// and a 16-byte vector costs one load for 8 or 4 events.
+// What bounds it: instructions and load latency.  On 12- or 8-byte records an
+// event cost 1.35 (FP32) or about 1.2 (BF16) warp instructions; the split layouts
+// move 2, 4 or 6 bytes an event, a 16-byte vector costs one load for 8 or 4 events,
+// and an event costs 0.54 warp instructions and 2.2 bytes of DRAM with equal
+// weights (1,314 spikes, 74 cells a run, 20.4 us cold at 37 % of the issue slots)
+// and 0.76 and 4.2 as integers (2,400 spikes, 37 words, 24.6 us at 40 %).
 //
 // Accumulation is exact fixed point: a weight w becomes x = w 2^(q-s),
 // split into hi = rint(x) and lo = rint((x - hi) 2^s) in [-2^(s-1), 2^(s-1)]
@@ -668,8 +670,8 @@ __device__ __forceinline__ void red_shared_u32(uint32_t addr, uint32_t x) {
   asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
 }
 // The same where K < n (and, CLIP, K >= lo), else into the lane's own spare
-// word `none`: a select, as a conditional reduction compiles to a branch (three
-// branch instructions per reduction, 1.25 against 0.8 instructions per event).
+// word `none`: a select (with the reduction under a condition an event took 1.25
+// warp instructions in place of 0.8).
 template <int K, bool CLIP>
 __device__ __forceinline__ void red_shared_u32_at(uint32_t addr, uint32_t x,
                                                   int n, int lo, uint32_t none) {

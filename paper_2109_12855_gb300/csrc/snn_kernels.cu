@@ -2139,6 +2139,14 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
   int t = (int)*reinterpret_cast<volatile long long*>(&v.ctl->t_now);
   unsigned long long logged = *reinterpret_cast<volatile unsigned long long*>(&v.ctl->log_count);
   unsigned long long my_events = 0, my_spikes = 0;
+  // (simulate_fits has shown on the host that the scales, and the counts of uniform
+  // weights, exist for every list; they do if they do for the largest one's bound,
+  // and this says so if the device finds otherwise)
+  if (r == 0 && tid == kTileThreads - 1) {
+    const FixScale f = fix_scale(v, 0xFFFFFFFFull, true);
+    if (!(f.fixed && (LAY != kLayHom || f.packed)))
+      atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_SCALES);
+  }
   // (a net whose cycle once gave up stays as it is until its errors are cleared:
   // its CTAs had stopped at different steps; a CTA that set out beside one that
   // finds this finds `stop` set)
@@ -2183,13 +2191,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
       }
     };
     // (1) the list's events for this tile into the accumulator
-    // (simulate_fits has shown on the host that the scales exist for every
-    // list, and the counts of uniform weights: this says so if they do not)
-    if (iv > 0 && tid == kTileThreads - 1) {
-      s_fx = fix_scale(v, n_sp, true);
-      if (n_sp && !(s_fx.fixed && (LAY != kLayHom || s_fx.packed)))
-        atomicOr(&v.ctl->error_flags, (unsigned)SNN_ERRF_SCALES);
-    }
+    if (iv > 0 && tid == kTileThreads - 1) s_fx = fix_scale(v, n_sp, true);
     uint32_t j0 = 0;
     do {
       const uint32_t nb = min(desc_cap, n_sp - j0);

@@ -310,7 +310,7 @@ struct NetView {
   uint64_t n_pad;           // records the store has room for
 #endif
   int d_base;
-  int lg;                   // log2 of the lanes that share a run
+  int lg, lg_cycle;         // log2 of the lanes that share a run; in k_simulate
   float mean_row;           // synapses per source
   uint32_t hom_split;
   float hom_w[2];

@@ -2252,7 +2252,7 @@ k_simulate(const __grid_constant__ NetView v, const __grid_constant__ UpdConst c
           s_desc[k] = sd;
         }
       }
-      uint32_t lg = (uint32_t)v.lg;
+      uint32_t lg = (uint32_t)v.lg_cycle;
       while (lg < 5u && (nb << (lg + 1u)) <= (uint32_t)kTileThreads) ++lg;
       __syncthreads();
       if (nb)

@@ -120,6 +120,9 @@ struct snn_net {
   // FP32 9 33.9, 38.0, 20 50.1, 40.4, 37 73.1, 48.8.  Words between 5.5 and 16 are a
   // compromise: 13 on 20,003 neurons take 19.2 us on 2 lanes and 21.2 on 4, but the
   // shorter lists of their one-launch cycle 1,428 and 1,378 us for 100 intervals.
+  // In that cycle (a few hundred spikes, rows already in L2) 8 lanes pay earlier,
+  // us an interval on 4 and 8: words 20 12.4, 12.8, 37 17.0, 15.8; cells (BF16) 30
+  // 16.2, 16.9, 40 16.5, 16.2, 50 17.0, 16.2, 74 28.6, 27.8, (FP32) 60 16.2, 16.3.
   void set_layout(NetView* v) const {
     v->lay = lay;
     v->d_base = d_base;
@@ -133,7 +136,7 @@ struct snn_net {
 #if SNN_CHECK
     v->n_pad = n_pad;
 #endif
-    v->lg = 0;
+    v->lg = v->lg_cycle = 0;
     v->mean_row = n_src ? (float)((double)n_syn / n_src) : 0.f;
     if (lay == kLayRecords) return;
     if (fmt == SNN_W_FP32_12B) {
@@ -146,16 +149,19 @@ struct snn_net {
     }
     const double run =
         n_src && n_tiles ? (double)n_syn / ((double)n_src * n_tiles) : 0.0;
+    v->lg = run_lanes(run, 0);
+    v->lg_cycle = run_lanes(run, 1);
+  }
+  int run_lanes(double run, int cycle) const {
     const int k = lay == kLayHom ? 0 : lay == kLayF32 ? 2 : 1;
     static const double first[3] = {9.5, 3.5, 3.0}, far_apart[3] = {4000, 1750, 1350};
-    static const double more[3][3] = {{92, 310, 500}, {47, 110, 235}, {0, 90, 320}};
+    static const double eight[2][2] = {{92, 47}, {45, 26}};
+    static const double more[3][2] = {{310, 500}, {110, 235}, {90, 320}};
     const double spread = run * sqrt((double)n_src);
-    if (run < first[k]) return;
-    v->lg = 1;
-    if (spread < far_apart[k]) return;
-    v->lg = 2;
-    if (k == 2 ? spread < 3000.0 : run < more[k][0]) return;
-    v->lg = run < more[k][1] ? 3 : run < more[k][2] ? 4 : 5;
+    if (run < first[k]) return 0;
+    if (spread < far_apart[k]) return 1;
+    if (k == 2 ? spread < 3000.0 : run < eight[cycle][k]) return 2;
+    return run < more[k][0] ? 3 : run < more[k][1] ? 4 : 5;
   }
 
   NetView view() const {

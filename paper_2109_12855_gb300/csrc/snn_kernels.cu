@@ -1978,7 +1978,7 @@ k_deliver_tiled_batch(const BatchNet* __restrict__ nets,
 // of the accumulation (about 11 of 30 us an interval at 112,500 neurons), then
 // latencies in series.  Per interval, two kernels in a graph on whole records,
 // on split stores, and here: 1,250 neurons FP32 13.9, 13.6, 8.5 us;
-// 20,003 BF16 19.7, 18.2, 13.6; 112,500 FP32 48.0, 34.0, 30.2.  Nets of more
+// 20,003 BF16 19.7, 18.2, 13.9; 112,500 FP32 48.0, 34.0, 30.2.  Nets of more
 // tiles than SMs keep the two kernels (562,500 neurons: 143 us against 178
 // with two tiles a CTA here).
 // ---------------------------------------------------------------------------
